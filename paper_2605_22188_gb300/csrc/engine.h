@@ -48,6 +48,9 @@ void gemm_link_f64(cudaStream_t s, int m, int n, int p, const double* V, const d
 void gemm_link_f32(cudaStream_t s, int m, int n, int p, const float* V, const float* X,
                    const float* y, int kind, float* out, const GemmScratch* scr);
 
+// w = G v / ||v|| for the p x p FP64 Gram matrix; *norm = ||v||.
+void gram_power_step(cudaStream_t s, int p, const double* G, const double* v, double* w, double* norm);
+
 // ---- tensor-core products (tcgen05, TMA); see gemm_tc.cu
 struct TcMap {
     alignas(64) unsigned char bytes[128];   // a CUtensorMap

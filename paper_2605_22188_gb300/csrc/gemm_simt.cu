@@ -14,6 +14,8 @@
 // fixed order s = 0..splits-1 (so the result does not depend on arrival
 // order), applies the epilogue and sets the counter back to 0.  No CTA waits
 // for another.
+#include <algorithm>
+
 #include "common.cuh"
 #include "engine.h"
 
@@ -204,6 +206,119 @@ __global__ __launch_bounds__((BM / TM) * (BN / TN)) void k_gemm_nt(int R, int C,
 
 constexpr int kSMs = 152;
 
+// The FP64 product for outputs that would leave most of a 64 x 64 tile empty
+// (the few nodes of a search's first batches, few features): a CTA computes
+// RT rows x 32 columns, a column per lane, its eight warps taking eight of
+// every 64 of K each, their partial sums added in warp order at the end.
+// What bounds it: GB300 retires about two FP64 FMAs per SM and cycle, so one
+// warp instruction holds the pipe for 16 cycles and the shared-memory loads
+// hide behind it whatever the tile; time is the FP64 work of the busiest SM,
+// padding included.  A 64 x 64 tile multiplies 262k FMAs per 64 of K for
+// output of any size: 207 us per launch of X^T R at n = 200, p = 30, m <= 8,
+// 8 us here (both between events of their own; S = X V 39 us before, 7 us here).
+template <int RT, typename Epi>
+__global__ __launch_bounds__(256) void k_gemm_f64_small(int R, int C, int K, const double* __restrict__ A, int lda,
+                                                        const double* __restrict__ B, int ldb, Epi epi, int kchunk,
+                                                        double* __restrict__ part, int* __restrict__ counters) {
+    constexpr int KT = 64, NW = 8;
+    __shared__ double Bs[32][KT + 1];                  // odd row stride: a column per lane without bank conflicts
+    __shared__ double As[RT][KT];
+    __shared__ double red[NW][RT][32];
+    __shared__ int s_last;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int r0 = blockIdx.y * RT, c0 = blockIdx.x * 32;
+    const int kbeg = blockIdx.z * kchunk, kend = min(K, kbeg + kchunk);
+    constexpr int BL = 32 * KT / 256;
+    double rb[BL], ra = 0.0, rc = 0.0;
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int l = 0; l < BL; ++l) {
+            const int v = tid + l * 256, col = v / KT, k = k0 + v % KT;
+            rb[l] = (c0 + col < C && k < kend) ? __ldg(B + (size_t)(c0 + col) * ldb + k) : 0.0;
+        }
+        // RT x 64 entries of A: at most two per thread
+        const int row = tid / KT, k = k0 + tid % KT;
+        ra = (row < RT && r0 + row < R && k < kend) ? __ldg(A + (size_t)(r0 + row) * lda + k) : 0.0;
+        if (RT > 4) rc = (r0 + row + 4 < R && k < kend) ? __ldg(A + (size_t)(r0 + row + 4) * lda + k) : 0.0;
+    };
+    double acc[RT];
+#pragma unroll
+    for (int r = 0; r < RT; ++r) acc[r] = 0.0;
+    if (kbeg < kend) load(kbeg);
+    for (int k0 = kbeg; k0 < kend; k0 += KT) {
+#pragma unroll
+        for (int l = 0; l < BL; ++l) {
+            const int v = tid + l * 256;
+            Bs[v / KT][v % KT] = rb[l];
+        }
+        if (tid / KT < RT) As[tid / KT][tid % KT] = ra;
+        if (RT > 4) As[(tid / KT + 4) % RT][tid % KT] = rc;
+        __syncthreads();
+        if (k0 + KT < kend) load(k0 + KT);
+        if (k0 + warp * (KT / NW) < kend) {            // the tail of K: no FP64 work on the zeros past it
+#pragma unroll
+            for (int kk = 0; kk < KT / NW; ++kk) {
+                const double b = Bs[lane][warp * (KT / NW) + kk];
+#pragma unroll
+                for (int r = 0; r < RT; ++r) acc[r] = fma(As[r][warp * (KT / NW) + kk], b, acc[r]);
+            }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int r = 0; r < RT; ++r) red[warp][r][lane] = acc[r];
+    __syncthreads();
+    const int row = tid / 32;                          // RT <= 8 rows, a warp each
+    const bool mine = row < RT && r0 + row < R && c0 + lane < C;
+    double v = 0.0;
+    if (mine) {
+#pragma unroll
+        for (int w = 0; w < NW; ++w) v += red[w][row][lane];
+    }
+    if (gridDim.z > 1) {
+        // split-K as in k_gemm_nt: the last CTA of a tile sums the partials in order
+        const int tile = blockIdx.y * gridDim.x + blockIdx.x, ntile = gridDim.x * gridDim.y;
+        if (row < RT) part[((size_t)blockIdx.z * ntile + tile) * (RT * 32) + row * 32 + lane] = v;
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) s_last = (atomicAdd(&counters[tile], 1) == (int)gridDim.z - 1);
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();
+        v = 0.0;
+        if (mine)
+            for (int s = 0; s < (int)gridDim.z; ++s)
+                v += __ldcg(part + ((size_t)s * ntile + tile) * (RT * 32) + row * 32 + lane);
+        if (tid == 0) counters[tile] = 0;
+    }
+    if (mine) epi(r0 + row, c0 + lane, v);
+}
+
+// One step of the power iteration on the symmetric Gram matrix: w = G v / ||v||,
+// a warp per row; every CTA forms ||v|| itself (the same sum in the same order),
+// CTA 0 records it.  A step reads G once (p x p from L2 where it fits).
+__global__ __launch_bounds__(256) void k_power_step(int p, const double* __restrict__ G, const double* __restrict__ v,
+                                                    double* __restrict__ w, double* __restrict__ norm) {
+    __shared__ double red[8];
+    double q[1] = {0.0};
+    for (int j = threadIdx.x; j < p; j += 256) q[0] = fma(v[j], v[j], q[0]);
+    block_sum<256, 1, double>(q, red);
+    const double nv = sqrt(q[0]);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *norm = nv;
+    const int lane = threadIdx.x & 31, r = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (r >= p) return;
+    const double* g = G + (size_t)r * p;
+    double s0 = 0.0, s1 = 0.0;
+    int j = lane;
+    for (; j + 32 < p; j += 64) {
+        s0 = fma(__ldg(g + j), v[j], s0);
+        s1 = fma(__ldg(g + j + 32), v[j + 32], s1);
+    }
+    if (j < p) s0 = fma(__ldg(g + j), v[j], s0);
+    const double s = warp_sum(s0 + s1);
+    if (lane == 0) w[r] = nv > 0.0 ? s / nv : 0.0;
+}
+
 template <typename T>
 struct Tile;
 template <> struct Tile<float> { static constexpr int BM = 128, BN = 128, BK = 8, TM = 8, TN = 8; };
@@ -253,12 +368,67 @@ GemmPlan plan_for(int R, int C, int K) {
     return g;
 }
 
+// FP64: the small-tile kernel where the FP64 work of its busiest SM (tiles of
+// RT x 32, padding included) is below that of the 64 x 64 tiles; true if it ran.
+// The work is counted in FMAs per SM, since the FP64 pipe is what both wait for:
+// at p = 30, m = 2 the small tiles do 1/80 of the 64 x 64 tile's, at m = 64,
+// n = 2000 the same, and the larger tile reads less.
+template <typename Epi>
+bool launch_small(cudaStream_t s, int R, int C, int K, const double* A, int lda, const double* B, int ldb, Epi epi,
+                  const GemmScratch* scr, const GemmPlan& big) {
+    if (K <= 0) return false;
+    const long bw = ((long)big.tiles * big.splits + kSMs - 1) / kSMs;
+    const double big_work = (double)bw * Tile<double>::BM * Tile<double>::BN * big.kchunk;
+    const int ct = (C + 31) / 32;
+    int best_rt = 0, best_split = 1, best_kc = K;
+    double best = big_work;
+    for (int rt = 1; rt <= 8; rt *= 2) {
+        const long tiles = (long)ct * ((R + rt - 1) / rt);
+        const bool can = scr != nullptr && scr->part != nullptr && scr->counters != nullptr && tiles <= scr->n_counters;
+        for (int sp = 1; sp <= 16; ++sp) {
+            int kc = (K + sp - 1) / sp;
+            kc = (kc + 63) / 64 * 64;
+            const int used = (K + kc - 1) / kc;
+            if (used != sp) continue;
+            if (sp > 1 && (!can || tiles * sp > 2 * kSMs ||
+                           (size_t)tiles * sp * rt * 32 * sizeof(double) > scr->part_bytes))
+                break;
+            const long waves = (tiles * sp + kSMs - 1) / kSMs;
+            // a split costs a pass over the partials: about 64 of K per split
+            const double work = (double)waves * rt * 32 * ((double)std::min(kc, K) + (sp > 1 ? 16.0 * sp : 0.0));
+            if (work < 0.9 * best) {
+                best = work;
+                best_rt = rt;
+                best_split = sp;
+                best_kc = kc;
+            }
+        }
+    }
+    if (best_rt == 0) return false;
+    const long rows = (R + best_rt - 1) / best_rt;
+    if (rows > 65535) return false;
+    const dim3 grid(ct, (unsigned)rows, best_split);
+    double* part = best_split > 1 ? static_cast<double*>(scr->part) : nullptr;
+    int* cnt = best_split > 1 ? scr->counters : nullptr;
+#define KGLM_SMALL(RT_) \
+    k_gemm_f64_small<RT_, Epi><<<grid, 256, 0, s>>>(R, C, K, A, lda, B, ldb, epi, best_kc, part, cnt)
+    if (best_rt == 1) KGLM_SMALL(1);
+    else if (best_rt == 2) KGLM_SMALL(2);
+    else if (best_rt == 4) KGLM_SMALL(4);
+    else KGLM_SMALL(8);
+#undef KGLM_SMALL
+    return true;
+}
+
 template <typename T, typename Epi>
 void launch(cudaStream_t s, int R, int C, int K, const T* A, int lda, const T* B, int ldb, Epi epi,
             const GemmScratch* scr) {
     if (R <= 0 || C <= 0) return;
     using TL = Tile<T>;
     GemmPlan g = plan_for<T>(R, C, K);
+    if constexpr (sizeof(T) == 8) {
+        if (launch_small(s, R, C, K, A, lda, B, ldb, epi, scr, g)) return;
+    }
     T* part = nullptr;
     int* cnt = nullptr;
     if (g.splits > 1) {
@@ -375,6 +545,10 @@ void gemm_link_f64(cudaStream_t s, int m, int n, int p, const double* V, const d
 void gemm_link_f32(cudaStream_t s, int m, int n, int p, const float* V, const float* X, const float* y,
                    int kind, float* out, const GemmScratch* scr) {
     launch<float>(s, m, n, p, V, p, X, p, EpiLink<float>{out, n, y, kind}, scr);
+}
+
+void gram_power_step(cudaStream_t s, int p, const double* G, const double* v, double* w, double* norm) {
+    k_power_step<<<(p + 7) / 8, 256, 0, s>>>(p, G, v, w, norm);
 }
 
 }  // namespace kglm
