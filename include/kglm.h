@@ -60,7 +60,8 @@ typedef enum { KGLM_LSQ = 0, KGLM_LOGISTIC = 1 } kglm_loss;
  * plus explicit rounding margins (the other modes; looser by ~1e-7
  * relative). */
 typedef enum {
-    KGLM_FP64 = 0,  /* FP64 products and prox */
+    KGLM_FP64 = 0,  /* FP64 products and prox (large products as exact BF16 digit products on the
+                       tensor cores, with an error below that of an FP64 sum) */
     KGLM_FP32 = 1,  /* FP32 products (CUDA cores) and prox */
     KGLM_BF16 = 2,  /* BF16 tensor-core products, FP32 accumulate and prox */
     KGLM_TF32 = 3,  /* TF32 tensor-core products, FP32 accumulate and prox */
@@ -330,7 +331,10 @@ kglm_status kglm_configure(kglm_ctx* ctx, const kglm_tune* cfg);
  * the memory per node; admission control needs the whole footprint before
  * any allocation).  Host-only arithmetic, no CUDA call.  Not included: one
  * max_batch x p FP64 buffer that kglm_push_nodes with warm_B, and one that
- * kglm_xtz, allocate on first use.  KGLM_EINVAL for a desc kglm_create would
+ * kglm_xtz, allocate on first use; and in the FP64 mode the digits of the
+ * tensor-core products (about 32 n p + 56 max_batch n + 112 max_batch p bytes),
+ * allocated at the first batch large enough for them and left out, with the
+ * products on the CUDA cores, where hbm_budget or the device does not hold them.  KGLM_EINVAL for a desc kglm_create would
  * reject on its sizes, ranges or enums. */
 kglm_status kglm_estimate_bytes(const kglm_desc* desc, int64_t* bytes);
 

@@ -130,6 +130,22 @@ struct kglm_ctx {
     TcMap mAz{}, mBx{};
     int bnx = 0;
     int gsplit_max = 4;
+    // FP64 mode: the products as BF16 digit products (split64.cu), set up at the
+    // first batch large enough for them
+    struct Split64 {
+        bool tried = false, on = false;
+        int pk = 0, nk = 0;                          // padded row lengths (multiples of 64)
+        __nv_bfloat16 *DX = nullptr, *DXt = nullptr; // digits of X (columns scaled by 1 / sxt) and X^T
+        __nv_bfloat16 *DV = nullptr, *DR = nullptr;  // of V (or beta) times sxt, and R (or zeta), reversed
+        double *sx = nullptr, *sxt = nullptr, *tv = nullptr, *tr = nullptr;   // their row scales
+        int* I = nullptr;                            // jobs' integers
+        size_t cap = 0;
+        int* flag = nullptr;
+        TcMap mV{}, mX{}, mR{}, mXt{};
+        int bnS = 0, bnG = 0;
+        SplitPlan pS{}, pG{};                        // plans of batch sizes mS and mG
+        int mS = -1, mG = -1;
+    } sp;
     // host mirror of the evaluated batch
     std::vector<int> h_kbar, h_pf, h_jstar;
     std::vector<double> h_lb, h_ub;
@@ -369,6 +385,118 @@ double gram_lambda_max(kglm_ctx* c) {
     return lam;
 }
 
+// ---- FP64 products on the tensor cores (split64.cu)
+// Where they pay: from about 2.5e7 FMAs per product on.  Microseconds per FISTA
+// iteration, digits against CUDA cores: m n p = 1.3e7 (n 2000, p 200) 112 / 103,
+// 2.0e7 (n 5000, p 1000) 244 / 167, 2.6e7 (n 2000, p 200) 113 / 147, 2.6e7 (n 1000,
+// p 100) 98 / 158, 8e7 (n 5000, p 1000) 207 / 386, 1.3e9 289 / 4552.
+bool split_pays(const kglm_ctx* c, int m) { return c->f64 && (double)m * c->n * c->p >= 2.5e7; }
+
+// Digits of X and the batch's buffers, once per context (16 bytes per entry of X
+// and X^T each, 16 per entry of V and R, the integers of the products).  Not
+// part of the footprint: where the budget or the device does not hold them, or the
+// data's rows span so many binades that fixed-point rows would lose to FP64, the
+// CUDA-core products stay.
+void split_setup(kglm_ctx* c) {
+    kglm_ctx::Split64& q = c->sp;
+    if (q.tried) return;
+    q.tried = true;
+    const size_t n = c->n, p = c->p, mc = c->mcap;
+    // 65536: levels of at most 2032 K slices a job make at most 24 jobs (the cap below always holds them)
+    if (!c->f64 || n > 65536 || !isfinite(c->eta) || c->M > 1e100) return;
+    if (split_prepare() != 0 || tc_prepare() != 0) return;
+    q.pk = (int)((p + 63) / 64 * 64);
+    q.nk = (int)((n + 63) / 64 * 64);
+    q.bnS = tc_tile_cols((int)n);
+    q.bnG = tc_tile_cols((int)p);
+    // room for whole levels of S, and for levels in pieces of G (or of a small batch)
+    q.cap = std::max(std::max(10 * mc * n, 24 * mc * p), (size_t)(8 << 20));
+    const size_t need = 16 * ((n + mc) * q.pk + (p + mc) * q.nk) + 8 * (n + p + 2 * mc) + 4 * q.cap + 64;
+    if (c->d.hbm_budget > 0 && (int64_t)(c->bytes + need) > c->d.hbm_budget) return;
+    const size_t had = c->allocs.size(), bytes0 = c->bytes;
+    int* tcerr0 = c->d_tcerr;
+    auto drop = [&] {
+        for (size_t i = had; i < c->allocs.size(); ++i) cudaFreeAsync(c->allocs[i], c->st);
+        c->allocs.resize(had);
+        c->bytes = bytes0;
+        c->d_tcerr = tcerr0;
+        q.on = false;
+    };
+    try {
+        q.DX = dalloc_t<__nv_bfloat16>(c, 8 * n * q.pk);
+        q.DXt = dalloc_t<__nv_bfloat16>(c, 8 * p * q.nk);
+        q.DV = dalloc_t<__nv_bfloat16>(c, 8 * mc * q.pk);
+        q.DR = dalloc_t<__nv_bfloat16>(c, 8 * mc * q.nk);
+        q.sx = dalloc_t<double>(c, n);
+        q.sxt = dalloc_t<double>(c, p);
+        q.tv = dalloc_t<double>(c, mc);
+        q.tr = dalloc_t<double>(c, mc);
+        q.I = dalloc_t<int>(c, q.cap);
+        q.flag = dalloc_t<int>(c, 1);
+        if (!c->d_tcerr) {
+            c->d_tcerr = dalloc_t<int>(c, 1);
+            CK(cudaMemsetAsync(c->d_tcerr, 0, sizeof(int), c->st));
+        }
+    } catch (const Fail&) {
+        drop();
+        return;
+    }
+    if (tc_make_map(&q.mX, q.DX, 1, (int)n, 8 * q.pk, 8 * q.pk, q.bnS) ||
+        tc_make_map(&q.mXt, q.DXt, 1, (int)p, 8 * q.nk, 8 * q.nk, q.bnG) ||
+        tc_make_map(&q.mV, q.DV, 1, (int)mc, 8 * q.pk, 8 * q.pk, 128) ||
+        tc_make_map(&q.mR, q.DR, 1, (int)mc, 8 * q.nk, 8 * q.nk, 128)) {
+        drop();
+        return;
+    }
+    CK(cudaMemsetAsync(q.flag, 0, sizeof(int), c->st));
+    split_digits(c->st, c->Xt64, (int)p, (int)n, n, q.nk, nullptr, 0, 0, q.DXt, q.sxt, q.flag);
+    split_digits(c->st, c->X64, (int)n, (int)p, p, q.pk, q.sxt, 1, 0, q.DX, q.sx, q.flag);
+    split_digits(c->st, c->y64, 1, (int)n, n, q.nk, nullptr, 0, 0, nullptr, nullptr, q.flag);
+    check_launch();
+    int bad = 0;
+    CK(cudaMemcpyAsync(&bad, q.flag, sizeof(int), cudaMemcpyDeviceToHost, c->st));
+    sync(c);
+    if (bad) {
+        drop();
+        return;
+    }
+    q.on = true;
+}
+
+bool split_on(const kglm_ctx* c, int m) { return c->sp.on && split_pays(c, m); }
+
+// The integers of S = X V (or X beta) from V's digits, or of X^T R (X^T zeta) from
+// R's; the plan of a batch size is kept for the next product of that size.
+const SplitPlan& split_product(kglm_ctx* c, int m, bool grad) {
+    kglm_ctx::Split64& q = c->sp;
+    SplitPlan& pl = grad ? q.pG : q.pS;
+    int& have = grad ? q.mG : q.mS;
+    const int N = grad ? c->p : c->n, K = grad ? c->n : c->p, bn = grad ? q.bnG : q.bnS;
+    if (have != m) {
+        if (!split_plan(m, N, K, bn, true, q.cap, &pl)) throw Fail{KGLM_ECUDA, "no plan for an FP64 digit product"};
+        have = m;
+    }
+    if (tc_gemm_jobs(c->st, grad ? q.mR : q.mV, grad ? q.mXt : q.mX, m, N, bn, pl.jobs, pl.njobs,
+                     reinterpret_cast<float*>(q.I), (size_t)m * N, N, c->d_tcerr, 1, kSplitChunk) != 0)
+        throw Fail{KGLM_ECUDA, "FP64 digit product setup failed"};
+    check_launch();
+    return pl;
+}
+
+// S = X V for m rows of V (m x p FP64) into out, and X^T R for R (m x n) into out.
+void split_xv(kglm_ctx* c, int m, const double* V, double* out) {
+    kglm_ctx::Split64& q = c->sp;
+    split_digits(c->st, V, m, c->p, c->p, q.pk, q.sxt, 0, 1, q.DV, q.tv, nullptr);
+    const SplitPlan& pl = split_product(c, m, false);
+    split_combine(c->st, m, c->n, q.I, (size_t)m * c->n, pl, q.tv, q.sx, out);
+}
+void split_xtr(kglm_ctx* c, int m, const double* R, double* out) {
+    kglm_ctx::Split64& q = c->sp;
+    split_digits(c->st, R, m, c->n, c->n, q.nk, nullptr, 0, 1, q.DR, q.tr, nullptr);
+    const SplitPlan& pl = split_product(c, m, true);
+    split_combine(c->st, m, c->p, q.I, (size_t)m * c->p, pl, q.tr, q.sxt, out);
+}
+
 // X^T zeta of the batch's dual points (c->zeta, m x n): FP64 GEMM into c->Q,
 // or in the reduced-precision modes the exact-splitting product on the
 // tensor cores, whose partials and bound are recorded in the certificate's
@@ -419,8 +547,10 @@ void certify(kglm_ctx* c) {
     }
     const double ws = c->f64 ? 8.0 : 4.0;
     {
-        Scope sc(c, PH_CERT_XB, 1, 2.0 * n * c->sum_pa);
-        if (c->f64) {
+        Scope sc(c, PH_CERT_XB, split_on(c, m) ? 3 : 1, 2.0 * n * c->sum_pa);
+        if (split_on(c, m)) {
+            split_xv(c, m, (const double*)c->B, (double*)c->R);
+        } else if (c->f64) {
             gemm_nt_f64(c->st, m, n, p, (const double*)c->B, p, c->X64, p, (double*)c->R, n, &c->gs64);
         } else if (c->tc) {
             // tensor-core modes: X beta as the TF32 hi + lo split (hi hi + hi lo + lo hi,
@@ -446,8 +576,9 @@ void certify(kglm_ctx* c) {
         check_launch();
     }
     {
-        Scope sc(c, PH_CERT_Q, c->cexact ? 2 : 1, 2.0 * n * c->sum_pa);
-        xtzeta(c, m, a);
+        Scope sc(c, PH_CERT_Q, split_on(c, m) ? 3 : c->cexact ? 2 : 1, 2.0 * n * c->sum_pa);
+        if (split_on(c, m)) split_xtr(c, m, c->zeta, c->Q);
+        else xtzeta(c, m, a);
         check_launch();
     }
     {
@@ -551,13 +682,26 @@ void iterate(kglm_ctx* c) {
         iterate_rows(c, c->st, 0, m, false);
         return;
     }
-    {
-        Scope sc(c, PH_GEMM_LINK, 1, flops);
-        if (c->f64) gemm_link_f64(c->st, m, n, p, (const double*)c->V, c->X64, c->y64, c->kind, (double*)c->R, &c->gs64);
-        else gemm_link_f32(c->st, m, n, p, (const float*)c->V, c->X32, c->y32, c->kind, (float*)c->R, &c->gs32);
+    if (split_on(c, m)) {
+        kglm_ctx::Split64& q = c->sp;
+        {
+            Scope sc(c, PH_GEMM_LINK, 3, flops);
+            split_digits(c->st, (const double*)c->V, m, p, p, q.pk, q.sxt, 0, 1, q.DV, q.tv, nullptr);
+            const SplitPlan& pl = split_product(c, m, false);
+            split_link(c->st, m, n, q.nk, q.I, (size_t)m * n, pl, q.tv, q.sx, c->y64, c->kind, (double*)c->R, q.DR, q.tr);
+            check_launch();
+        }
+        Scope sc(c, PH_GEMM_GRAD, 2, flops);
+        const SplitPlan& pl = split_product(c, m, true);
+        split_combine(c->st, m, p, q.I, (size_t)m * p, pl, q.tr, q.sxt, (double*)c->G);
         check_launch();
-    }
-    {
+    } else {
+        {
+            Scope sc(c, PH_GEMM_LINK, 1, flops);
+            if (c->f64) gemm_link_f64(c->st, m, n, p, (const double*)c->V, c->X64, c->y64, c->kind, (double*)c->R, &c->gs64);
+            else gemm_link_f32(c->st, m, n, p, (const float*)c->V, c->X32, c->y32, c->kind, (float*)c->R, &c->gs32);
+            check_launch();
+        }
         Scope sc(c, PH_GEMM_GRAD, 1, flops);
         if (c->f64) gemm_nt_f64(c->st, m, p, n, (const double*)c->R, n, c->Xt64, n, (double*)c->G, p, &c->gs64);
         else gemm_nt_f32(c->st, m, p, n, (const float*)c->R, n, c->Xt32, n, (float*)c->G, p, &c->gs32);
@@ -675,6 +819,7 @@ void run_iters(kglm_ctx* c, int count) {
 // final certificate, bound fold and re-optimization.
 void evaluate_begin(kglm_ctx* c, int iters) {
     const int m = c->m;
+    if (split_pays(c, m)) split_setup(c);              // before any capture of this batch's iterations
     const unsigned gb = (unsigned)((m + 255) / 256);
     Scope sc(c, PH_SMALL, 2, 0.0);
     k_fill<<<gb, 256, 0, c->st>>>(m, c->lb_best, -INFINITY);
@@ -722,7 +867,7 @@ void evaluate_end(kglm_ctx* c) {
         if (reopt_launch(c->st, r) != 0) throw Fail{KGLM_ECUDA, "re-optimization kernel: shared memory for k refused"};
         check_launch();
     }
-    if (c->tc || c->cexact) {
+    if (c->tc || c->cexact || c->sp.on) {
         // read back with the results (one synchronisation), checked by finish_tc_check
         CK(cudaMemcpyAsync(c->pinned<int>(c->off_tcerr()), c->d_tcerr, sizeof(int), cudaMemcpyDeviceToHost, c->st));
         c->tc_check_pending = true;
@@ -2191,6 +2336,26 @@ kglm_status kglm_xtr(kglm_ctx* ctx, int32_t m, const void* R, void* G) {
             sync(ctx);
             check_tc_error(ctx);
             return;
+        }
+        if (split_pays(ctx, m)) split_setup(ctx);
+        if (split_on(ctx, m)) {
+            // the caller's R is any data: its rows' spread is read back before the
+            // fixed-point product is taken
+            kglm_ctx::Split64& q = ctx->sp;
+            int bad = 0;
+            CK(cudaMemsetAsync(q.flag, 0, sizeof(int), ctx->st));
+            split_digits(ctx->st, (const double*)R, m, ctx->n, ctx->n, q.nk, nullptr, 0, 1, q.DR, q.tr, q.flag);
+            check_launch();
+            CK(cudaMemcpyAsync(&bad, q.flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
+            sync(ctx);
+            if (!bad) {
+                const SplitPlan& pl = split_product(ctx, m, true);
+                split_combine(ctx->st, m, ctx->p, q.I, (size_t)m * ctx->p, pl, q.tr, q.sxt, (double*)G);
+                check_launch();
+                sync(ctx);
+                check_tc_error(ctx);
+                return;
+            }
         }
         if (ctx->f64)
             gemm_nt_f64(ctx->st, m, ctx->p, ctx->n, (const double*)R, ctx->n, ctx->Xt64, ctx->n, (double*)G, ctx->p,

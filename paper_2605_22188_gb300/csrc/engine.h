@@ -111,8 +111,11 @@ struct TcJob {
 // out slice jobs[z].slice (at pout + slice * pstride, row stride pld) =
 // A[:, K range of job z] . B[:, K range of job z]^T for every job, in one launch.
 // pair_on: as CTA pairs (256-row tiles) where the B map has a half box.
+// chunk > 0 (even): the products are of integers and pout holds 32-bit integers; the
+// sums over every chunk of that many K slices are exact in FP32 (at most 2^24) and
+// are added up as integers (a job's whole sum stays below 2^31).
 int tc_gemm_jobs(cudaStream_t s, const TcMap& A, const TcMap& B, int M, int N, int bn, const TcJob* jobs,
-                 int njobs, float* pout, size_t pstride, int pld, int* err, int pair_on);
+                 int njobs, float* pout, size_t pstride, int pld, int* err, int pair_on, int chunk = 0, int pdl = 0);
 // Exact-splitting certificate product (cert_exact.cu): jobs of the level
 // products, their weights 2^(-beta l) and the bound n E per unit sigma tau.
 struct ExactPlan {
@@ -135,6 +138,28 @@ void exact_digits(cudaStream_t s, const double* V, int rows, int n, size_t ldv, 
 // jobs' weights (host array of nq values).
 void exact_combine(cudaStream_t s, int m, int p, const float* Qs, int nq, size_t stride, const double* w,
                    const double* sigma, const double* tau, double ebound, double* Q, double* E);
+// FP64 products as BF16 digit products (split64.cu): the jobs of the levels 2 .. 9
+// (digit pairs a + c = level), largest first.
+constexpr int kSplitChunk = 16;    // K slices of 64 whose digit products sum to at most 2^24
+struct SplitPlan {
+    int kbs, njobs;                // K slices per digit
+    TcJob jobs[kTcMaxJobs];
+    int level[kTcMaxJobs];
+};
+// Jobs for an M x N output over K with column tiles of bn, such that jobs M N <= max_ints; false if none fit.
+bool split_plan(int M, int N, int K, int bn, bool pair, size_t max_ints, SplitPlan* out);
+// Eight digits of every row of V (entries times cs[j], or over it with inv) and the row scales.
+void split_digits(cudaStream_t s, const double* V, int rows, int n, size_t ldv, int npad, const double* cs, int inv,
+                  int reversed, __nv_bfloat16* D, double* scale, int* flag);
+// out (rows x cols) from the jobs' integers (slice t at I + t stride).
+void split_combine(cudaStream_t s, int rows, int cols, const int* I, size_t stride, const SplitPlan& pl,
+                   const double* sr, const double* sc, double* out);
+// R = dl(S, y) from the jobs' integers of S = X V, as reversed digits with row scales tr
+// (Rg: FP64 rows to work in where n is too large for shared memory).
+void split_link(cudaStream_t s, int m, int n, int npad, const int* I, size_t stride, const SplitPlan& pl,
+                const double* tv, const double* sx, const double* y, int kind, double* Rg, __nv_bfloat16* D,
+                double* tr);
+int split_prepare();
 int tc_gemm(cudaStream_t s, const TcMap& A, const TcMap& B, const TcMap* B2, const TcGemm& g,
             const GemmScratch* scr);
 // One problem of a grouped BF16 product (single operands): out[r][c] = sum_k A[arow0 + r][k] B[c][k],

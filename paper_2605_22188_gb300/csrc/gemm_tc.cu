@@ -124,6 +124,7 @@ struct TcArgs {
     float* part;              // split-K partial tiles (nz > 1, epi != PARTIAL)
     int* counters;
     int* err;
+    int chunk;                // integer products: K slices per accumulator, whose sums are then exact
     int njobs;                // > 0: K range z is job z (its own K offsets in A and B, and slice)
     TcJob jobs[kTcMaxJobs];
 };
@@ -431,9 +432,17 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 
 // The kernel body over a source of units and problems: SrcOne (the launch's
 // operand maps and TcArgs) or SrcGroup (a table of problems).
-template <int KIND, int NB, int NA, int CL, class S>
+// INT: products of integer digits whose sums do not fit 24 bits over a unit's
+// whole K range.  A unit's K range is taken in chunks of a.chunk K slices, each
+// an accumulator of its own (exact in FP32); the epilogue adds the chunks up as
+// 32-bit integers in registers (16 columns x 8 chunks of columns per thread) and
+// stores the integers.  Two accumulators alternate over the chunks as they do
+// over the units otherwise, so that a chunk's drain (128 conversions per thread,
+// about 2000 cycles) hides behind the next chunk's products (8192 cycles).
+template <int KIND, int NB, int NA, int CL, bool INT, class S>
 __device__ __forceinline__ void tc_body(const TcArgs& a, const S& src) {
     static_assert(CL == 1 || (KIND == 0 && NA == 1 && NB == 1), "CTA pairs: BF16 single operands");
+    static_assert(!INT || (KIND == 0 && NA == 1 && NB == 1), "integer products: BF16 single operands");
     const int STAGES = a.stages;
     // B rows per CTA: a pair's CTAs hold half of the tile's columns each
     const int bnl = CL == 2 ? a.bn / 2 : a.bn;
@@ -468,7 +477,17 @@ __device__ __forceinline__ void tc_body(const TcArgs& a, const S& src) {
     const bool leader = crank == 0;
     const int units = src.units(CL);
     const int ucta = blockIdx.x / CL, ustride = gridDim.x / CL;
-    auto unit = [&](int u) { return src.unit(u, CL, crank); };
+    // INT: the units come largest first; every second pass over the CTAs runs
+    // backwards, so that the CTA with the largest unit gets the smallest next
+    auto unit = [&](int u) {
+        if constexpr (INT) {
+            const int pass = u / ustride, at = u - pass * ustride;
+            const int rev = (pass + 1) * ustride <= units ? ustride - 1 - at : units - 1 - pass * ustride - at;
+            return src.unit(pass * ustride + ((pass & 1) ? rev : at), CL, crank);
+        } else {
+            return src.unit(u, CL, crank);
+        }
+    };
 
     pdl_trigger();
     if (threadIdx.x == 32) {
@@ -555,15 +574,19 @@ __device__ __forceinline__ void tc_body(const TcArgs& a, const S& src) {
             // MMA issuer
             int g = 0, li = 0;
             bool ok = true;
-            for (int u = ucta; u < units && ok; u += ustride, ++li) {
-                const Unit w = unit(u);
+            for (int u = ucta; u < units && ok; u += ustride) {
+              const Unit w = unit(u);
+              const int nst = (w.nloc + KS - 1) / KS;
+              // stages per accumulator: a chunk's, or the unit's
+              const int cst = INT ? a.chunk / KS : nst;
+              for (int i0 = 0; ok; i0 += cst, ++li) {
                 const int b = li & 1;
                 const uint32_t use = (uint32_t)(li >> 1) & 1u;
-                if (!mbar_wait(smem_u32(&tempty[b]), use ^ 1u, a.err)) break;
+                if (!mbar_wait(smem_u32(&tempty[b]), use ^ 1u, a.err)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t acc = tmem + (uint32_t)(b * MAXBN);
-                const int nst = (w.nloc + KS - 1) / KS;
-                for (int i = 0; i < nst; ++i, ++g) {
+                const int i1 = INT ? min(nst, i0 + cst) : nst;
+                for (int i = i0; i < i1; ++i, ++g) {
                     const int s = g % STAGES;
                     const uint32_t ph = (uint32_t)(g / STAGES) & 1u;
                     if (!mbar_wait(smem_u32(&full[s]), ph, a.err)) { ok = false; break; }
@@ -573,7 +596,7 @@ __device__ __forceinline__ void tc_body(const TcArgs& a, const S& src) {
                         const uint32_t aa = smem_u32(smem + (size_t)s * SSTR + (size_t)t * SLSTR), bb = aa + offB;
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk) {   // four MMAs of 32 bytes of K each (per B part)
-                            const uint32_t accf = (i > 0 || t > 0 || kk > 0) ? 1u : 0u;
+                            const uint32_t accf = (i > i0 || t > 0 || kk > 0) ? 1u : 0u;
                             if constexpr (CL == 2) {
                                 umma_pair(acc, smem_desc(aa + kk * 32), smem_desc(bb + kk * 32), a.idesc, accf);
                             } else {
@@ -592,6 +615,8 @@ __device__ __forceinline__ void tc_body(const TcArgs& a, const S& src) {
                 // the accumulator is complete (or abandoned)
                 if constexpr (CL == 2) umma_commit_pair_mc(smem_u32(&tfull[b]));
                 else umma_commit(smem_u32(&tfull[b]));
+                if (!INT || i1 >= nst) { ++li; break; }
+              }
             }
             // every product issued so far has finished once this commit arrives
             if constexpr (CL == 2) umma_commit_pair(smem_u32(drain));
@@ -607,6 +632,79 @@ __device__ __forceinline__ void tc_body(const TcArgs& a, const S& src) {
         const int h = (warp - 2) >> 2;
         float* tb = sT + (warp - 2) * 32 * TPAD;
         int li = 0;
+        if constexpr (INT) {
+            for (int u = ucta; u < units; u += ustride) {
+                const Unit w = unit(u);
+                const auto& pq = src.q(w.pi);
+                const int nst = (w.nloc + KS - 1) / KS, cst = a.chunk / KS;
+                int sum[MAXBN / 32][16];
+#pragma unroll
+                for (int q = 0; q < MAXBN / 32; ++q)
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) sum[q][j] = 0;
+                bool ok = true;
+                for (int i0 = 0; i0 < nst; i0 += cst, ++li) {
+                    const int b = li & 1;
+                    const uint32_t use = (uint32_t)(li >> 1) & 1u;
+                    ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&tfull[b]), use, a.err));
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t tl = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(b * MAXBN);
+#pragma unroll
+                    for (int q = 0; q < MAXBN / 32; ++q) {
+                        const int c = 16 * h + 32 * q;
+                        if (c < a.bn) {
+                            float v[16];
+                            tmem_ld16(tl + (uint32_t)c, v);
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) sum[q][j] += __float2int_rn(v[j]);
+                        }
+                    }
+                    tc_fence_before();
+                    if constexpr (CL == 2) {
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive_cluster(mapa_rank(smem_u32(&tempty[b]), 0));
+                    } else {
+                        mbar_arrive(smem_u32(&tempty[b]));
+                    }
+                }
+                if (!ok) break;
+                const int rbase = w.mtile * BM + quad * 32, n0 = w.ntile * a.bn;
+                int* o = reinterpret_cast<int*>(pq.pout + (size_t)w.slice * pq.pstride);
+                const size_t ld = (size_t)pq.pld;
+                const int qq = lane & 3, r0 = lane >> 2;
+                int* ti = reinterpret_cast<int*>(tb);
+#pragma unroll
+                for (int q = 0; q < MAXBN / 32; ++q) {
+                    const int c = 16 * h + 32 * q;
+                    if (c < a.bn) {
+#pragma unroll
+                        for (int j = 0; j < 16; j += 4)
+                            *reinterpret_cast<int4*>(ti + lane * TPAD + j) =
+                                make_int4(sum[q][j], sum[q][j + 1], sum[q][j + 2], sum[q][j + 3]);
+                        __syncwarp();
+                        const int c0 = n0 + c + 4 * qq;
+                        const bool vec = (ld % 4) == 0 && (reinterpret_cast<uintptr_t>(o) % 16) == 0 && c0 + 4 <= pq.N;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const int r = r0 + 8 * i, row = rbase + r;
+                            if (row >= pq.M) continue;
+                            const int4 x = *reinterpret_cast<const int4*>(ti + r * TPAD + 4 * qq);
+                            int* dst = o + (size_t)row * ld + c0;
+                            if (vec) {
+                                *reinterpret_cast<int4*>(dst) = x;
+                            } else {
+                                const int xs[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                                for (int t = 0; t < 4; ++t)
+                                    if (c0 + t < pq.N) dst[t] = xs[t];
+                            }
+                        }
+                        __syncwarp();
+                    }
+                }
+            }
+        } else
         for (int u = ucta; u < units; u += ustride, ++li) {
             const Unit w = unit(u);
             const auto& pq = src.q(w.pi);
@@ -865,20 +963,20 @@ struct SrcGroup {
     }
 };
 
-template <int KIND, int NB, int NA, int CL>
+template <int KIND, int NB, int NA, int CL, bool INT = false>
 __global__ void __launch_bounds__(NT, 1) k_tc_gemm(const __grid_constant__ CUtensorMap tmA,
                                                    const __grid_constant__ CUtensorMap tmB,
                                                    const __grid_constant__ CUtensorMap tmB2,
                                                    const __grid_constant__ CUtensorMap tmA2,
                                                    const __grid_constant__ TcArgs a) {
     const SrcOne src{&tmA, &tmB, &tmB2, &tmA2, a};
-    tc_body<KIND, NB, NA, CL>(a, src);
+    tc_body<KIND, NB, NA, CL, INT>(a, src);
 }
 
 // Several problems (the instances of the serving loop) in one persistent launch.
 __global__ void __launch_bounds__(NT, 1) k_tc_gemm_group(const __grid_constant__ TcGroupArgs g) {
     const SrcGroup src{g};
-    tc_body<0, 1, 1, 1>(g.a, src);
+    tc_body<0, 1, 1, 1, false>(g.a, src);
 }
 
 // A wait that nothing ends: one thread waits on an mbarrier no thread arrives
@@ -913,10 +1011,10 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
     return fn;
 }
 
-template <int KIND, int NB, int NA, int CL = 1>
+template <int KIND, int NB, int NA, int CL = 1, bool INT = false>
 int set_smem_attr() {
     // once per process (thread-safe static initialisation: serving contexts launch from several threads)
-    static const int rc = cudaFuncSetAttribute(k_tc_gemm<KIND, NB, NA, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    static const int rc = cudaFuncSetAttribute(k_tc_gemm<KIND, NB, NA, CL, INT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)kSmemMax) == cudaSuccess ? 0 : -1;
     return rc;
 }
@@ -952,7 +1050,8 @@ void wait_probe(cudaStream_t s, uint32_t rounds, int* err) { k_wait_probe<<<1, 3
 
 int tc_prepare() {
     return set_smem_attr<0, 1, 1>() | set_smem_attr<0, 2, 1>() | set_smem_attr<1, 1, 1>() | set_smem_attr<1, 2, 1>() |
-           set_smem_attr<1, 2, 2>() | set_smem_attr<0, 1, 1, 2>() | (pair_clusters() > 0 ? 0 : 0);
+           set_smem_attr<1, 2, 2>() | set_smem_attr<0, 1, 1, 2>() | set_smem_attr<0, 1, 1, 1, true>() |
+           set_smem_attr<0, 1, 1, 2, true>() | (pair_clusters() > 0 ? 0 : 0);
 }
 
 int tc_make_map(TcMap* out, const void* base, int is_bf16, int rows, int cols, int ld, int box_rows) {
@@ -1156,10 +1255,11 @@ int tc_gemm_group(cudaStream_t s, const TcGroupItem* items, int np, int bn, int 
 }
 
 int tc_gemm_jobs(cudaStream_t s, const TcMap& A, const TcMap& B, int M, int N, int bn, const TcJob* jobs,
-                 int njobs, float* pout, size_t pstride, int pld, int* err, int pair_on) {
+                 int njobs, float* pout, size_t pstride, int pld, int* err, int pair_on, int chunk, int pdl) {
     if (M <= 0 || N <= 0 || njobs <= 0) return 0;
     if (bn < 16 || bn > MAXBN || bn % 16 != 0 || njobs > kTcMaxJobs) return -4;
-    if (set_smem_attr<0, 1, 1>()) return -5;
+    if (chunk < 0 || chunk % 2 != 0) return -4;
+    if (chunk ? (set_smem_attr<0, 1, 1, 1, true>() | set_smem_attr<0, 1, 1, 2, true>()) : set_smem_attr<0, 1, 1>()) return -5;
     TcArgs a{};
     a.M = M; a.N = N; a.bn = bn;
     a.mt = (M + BM - 1) / BM;
@@ -1173,34 +1273,40 @@ int tc_gemm_jobs(cudaStream_t s, const TcMap& A, const TcMap& B, int M, int N, i
     a.pout = pout; a.pstride = pstride; a.pld = pld;
     a.err = err;
     a.njobs = njobs;
+    a.chunk = chunk;
     for (int j = 0; j < njobs; ++j) a.jobs[j] = jobs[j];
     const CUtensorMap& ma = *reinterpret_cast<const CUtensorMap*>(A.bytes);
     const CUtensorMap& mb = *reinterpret_cast<const CUtensorMap*>(B.bytes);
     // CTA pairs as in tc_gemm: 256-row tiles, half of B per CTA, two K slices per stage
     const bool pair = pair_on && a.mt >= 2 && B.has_half && pair_clusters() > 0;
+    cudaLaunchConfig_t cfg{};
+    cfg.blockDim = dim3(NT);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    cfg.attrs = attr;
+    if (pdl) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
     if (!pair) {
-        const dim3 grid(grid_of(a.mt * a.nt * njobs));
-        k_tc_gemm<0, 1, 1, 1><<<grid, NT, smem_for(1, 1, bn), s>>>(ma, mb, mb, ma, a);
-        return 0;
+        cfg.gridDim = dim3(grid_of(a.mt * a.nt * njobs));
+        cfg.dynamicSmemBytes = smem_for(1, 1, bn);
+        return (chunk ? cudaLaunchKernelEx(&cfg, k_tc_gemm<0, 1, 1, 1, true>, ma, mb, mb, ma, a)
+                      : cudaLaunchKernelEx(&cfg, k_tc_gemm<0, 1, 1, 1>, ma, mb, mb, ma, a)) == cudaSuccess ? 0 : -7;
     }
     a.ks = 2;
     const size_t sl = stage_stride(1, 1, bn / 2);
     a.stages = (int)std::min<size_t>((kSmemMax - kSmemFixed) / (2 * sl), kMaxStages);
     a.idesc = (a.idesc & ~(0x1Fu << 24)) | ((uint32_t)((2 * BM) >> 4) << 24);
-    cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(2 * std::max(1, std::min(((a.mt + 1) / 2) * a.nt * njobs, pair_clusters())));
-    cfg.blockDim = dim3(NT);
     cfg.dynamicSmemBytes = kSmemFixed + (size_t)a.stages * 2 * sl;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs].val.clusterDim.x = 2;
+    attr[cfg.numAttrs].val.clusterDim.y = 1;
+    attr[cfg.numAttrs++].val.clusterDim.z = 1;
     const CUtensorMap& mbh = *reinterpret_cast<const CUtensorMap*>(B.half);
-    return cudaLaunchKernelEx(&cfg, k_tc_gemm<0, 1, 1, 2>, ma, mbh, mbh, ma, a) == cudaSuccess ? 0 : -7;
+    return (chunk ? cudaLaunchKernelEx(&cfg, k_tc_gemm<0, 1, 1, 2, true>, ma, mbh, mbh, ma, a)
+                  : cudaLaunchKernelEx(&cfg, k_tc_gemm<0, 1, 1, 2>, ma, mbh, mbh, ma, a)) == cudaSuccess ? 0 : -7;
 }
 
 }  // namespace kglm

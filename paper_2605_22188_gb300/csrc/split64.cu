@@ -1,0 +1,328 @@
+// FP64 products on the BF16 tensor cores, by the error-free splitting of
+// cert_exact.cu (Ozaki et al. 2012) carried to the end of an FP64 significand.
+//
+// GB300 retires two FP64 FMAs per SM and cycle (about 1.1 TFLOP/s over the
+// chip), 1/1700 of its BF16 tensor rate, so an FP64 product is the whole cost
+// of an FP64 iteration, and 36 exact BF16 products in its place are some 40
+// times cheaper.  X^T R of 256 nodes at n = 5000, p = 1000: 2.17 ms on the FP64
+// pipe, 69 us as digits; a whole FISTA iteration 4.55 -> 0.29 ms.
+//
+// Row r of an operand (K-contiguous) is scaled by 2^e > 2 max_k |v_rk| and
+// rounded to the 64-bit integer V = rint(v 2^(64 - e)), |V| < 2^63, which is cut
+// exactly into eight signed bytes from the bottom, v = 2^e sum_a d_a 2^(-8a),
+// |d_a| <= 128: exact in BF16.  The digit pairs (a, c) of one level l = a + c
+// share the weight 2^(-8l) and are concatenated along K (the second operand's
+// digits are stored in reverse order, so that level l is a prefix of one row
+// against a window of the other).  Sums of digit products over 16 slices of 64 are
+// integers of at most 16 * 64 * 2^14 = 2^24, exact in the tensor core's FP32
+// accumulator; the product's epilogue adds such chunks up in 32-bit integers
+// (gemm_tc.cu, INT), and the kernels here add the jobs of a level and the levels
+// 2 .. 9 in 64-bit integers:
+//   H = sum_{l <= 5} 2^(8 (5 - l)) I_l,  L = sum_{l >= 6} 2^(8 (9 - l)) I_l,
+//   C = 2^(ea + eb) (2^-40 H + 2^-72 L),
+// |H| < 2^38 K (1 + 2^-6), |L| < 2^41 K (1 + 2^-6): no overflow for K < 2^21.
+// Left out are the levels 10 .. 16, at most 7 K 2^14 2^-80 (1 + 2^-7) of the
+// scales' product, and the rounding of the operands, 2^-65 of each scale; the last
+// FMA rounds once.  So the error is a few K 2^-64 of (2 max |a_r|)(2 max |b_c|)
+// plus half an ulp of the result.  An FP64 FMA chain has K 2^-53 of
+// sum_k |a_rk b_ck| as its bound and rounds at every one of the K partial sums:
+// against exact sums (tests/test_gpu_fp64_split.py) its root-mean-square error is
+// 4.3e-16 to 8e-16 of the results' size over n = 640 .. 20011, p = 111 .. 2000,
+// this one's 5e-20 to 4e-17.
+// The two bounds part where the entries of a row span many binades; the engine
+// takes this path only for instances whose rows are not spread so (the flag of
+// k_split_digits), with the columns of X scaled to comparable size (powers of two
+// moved from X to the other operand, exactly).
+#include <algorithm>
+
+#include "common.cuh"
+#include "engine.h"
+
+namespace kglm {
+namespace {
+
+// The eight digits of z (a = 8 is the lowest byte), as BF16.
+struct Digits {
+    __nv_bfloat16 d[8];
+};
+__device__ __forceinline__ void cut(long long z, __nv_bfloat16 (&d)[8]) {
+#pragma unroll
+    for (int a = 7; a >= 1; --a) {
+        const int v = (int)(signed char)z;
+        z = (z - v) >> 8;
+        d[a] = __int2bfloat16_rn(v);
+    }
+    d[0] = __int2bfloat16_rn((int)z);
+}
+
+// v 2^(64 - e) rounded to an integer; f = 2^(64 - e) where that is a normal number.
+__device__ __forceinline__ long long fixed(double v, double f, int e) {
+    return __double2ll_rn(e > -900 ? v * f : ldexp(v, 64 - e));
+}
+
+// Digits of four consecutive entries i .. i + 3 of a row into its eight segments.
+__device__ __forceinline__ void store_digits(const long long (&z)[4], __nv_bfloat16* row, size_t npad, int i, int reversed) {
+    __nv_bfloat16 d[4][8];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) cut(z[t], d[t]);
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+        __nv_bfloat162 lo, hi;
+        lo.x = d[0][a]; lo.y = d[1][a];
+        hi.x = d[2][a]; hi.y = d[3][a];
+        uint2 w;
+        w.x = *reinterpret_cast<const uint32_t*>(&lo);
+        w.y = *reinterpret_cast<const uint32_t*>(&hi);
+        *reinterpret_cast<uint2*>(row + (size_t)(reversed ? 7 - a : a) * npad + i) = w;
+    }
+}
+
+// Scale of a row from its largest magnitude: e with 2^e > 2 max (0 for a zero row).
+__device__ __forceinline__ int row_exp(double mx) { return mx > 0.0 ? ilogb(mx) + 2 : 0; }
+
+// Rows of V (rows x n, stride ldv; entry j times cs[j], or over it with inv) into digit
+// rows of D (8 npad entries each, zero past n; NULL: none) and their scales 2^e (NaN
+// for a row with a non-finite entry, whose products are then NaN).  GS threads
+// per row.  flag: set for a row whose largest magnitude is above 2^10 times the mean
+// of its nonzero ones, whose scale is outside 2^(-+400), or with a non-finite entry.
+template <int GS>
+__global__ __launch_bounds__(256) void k_split_digits(const double* __restrict__ V, int rows, int n, size_t ldv,
+                                                      int npad, const double* __restrict__ cs, int inv, int reversed,
+                                                      __nv_bfloat16* __restrict__ D, double* __restrict__ scale,
+                                                      int* flag) {
+    __shared__ double red[2 * 8];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int g = threadIdx.x / GS, t = threadIdx.x % GS;
+    const int r = blockIdx.x * (256 / GS) + g;
+    if (GS == 32 && r >= rows) return;                       // whole warps; one CTA per row otherwise
+    const double* v = V + (size_t)r * ldv;
+    auto at = [&](int i) {
+        const double x = v[i];
+        return cs ? (inv ? x / cs[i] : x * cs[i]) : x;
+    };
+    double mx = 0.0, bad = 0.0;
+    for (int i = t; i < n; i += GS) {
+        const double x = fabs(at(i));
+        bad = isfinite(x) ? bad : 1.0;
+        mx = fmax(mx, x);
+    }
+    if (GS == 32) {
+        mx = warp_max(mx);
+        bad = warp_max(bad);
+    } else {
+        mx = block_max<256, double>(mx, red);
+        bad = block_max<256, double>(bad, red + 8);
+    }
+    const int e = row_exp(bad > 0.0 ? 0.0 : mx);
+    if (t == 0 && scale) scale[r] = bad > 0.0 ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(1.0, e);
+    if (flag) {
+        double q[2] = {0.0, 0.0};
+        for (int i = t; i < n; i += GS) {
+            const double x = fabs(at(i));
+            if (x > 0.0) { q[0] += x / mx; q[1] += 1.0; }
+        }
+        if (GS == 32) { q[0] = warp_sum(q[0]); q[1] = warp_sum(q[1]); }
+        else block_sum<256, 2, double>(q, red);
+        if (t == 0 && (bad > 0.0 || e < -400 || e > 400 || q[1] > 1024.0 * q[0])) atomicOr(flag, 1);
+    }
+    if (!D) return;
+    __nv_bfloat16* d = D + (size_t)r * 8 * npad;
+    const double f = e > -900 ? ldexp(1.0, 64 - e) : 0.0;
+    for (int i = 4 * t; i < npad; i += 4 * GS) {
+        long long z[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) z[q] = (i + q < n && !(bad > 0.0)) ? fixed(at(i + q), f, e) : 0ll;
+        store_digits(z, d, (size_t)npad, i, reversed);
+    }
+}
+
+struct Levels {
+    int n;
+    signed char hi[kTcMaxJobs];      // 1: the job's level is at most 5
+    signed char sh[kTcMaxJobs];      // its shift within its half
+};
+
+// One entry of the product from its jobs' integers (scale: 2^(ea + eb - 40)).
+__device__ __forceinline__ double combine(const int* __restrict__ I, size_t stride, size_t idx, const Levels& lv,
+                                          double scale) {
+    long long H = 0, L = 0;
+    for (int t0 = 0; t0 < lv.n; t0 += 8) {                   // eight jobs' loads in flight
+        int v[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) v[t] = t0 + t < lv.n ? __ldg(I + (size_t)(t0 + t) * stride + idx) : 0;
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            if (t0 + t < lv.n) {
+                const long long x = (long long)v[t] << lv.sh[t0 + t];
+                if (lv.hi[t0 + t]) H += x; else L += x;
+            }
+        }
+    }
+    return fma((double)L, 0x1p-32, (double)H) * scale;
+}
+
+// out[b][j] = sr[b] sc[j] (product of digits) for a rows x cols output.
+__global__ __launch_bounds__(256) void k_split_combine(int rows, int cols, const int* __restrict__ I, size_t stride,
+                                                       const __grid_constant__ Levels lv, const double* __restrict__ sr,
+                                                       const double* __restrict__ sc, double* __restrict__ out) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int b = blockIdx.y;
+    const double s = sr[b] * 0x1p-40;
+    const size_t base = (size_t)b * cols;
+    for (int j = blockIdx.x * 256 + threadIdx.x; j < cols; j += gridDim.x * 256)
+        out[base + j] = combine(I, stride, base + j, lv, s * sc[j]);
+}
+
+// S = X V of one node per CTA, its loss derivative R and R's digits: the row stays
+// in shared memory between the two (in Rg where it does not fit), so that neither S
+// nor R is written in FP64.  Bound by the FP64 pipe: five operations per entry to
+// put S together, the link's (two, or about forty for the logistic loss) and two
+// for the digits.
+constexpr int kLinkNT = 512;
+__global__ __launch_bounds__(kLinkNT) void k_split_link(int n, int npad, const int* __restrict__ I, size_t stride,
+                                                        const __grid_constant__ Levels lv, const double* __restrict__ tv,
+                                                        const double* __restrict__ sx, const double* __restrict__ y,
+                                                        int kind, double* Rg, __nv_bfloat16* __restrict__ D,
+                                                        double* __restrict__ tr) {
+    extern __shared__ __align__(16) double srow[];
+    __shared__ double red[2 * (kLinkNT / 32)];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int b = blockIdx.x, t = threadIdx.x;
+    const size_t base = (size_t)b * n;
+    double* row = Rg ? Rg + base : srow;
+    const double s = tv[b] * 0x1p-40;
+    double mx = 0.0, bad = 0.0;
+    for (int i = t; i < n; i += kLinkNT) {
+        const double r = dloss(combine(I, stride, base + i, lv, s * sx[i]), y[i], kind);
+        row[i] = r;
+        bad = isfinite(r) ? bad : 1.0;
+        mx = fmax(mx, fabs(r));
+    }
+    mx = block_max<kLinkNT, double>(mx, red);
+    bad = block_max<kLinkNT, double>(bad, red + kLinkNT / 32);   // its barriers also publish the row
+    const int e = row_exp(bad > 0.0 ? 0.0 : mx);
+    if (t == 0) tr[b] = bad > 0.0 ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(1.0, e);
+    __nv_bfloat16* d = D + (size_t)b * 8 * npad;
+    const double f = e > -900 ? ldexp(1.0, 64 - e) : 0.0;
+    for (int i = 4 * t; i < npad; i += 4 * kLinkNT) {
+        long long z[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) z[q] = (i + q < n && !(bad > 0.0)) ? fixed(row[i + q], f, e) : 0ll;
+        store_digits(z, d, (size_t)npad, i, 1);
+    }
+}
+
+Levels levels_of(const SplitPlan& pl) {
+    Levels lv{};
+    lv.n = pl.njobs;
+    for (int t = 0; t < pl.njobs; ++t) {
+        lv.hi[t] = pl.level[t] <= 5;
+        lv.sh[t] = (signed char)(8 * ((pl.level[t] <= 5 ? 5 : 9) - pl.level[t]));
+    }
+    return lv;
+}
+
+constexpr size_t kLinkSmem = 200 * 1024;
+
+}  // namespace
+
+bool split_plan(int M, int N, int K, int bn, bool pair, size_t max_ints, SplitPlan* out) {
+    const int kbs = (K + 63) / 64, chunk = kSplitChunk;
+    const int mt = (M + 127) / 128, nt = (N + bn - 1) / bn;
+    pair = pair && mt >= 2;
+    const long tiles = (long)(pair ? (mt + 1) / 2 : mt) * nt;
+    const int workers = pair ? 76 : 152;
+    const double total = 36.0 * kbs * (double)tiles;
+    // microseconds of one K slice of a tile (operands at ~68 bytes per cycle and SM, as
+    // the link product measures), of a unit's start and end, and of a slice's trip
+    // through memory
+    const double us_kb = (128.0 + (pair ? bn / 2 : bn)) * 128.0 / 68.0 / 1900.0;
+    const double us_unit = 2.0, us_slice = (double)M * N * 8.0 / 6.0e6;
+    double best = 1e300;
+    for (int w : {0, 1, 2, 3, 4, 6, 8}) {
+        // pieces of at most J slices (whole chunks; a job's sum stays below 2^31); w = 0: as few as possible
+        long J = w == 0 ? 2032 : (long)(total / ((double)workers * w)) + 1;
+        J = std::min<long>(2032, std::max<long>(2 * chunk, (J + chunk - 1) / chunk * chunk));
+        SplitPlan p{};
+        p.kbs = kbs;
+        bool fits = true;
+        for (int l = 9; l >= 2 && fits; --l) {
+            const int kb = (l - 1) * kbs, cnt = (int)((kb + J - 1) / J);
+            const int per = ((kb + cnt - 1) / cnt + chunk - 1) / chunk * chunk;
+            for (int u0 = 0; u0 < kb; u0 += per) {
+                if (p.njobs >= kTcMaxJobs) { fits = false; break; }
+                p.jobs[p.njobs] = {(9 - l) * kbs + u0, u0, std::min(per, kb - u0), 0};
+                p.level[p.njobs++] = l;
+            }
+        }
+        if (!fits || (size_t)p.njobs * M * N > max_ints) continue;
+        int at[kTcMaxJobs];
+        for (int t = 0; t < p.njobs; ++t) at[t] = t;
+        std::stable_sort(at, at + p.njobs, [&](int a, int b) { return p.jobs[a].nkb > p.jobs[b].nkb; });
+        SplitPlan q = p;
+        for (int t = 0; t < p.njobs; ++t) {
+            q.jobs[t] = p.jobs[at[t]];
+            q.jobs[t].slice = t;
+            q.level[t] = p.level[at[t]];
+        }
+        // the busiest worker: units dealt forwards and backwards in turn (gemm_tc.cu)
+        double worst;
+        const long units = tiles * q.njobs;
+        if (units > 64L * workers) {
+            worst = (total * us_kb + units * us_unit) / workers;
+        } else {
+            double load[152] = {};
+            for (long u = 0; u < units; ++u) {
+                const long pass = u / workers, a = u - pass * workers;
+                const long width = std::min<long>(workers, units - pass * workers);
+                load[(pass & 1) ? width - 1 - a : a] += q.jobs[u / tiles].nkb * us_kb + us_unit;
+            }
+            worst = *std::max_element(load, load + workers);
+        }
+        const double cost = worst + q.njobs * us_slice;
+        if (cost < best) {
+            best = cost;
+            *out = q;
+        }
+    }
+    return best < 1e300;
+}
+
+void split_digits(cudaStream_t s, const double* V, int rows, int n, size_t ldv, int npad, const double* cs, int inv,
+                  int reversed, __nv_bfloat16* D, double* scale, int* flag) {
+    if (rows <= 0) return;
+    if (n <= 512) k_split_digits<32><<<(rows + 7) / 8, 256, 0, s>>>(V, rows, n, ldv, npad, cs, inv, reversed, D, scale, flag);
+    else k_split_digits<256><<<rows, 256, 0, s>>>(V, rows, n, ldv, npad, cs, inv, reversed, D, scale, flag);
+}
+
+void split_combine(cudaStream_t s, int rows, int cols, const int* I, size_t stride, const SplitPlan& pl,
+                   const double* sr, const double* sc, double* out) {
+    // rows on the grid's y axis, in runs of at most 65535
+    for (int b0 = 0; b0 < rows; b0 += 65535) {
+        const int rr = std::min(65535, rows - b0);
+        const dim3 grid(std::max(1, std::min(8, (cols + 255) / 256)), rr);
+        k_split_combine<<<grid, 256, 0, s>>>(rr, cols, I + (size_t)b0 * cols, stride, levels_of(pl), sr + b0, sc,
+                                             out + (size_t)b0 * cols);
+    }
+}
+
+int split_prepare() {
+    static const int rc = cudaFuncSetAttribute(k_split_link, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)kLinkSmem) == cudaSuccess ? 0 : -1;
+    return rc;
+}
+
+void split_link(cudaStream_t s, int m, int n, int npad, const int* I, size_t stride, const SplitPlan& pl,
+                const double* tv, const double* sx, const double* y, int kind, double* Rg, __nv_bfloat16* D,
+                double* tr) {
+    if (m <= 0) return;
+    const size_t need = (size_t)n * sizeof(double);
+    const bool sm = need <= kLinkSmem;
+    k_split_link<<<m, kLinkNT, sm ? need : 0, s>>>(n, npad, I, stride, levels_of(pl), tv, sx, y, kind,
+                                                   sm ? nullptr : Rg, D, tr);
+}
+
+}  // namespace kglm
