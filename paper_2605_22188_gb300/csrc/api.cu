@@ -135,9 +135,9 @@ struct kglm_ctx {
     struct Split64 {
         bool tried = false, on = false;
         int pk = 0, nk = 0;                          // padded row lengths (multiples of 64)
-        __nv_bfloat16 *DX = nullptr, *DXt = nullptr; // digits of X (columns scaled by 1 / sxt) and X^T
-        __nv_bfloat16 *DV = nullptr, *DR = nullptr;  // of V (or beta) times sxt, and R (or zeta), reversed
-        double *sx = nullptr, *sxt = nullptr, *tv = nullptr, *tr = nullptr;   // their row scales
+        __nv_bfloat16 *DX = nullptr, *DXt = nullptr; // digits of X (columns scaled by 2^-sxt) and X^T
+        __nv_bfloat16 *DV = nullptr, *DR = nullptr;  // of V (or beta) times 2^sxt, and R (or zeta), reversed
+        int *sx = nullptr, *sxt = nullptr, *tv = nullptr, *tr = nullptr;      // their row scales' exponents
         int* I = nullptr;                            // jobs' integers
         size_t cap = 0;
         int* flag = nullptr;
@@ -386,10 +386,11 @@ double gram_lambda_max(kglm_ctx* c) {
 }
 
 // ---- FP64 products on the tensor cores (split64.cu)
-// Where they pay: from about 2.5e7 FMAs per product on.  Microseconds per FISTA
-// iteration, digits against CUDA cores: m n p = 1.3e7 (n 2000, p 200) 112 / 103,
-// 2.0e7 (n 5000, p 1000) 244 / 167, 2.6e7 (n 2000, p 200) 113 / 147, 2.6e7 (n 1000,
-// p 100) 98 / 158, 8e7 (n 5000, p 1000) 207 / 386, 1.3e9 289 / 4552.
+// Where they pay: from about 2e7 FMAs per product on.  Microseconds per FISTA
+// iteration, digits against CUDA cores: m n p = 2.0e7 (n 5000, p 1000) 165 / 165,
+// 2.6e7 (n 2000, p 200) 100 / 146, 2.6e7 (n 1000, p 100) 80 / 158, 3.2e7 (n 5000,
+// p 400) 152 / 187, 8e7 (n 5000, p 1000) 171 / 385, 1.3e9 255 / 4554; at 1.3e7
+// (n 2000, p 200) the CUDA cores take 104.
 bool split_pays(const kglm_ctx* c, int m) { return c->f64 && (double)m * c->n * c->p >= 2.5e7; }
 
 // Digits of X and the batch's buffers, once per context (16 bytes per entry of X
@@ -411,7 +412,7 @@ void split_setup(kglm_ctx* c) {
     q.bnG = tc_tile_cols((int)p);
     // room for whole levels of S, and for levels in pieces of G (or of a small batch)
     q.cap = std::max(std::max(10 * mc * n, 24 * mc * p), (size_t)(8 << 20));
-    const size_t need = 16 * ((n + mc) * q.pk + (p + mc) * q.nk) + 8 * (n + p + 2 * mc) + 4 * q.cap + 64;
+    const size_t need = 16 * ((n + mc) * q.pk + (p + mc) * q.nk) + 4 * (n + p + 2 * mc) + 4 * q.cap + 64;
     if (c->d.hbm_budget > 0 && (int64_t)(c->bytes + need) > c->d.hbm_budget) return;
     const size_t had = c->allocs.size(), bytes0 = c->bytes;
     int* tcerr0 = c->d_tcerr;
@@ -427,10 +428,10 @@ void split_setup(kglm_ctx* c) {
         q.DXt = dalloc_t<__nv_bfloat16>(c, 8 * p * q.nk);
         q.DV = dalloc_t<__nv_bfloat16>(c, 8 * mc * q.pk);
         q.DR = dalloc_t<__nv_bfloat16>(c, 8 * mc * q.nk);
-        q.sx = dalloc_t<double>(c, n);
-        q.sxt = dalloc_t<double>(c, p);
-        q.tv = dalloc_t<double>(c, mc);
-        q.tr = dalloc_t<double>(c, mc);
+        q.sx = dalloc_t<int>(c, n);
+        q.sxt = dalloc_t<int>(c, p);
+        q.tv = dalloc_t<int>(c, mc);
+        q.tr = dalloc_t<int>(c, mc);
         q.I = dalloc_t<int>(c, q.cap);
         q.flag = dalloc_t<int>(c, 1);
         if (!c->d_tcerr) {
@@ -688,7 +689,8 @@ void iterate(kglm_ctx* c) {
             Scope sc(c, PH_GEMM_LINK, 3, flops);
             split_digits(c->st, (const double*)c->V, m, p, p, q.pk, q.sxt, 0, 1, q.DV, q.tv, nullptr);
             const SplitPlan& pl = split_product(c, m, false);
-            split_link(c->st, m, n, q.nk, q.I, (size_t)m * n, pl, q.tv, q.sx, c->y64, c->kind, (double*)c->R, q.DR, q.tr);
+            if (split_link(c->st, m, n, q.nk, q.I, (size_t)m * n, pl, q.tv, q.sx, c->y64, c->kind, q.DR, q.tr) != 0)
+                throw Fail{KGLM_ECUDA, "FP64 link launch failed"};
             check_launch();
         }
         Scope sc(c, PH_GEMM_GRAD, 2, flops);

@@ -148,17 +148,15 @@ struct SplitPlan {
 };
 // Jobs for an M x N output over K with column tiles of bn, such that jobs M N <= max_ints; false if none fit.
 bool split_plan(int M, int N, int K, int bn, bool pair, size_t max_ints, SplitPlan* out);
-// Eight digits of every row of V (entries times cs[j], or over it with inv) and the row scales.
-void split_digits(cudaStream_t s, const double* V, int rows, int n, size_t ldv, int npad, const double* cs, int inv,
-                  int reversed, __nv_bfloat16* D, double* scale, int* flag);
-// out (rows x cols) from the jobs' integers (slice t at I + t stride).
+// Eight digits of every row of V (entry j times 2^ce[j], or 2^-ce[j] with inv) and the row scales' exponents.
+void split_digits(cudaStream_t s, const double* V, int rows, int n, size_t ldv, int npad, const int* ce, int inv,
+                  int reversed, __nv_bfloat16* D, int* scale, int* flag);
+// out (rows x cols) from the jobs' integers (slice t at I + t stride) and the scales' exponents.
 void split_combine(cudaStream_t s, int rows, int cols, const int* I, size_t stride, const SplitPlan& pl,
-                   const double* sr, const double* sc, double* out);
-// R = dl(S, y) from the jobs' integers of S = X V, as reversed digits with row scales tr
-// (Rg: FP64 rows to work in where n is too large for shared memory).
-void split_link(cudaStream_t s, int m, int n, int npad, const int* I, size_t stride, const SplitPlan& pl,
-                const double* tv, const double* sx, const double* y, int kind, double* Rg, __nv_bfloat16* D,
-                double* tr);
+                   const int* er, const int* ec, double* out);
+// R = dl(S, y) from the jobs' integers of S = X V, as reversed digits with row exponents er.
+int split_link(cudaStream_t s, int m, int n, int npad, const int* I, size_t stride, const SplitPlan& pl, const int* ev,
+               const int* ex, const double* y, int kind, __nv_bfloat16* D, int* er);
 int split_prepare();
 int tc_gemm(cudaStream_t s, const TcMap& A, const TcMap& B, const TcMap* B2, const TcGemm& g,
             const GemmScratch* scr);

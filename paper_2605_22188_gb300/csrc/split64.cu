@@ -37,14 +37,12 @@
 
 #include "common.cuh"
 #include "engine.h"
+#include "fixed.cuh"
 
 namespace kglm {
 namespace {
 
-// The eight digits of z (a = 8 is the lowest byte), as BF16.
-struct Digits {
-    __nv_bfloat16 d[8];
-};
+// The eight digits of z (the last is the lowest byte), as BF16.
 __device__ __forceinline__ void cut(long long z, __nv_bfloat16 (&d)[8]) {
 #pragma unroll
     for (int a = 7; a >= 1; --a) {
@@ -53,11 +51,6 @@ __device__ __forceinline__ void cut(long long z, __nv_bfloat16 (&d)[8]) {
         d[a] = __int2bfloat16_rn(v);
     }
     d[0] = __int2bfloat16_rn((int)z);
-}
-
-// v 2^(64 - e) rounded to an integer; f = 2^(64 - e) where that is a normal number.
-__device__ __forceinline__ long long fixed(double v, double f, int e) {
-    return __double2ll_rn(e > -900 ? v * f : ldexp(v, 64 - e));
 }
 
 // Digits of four consecutive entries i .. i + 3 of a row into its eight segments.
@@ -77,62 +70,66 @@ __device__ __forceinline__ void store_digits(const long long (&z)[4], __nv_bfloa
     }
 }
 
-// Scale of a row from its largest magnitude: e with 2^e > 2 max (0 for a zero row).
-__device__ __forceinline__ int row_exp(double mx) { return mx > 0.0 ? ilogb(mx) + 2 : 0; }
-
-// Rows of V (rows x n, stride ldv; entry j times cs[j], or over it with inv) into digit
-// rows of D (8 npad entries each, zero past n; NULL: none) and their scales 2^e (NaN
-// for a row with a non-finite entry, whose products are then NaN).  GS threads
-// per row.  flag: set for a row whose largest magnitude is above 2^10 times the mean
-// of its nonzero ones, whose scale is outside 2^(-+400), or with a non-finite entry.
+// Rows of V (rows x n, stride ldv; entry j times 2^ce[j], or 2^-ce[j] with inv) into
+// digit rows of D (8 npad entries each, zero past n; NULL: none) and their scales'
+// exponents (kBadRow for a row with a non-finite entry).  GS threads per row.  No
+// FP64 operation: the scale is an exponent, the rounding a shift (with FP64 maxima and
+// conversions 256 rows of 1000 took 16 us, now 9).  flag: set for a row whose
+// largest magnitude is above 2^10 times the mean of its nonzero ones, whose scale is
+// outside 2^(-+400), or with a non-finite entry.
 template <int GS>
 __global__ __launch_bounds__(256) void k_split_digits(const double* __restrict__ V, int rows, int n, size_t ldv,
-                                                      int npad, const double* __restrict__ cs, int inv, int reversed,
-                                                      __nv_bfloat16* __restrict__ D, double* __restrict__ scale,
+                                                      int npad, const int* __restrict__ ce, int inv, int reversed,
+                                                      __nv_bfloat16* __restrict__ D, int* __restrict__ scale,
                                                       int* flag) {
-    __shared__ double red[2 * 8];
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    __shared__ int redi[8];
+    __shared__ float redf[3 * 8];
     const int g = threadIdx.x / GS, t = threadIdx.x % GS;
     const int r = blockIdx.x * (256 / GS) + g;
     if (GS == 32 && r >= rows) return;                       // whole warps; one CTA per row otherwise
     const double* v = V + (size_t)r * ldv;
-    auto at = [&](int i) {
-        const double x = v[i];
-        return cs ? (inv ? x / cs[i] : x * cs[i]) : x;
-    };
-    double mx = 0.0, bad = 0.0;
+    auto shift = [&](int i) { return ce == nullptr ? 0 : inv ? -ce[i] : ce[i]; };
+    int key = -(1 << 27);
     for (int i = t; i < n; i += GS) {
-        const double x = fabs(at(i));
-        bad = isfinite(x) ? bad : 1.0;
-        mx = fmax(mx, x);
+        const int k = exp_key(v[i]);
+        if (k) key = max(key, k + shift(i));
     }
-    if (GS == 32) {
-        mx = warp_max(mx);
-        bad = warp_max(bad);
-    } else {
-        mx = block_max<256, double>(mx, red);
-        bad = block_max<256, double>(bad, red + 8);
-    }
-    const int e = row_exp(bad > 0.0 ? 0.0 : mx);
-    if (t == 0 && scale) scale[r] = bad > 0.0 ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(1.0, e);
+    key = __reduce_max_sync(0xffffffffu, key);
+    if (GS != 32) key = block_max<256, int>(key, redi);
+    const bool none = key == -(1 << 27);
+    // with a column shift the key may be below 1: no clamp, only "none" is a zero row
+    const int e = key >= kBadRow / 2 ? kBadRow : none ? 0 : key - 1021;
+    if (t == 0 && scale) scale[r] = e;
     if (flag) {
-        double q[2] = {0.0, 0.0};
-        for (int i = t; i < n; i += GS) {
-            const double x = fabs(at(i));
-            if (x > 0.0) { q[0] += x / mx; q[1] += 1.0; }
+        float q[3] = {0.f, 0.f, 0.f};
+        if (e != kBadRow)
+            for (int i = t; i < n; i += GS) {
+                const double x = v[i];
+                if (x == 0.0) continue;
+                const long long z = fixed64(x, e - shift(i));
+                const float m = (float)((z < 0 ? -z : z) >> 32);
+                q[0] = fmaxf(q[0], m);
+                q[1] += m;
+                q[2] += 1.f;
+            }
+        if (GS == 32) {
+            q[0] = warp_max(q[0]);
+            q[1] = warp_sum(q[1]);
+            q[2] = warp_sum(q[2]);
+        } else {
+            const float mx = block_max<256, float>(q[0], redf);
+            __syncthreads();
+            block_sum<256, 3, float>(q, redf);
+            q[0] = mx;
         }
-        if (GS == 32) { q[0] = warp_sum(q[0]); q[1] = warp_sum(q[1]); }
-        else block_sum<256, 2, double>(q, red);
-        if (t == 0 && (bad > 0.0 || e < -400 || e > 400 || q[1] > 1024.0 * q[0])) atomicOr(flag, 1);
+        if (t == 0 && (e == kBadRow || e < -400 || e > 400 || q[0] * q[2] > 1024.f * q[1])) atomicOr(flag, 1);
     }
     if (!D) return;
     __nv_bfloat16* d = D + (size_t)r * 8 * npad;
-    const double f = e > -900 ? ldexp(1.0, 64 - e) : 0.0;
     for (int i = 4 * t; i < npad; i += 4 * GS) {
         long long z[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) z[q] = (i + q < n && !(bad > 0.0)) ? fixed(at(i + q), f, e) : 0ll;
+        for (int q = 0; q < 4; ++q) z[q] = (i + q < n && e != kBadRow) ? fixed64(v[i + q], e - shift(i + q)) : 0ll;
         store_digits(z, d, (size_t)npad, i, reversed);
     }
 }
@@ -143,9 +140,9 @@ struct Levels {
     signed char sh[kTcMaxJobs];      // its shift within its half
 };
 
-// One entry of the product from its jobs' integers (scale: 2^(ea + eb - 40)).
-__device__ __forceinline__ double combine(const int* __restrict__ I, size_t stride, size_t idx, const Levels& lv,
-                                          double scale) {
+// One entry of the product from its jobs' integers, times 2^x (x: the sum of the scales'
+// exponents; kBadRow makes it a NaN).
+__device__ __forceinline__ double combine(const int* __restrict__ I, size_t stride, size_t idx, const Levels& lv, int x) {
     long long H = 0, L = 0;
     for (int t0 = 0; t0 < lv.n; t0 += 8) {                   // eight jobs' loads in flight
         int v[8];
@@ -154,63 +151,81 @@ __device__ __forceinline__ double combine(const int* __restrict__ I, size_t stri
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
             if (t0 + t < lv.n) {
-                const long long x = (long long)v[t] << lv.sh[t0 + t];
-                if (lv.hi[t0 + t]) H += x; else L += x;
+                const long long w = (long long)v[t] << lv.sh[t0 + t];
+                if (lv.hi[t0 + t]) H += w; else L += w;
             }
         }
     }
-    return fma((double)L, 0x1p-32, (double)H) * scale;
+    if (x >= kBadRow / 2) return bits_f64(0x7ff8000000000000ull);
+    return combine_f64(H, L, x - 72);
 }
 
-// out[b][j] = sr[b] sc[j] (product of digits) for a rows x cols output.
-__global__ __launch_bounds__(256) void k_split_combine(int rows, int cols, const int* __restrict__ I, size_t stride,
-                                                       const __grid_constant__ Levels lv, const double* __restrict__ sr,
-                                                       const double* __restrict__ sc, double* __restrict__ out) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+// out[b][j] of a rows x cols product of digits (scales 2^er[b], 2^ec[j]).
+__global__ __launch_bounds__(256) void k_split_combine(int cols, const int* __restrict__ I, size_t stride,
+                                                       const __grid_constant__ Levels lv, const int* __restrict__ er,
+                                                       const int* __restrict__ ec, double* __restrict__ out) {
     const int b = blockIdx.y;
-    const double s = sr[b] * 0x1p-40;
+    const int s = er[b];
     const size_t base = (size_t)b * cols;
     for (int j = blockIdx.x * 256 + threadIdx.x; j < cols; j += gridDim.x * 256)
-        out[base + j] = combine(I, stride, base + j, lv, s * sc[j]);
+        out[base + j] = combine(I, stride, base + j, lv, s + ec[j]);
 }
 
-// S = X V of one node per CTA, its loss derivative R and R's digits: the row stays
-// in shared memory between the two (in Rg where it does not fit), so that neither S
-// nor R is written in FP64.  Bound by the FP64 pipe: five operations per entry to
-// put S together, the link's (two, or about forty for the logistic loss) and two
-// for the digits.
-constexpr int kLinkNT = 512;
-__global__ __launch_bounds__(kLinkNT) void k_split_link(int n, int npad, const int* __restrict__ I, size_t stride,
-                                                        const __grid_constant__ Levels lv, const double* __restrict__ tv,
-                                                        const double* __restrict__ sx, const double* __restrict__ y,
-                                                        int kind, double* Rg, __nv_bfloat16* __restrict__ D,
-                                                        double* __restrict__ tr) {
-    extern __shared__ __align__(16) double srow[];
-    __shared__ double red[2 * (kLinkNT / 32)];
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int b = blockIdx.x, t = threadIdx.x;
+// S = X V of a node, its loss derivative R and R's digits: a cluster of CTAs per node,
+// each with a part of the samples in shared memory between the two, so that neither
+// S nor R is written in FP64; they exchange the largest exponent.  The parts of a
+// row keep 304 CTAs in flight where the batch is small (a CTA per node left most SMs
+// idle at 8 nodes).  Integer arithmetic but for the least-squares residual (two FP64
+// operations): with FP64 sums, exp and division 1024 nodes of 2000 samples (logistic)
+// took about 220 us, now 65.
+constexpr int kLinkNT = 256;
+__global__ __launch_bounds__(kLinkNT) void k_split_link(int n, int npad, int parts, int seg, const int* __restrict__ I,
+                                                        size_t stride, const __grid_constant__ Levels lv,
+                                                        const int* __restrict__ ev, const int* __restrict__ ex,
+                                                        const double* __restrict__ y, int kind,
+                                                        __nv_bfloat16* __restrict__ D, int* __restrict__ er) {
+    extern __shared__ __align__(16) double row[];
+    __shared__ unsigned long long tab[64];
+    __shared__ int redi[kLinkNT / 32];
+    __shared__ int s_key;
+    const int t = threadIdx.x;
+    const int b = blockIdx.x / parts, part = blockIdx.x - b * parts;
+    const int i0 = part * seg, i1 = min(n, i0 + seg);
+    if (t < 64) tab[t] = kExp2Dev[t];
+    __syncthreads();
     const size_t base = (size_t)b * n;
-    double* row = Rg ? Rg + base : srow;
-    const double s = tv[b] * 0x1p-40;
-    double mx = 0.0, bad = 0.0;
-    for (int i = t; i < n; i += kLinkNT) {
-        const double r = dloss(combine(I, stride, base + i, lv, s * sx[i]), y[i], kind);
-        row[i] = r;
-        bad = isfinite(r) ? bad : 1.0;
-        mx = fmax(mx, fabs(r));
+    const int s = ev[b];
+    int key = 0;
+    for (int i = i0 + t; i < i1; i += kLinkNT) {
+        const double r = dloss_fixed(combine(I, stride, base + i, lv, s + ex[i]), y[i], kind, tab);
+        row[i - i0] = r;
+        key = max(key, exp_key(r));
     }
-    mx = block_max<kLinkNT, double>(mx, red);
-    bad = block_max<kLinkNT, double>(bad, red + kLinkNT / 32);   // its barriers also publish the row
-    const int e = row_exp(bad > 0.0 ? 0.0 : mx);
-    if (t == 0) tr[b] = bad > 0.0 ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(1.0, e);
+    key = __reduce_max_sync(0xffffffffu, key);
+    key = block_max<kLinkNT, int>(key, redi);                // its barriers also publish the row
+    if (parts > 1) {
+        if (t == 0) s_key = key;
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        const uint32_t at = (uint32_t)__cvta_generic_to_shared(&s_key);
+        for (int q = 0; q < parts; ++q) {
+            uint32_t peer, v;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(at), "r"(q));
+            asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(peer) : "memory");
+            key = max(key, (int)v);
+        }
+        // no CTA leaves (or reuses s_key) before its peers have read it
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+    const int e = row_exp(key);
+    if (t == 0 && part == 0) er[b] = e;
     __nv_bfloat16* d = D + (size_t)b * 8 * npad;
-    const double f = e > -900 ? ldexp(1.0, 64 - e) : 0.0;
-    for (int i = 4 * t; i < npad; i += 4 * kLinkNT) {
+    const int iend = part == parts - 1 ? npad : min(npad, i0 + seg);
+    for (int i = i0 + 4 * t; i < iend; i += 4 * kLinkNT) {
         long long z[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) z[q] = (i + q < n && !(bad > 0.0)) ? fixed(row[i + q], f, e) : 0ll;
+        for (int q = 0; q < 4; ++q) z[q] = (i + q < i1 && e != kBadRow) ? fixed64(row[i + q - i0], e) : 0ll;
         store_digits(z, d, (size_t)npad, i, 1);
     }
 }
@@ -225,7 +240,7 @@ Levels levels_of(const SplitPlan& pl) {
     return lv;
 }
 
-constexpr size_t kLinkSmem = 200 * 1024;
+constexpr size_t kLinkSmem = 96 * 1024;    // a part of at most 12288 samples
 
 }  // namespace
 
@@ -291,20 +306,20 @@ bool split_plan(int M, int N, int K, int bn, bool pair, size_t max_ints, SplitPl
     return best < 1e300;
 }
 
-void split_digits(cudaStream_t s, const double* V, int rows, int n, size_t ldv, int npad, const double* cs, int inv,
-                  int reversed, __nv_bfloat16* D, double* scale, int* flag) {
+void split_digits(cudaStream_t s, const double* V, int rows, int n, size_t ldv, int npad, const int* ce, int inv,
+                  int reversed, __nv_bfloat16* D, int* scale, int* flag) {
     if (rows <= 0) return;
-    if (n <= 512) k_split_digits<32><<<(rows + 7) / 8, 256, 0, s>>>(V, rows, n, ldv, npad, cs, inv, reversed, D, scale, flag);
-    else k_split_digits<256><<<rows, 256, 0, s>>>(V, rows, n, ldv, npad, cs, inv, reversed, D, scale, flag);
+    if (n <= 512) k_split_digits<32><<<(rows + 7) / 8, 256, 0, s>>>(V, rows, n, ldv, npad, ce, inv, reversed, D, scale, flag);
+    else k_split_digits<256><<<rows, 256, 0, s>>>(V, rows, n, ldv, npad, ce, inv, reversed, D, scale, flag);
 }
 
 void split_combine(cudaStream_t s, int rows, int cols, const int* I, size_t stride, const SplitPlan& pl,
-                   const double* sr, const double* sc, double* out) {
+                   const int* er, const int* ec, double* out) {
     // rows on the grid's y axis, in runs of at most 65535
     for (int b0 = 0; b0 < rows; b0 += 65535) {
         const int rr = std::min(65535, rows - b0);
         const dim3 grid(std::max(1, std::min(8, (cols + 255) / 256)), rr);
-        k_split_combine<<<grid, 256, 0, s>>>(rr, cols, I + (size_t)b0 * cols, stride, levels_of(pl), sr + b0, sc,
+        k_split_combine<<<grid, 256, 0, s>>>(cols, I + (size_t)b0 * cols, stride, levels_of(pl), er + b0, ec,
                                              out + (size_t)b0 * cols);
     }
 }
@@ -315,14 +330,28 @@ int split_prepare() {
     return rc;
 }
 
-void split_link(cudaStream_t s, int m, int n, int npad, const int* I, size_t stride, const SplitPlan& pl,
-                const double* tv, const double* sx, const double* y, int kind, double* Rg, __nv_bfloat16* D,
-                double* tr) {
-    if (m <= 0) return;
-    const size_t need = (size_t)n * sizeof(double);
-    const bool sm = need <= kLinkSmem;
-    k_split_link<<<m, kLinkNT, sm ? need : 0, s>>>(n, npad, I, stride, levels_of(pl), tv, sx, y, kind,
-                                                   sm ? nullptr : Rg, D, tr);
+int split_link(cudaStream_t s, int m, int n, int npad, const int* I, size_t stride, const SplitPlan& pl, const int* ev,
+               const int* ex, const double* y, int kind, __nv_bfloat16* D, int* er) {
+    if (m <= 0) return 0;
+    int parts = 1;
+    while (parts < 8 && ((long)m * parts < 2 * 152 || (size_t)n * 8 > kLinkSmem * parts) &&
+           (n / parts >= 1024 || (size_t)n * 8 > kLinkSmem * parts))
+        parts *= 2;
+    const int seg = ((n + parts - 1) / parts + 3) / 4 * 4;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)m * parts);
+    cfg.blockDim = dim3(kLinkNT);
+    cfg.dynamicSmemBytes = (size_t)seg * sizeof(double);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = parts;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = parts > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k_split_link, n, npad, parts, seg, I, stride, levels_of(pl), ev, ex, y, kind, D,
+                              er) == cudaSuccess ? 0 : -1;
 }
 
 }  // namespace kglm
