@@ -175,10 +175,70 @@ __device__ __forceinline__ void stream_pad(unsigned char* rows, int p, int W, in
     __syncwarp();
 }
 
-// A. node b's masks, G and V rows into the row set `rows` (asynchronous copies,
-// one commit group).
+// G's row in shared memory (its first slice) plus the other split slices, in order,
+// several coordinates' and slices' loads in flight.
 template <int VEC>
-__device__ __forceinline__ void stream_issue(const ProxArgs& a, int b, int lane, unsigned char* rows) {
+__device__ __forceinline__ void stream_sum(const ProxArgs& a, size_t base, int lane, float* su) {
+    using VT = typename std::conditional<VEC == 4, float4, float>::type;
+    constexpr int U = VEC == 4 ? 2 : 4, SB = 4;
+    const int nq = a.p / VEC;
+    const float* G = a.Gpart + base;
+    auto add = [](VT& x, const VT& y) {
+        if constexpr (VEC == 4) { x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w; }
+        else x += y;
+    };
+    for (int q0 = lane; q0 < nq; q0 += 32 * U) {
+        VT g[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (q0 + 32 * u < nq) g[u] = reinterpret_cast<const VT*>(su)[q0 + 32 * u];
+        for (int s0 = 1; s0 < a.gsplits; s0 += SB) {
+            VT t[SB][U];
+#pragma unroll
+            for (int s = 0; s < SB; ++s)
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (s0 + s < a.gsplits && q0 + 32 * u < nq)
+                        t[s][u] = reinterpret_cast<const VT*>(G + (size_t)(s0 + s) * a.gstride)[q0 + 32 * u];
+#pragma unroll
+            for (int s = 0; s < SB; ++s)
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (s0 + s < a.gsplits && q0 + 32 * u < nq) add(g[u], t[s][u]);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (q0 + 32 * u < nq) reinterpret_cast<VT*>(su)[q0 + 32 * u] = g[u];
+    }
+    __syncwarp();
+}
+
+// The same sum by the whole CTA, for the node of its first warp where every CTA has at
+// most one node: a batch that small has up to 16 slices, whose loads one warp takes
+// longer over than over much of the rest (a launch between its events: 28.6 us at one
+// node of p = 1000, now 18.9; 17.9 at 64 nodes of p = 611, now 15.9).
+__device__ __forceinline__ void stream_sum_cta(const ProxArgs& a, int b, unsigned char* rows0) {
+    float* su = reinterpret_cast<float*>(rows0 + 2 * mask_bytes(a.W));
+    const float* G = a.Gpart + (size_t)b * a.p;
+    for (int j = threadIdx.x; j < a.p; j += blockDim.x) {
+        float g = G[j];
+        for (int s0 = 1; s0 < a.gsplits; s0 += 8) {
+            float t[8];
+#pragma unroll
+            for (int s = 0; s < 8; ++s) t[s] = s0 + s < a.gsplits ? G[(size_t)(s0 + s) * a.gstride + j] : 0.f;
+#pragma unroll
+            for (int s = 0; s < 8; ++s)
+                if (s0 + s < a.gsplits) g += t[s];
+        }
+        su[j] = g;
+    }
+    __syncthreads();
+}
+
+// A. node b's masks, G and V rows into the row set `rows` (asynchronous copies,
+// one commit group); summed: G is there already.
+template <int VEC>
+__device__ __forceinline__ void stream_issue(const ProxArgs& a, int b, int lane, unsigned char* rows, bool summed) {
     const int p = a.p, W = a.W, nq = p / VEC;
     uint32_t* smi = reinterpret_cast<uint32_t*>(rows);
     uint32_t* smo = reinterpret_cast<uint32_t*>(rows + mask_bytes(W));
@@ -193,10 +253,10 @@ __device__ __forceinline__ void stream_issue(const ProxArgs& a, int b, int lane,
     }
     for (int q = lane; q < nq; q += 32) {
         if constexpr (VEC == 4) {
-            cp_async16(su + 4 * q, G0 + 4 * q);
+            if (!summed) cp_async16(su + 4 * q, G0 + 4 * q);
             cp_async16(sv + 4 * q, V + 4 * q);
         } else {
-            cp_async4(su + q, G0 + q);
+            if (!summed) cp_async4(su + q, G0 + q);
             cp_async4(sv + q, V + q);
         }
     }
@@ -207,7 +267,8 @@ __device__ __forceinline__ void stream_issue(const ProxArgs& a, int b, int lane,
 // stream_issue (the node's scalars are read while they arrive), laid out for
 // a.p and a.W with the padding zeroed.
 template <int VEC>
-__device__ __forceinline__ void stream_node(const ProxArgs& a, int b, int lane, WarpHdr& h, unsigned char* rows) {
+__device__ __forceinline__ void stream_node(const ProxArgs& a, int b, int lane, WarpHdr& h, unsigned char* rows,
+                                            bool summed) {
     const int p = a.p, p4 = (p + 3) >> 2, W = a.W;
     uint32_t* smi = reinterpret_cast<uint32_t*>(rows);
     uint32_t* smo = reinterpret_cast<uint32_t*>(rows + mask_bytes(W));
@@ -228,23 +289,25 @@ __device__ __forceinline__ void stream_node(const ProxArgs& a, int b, int lane, 
         const float tg = tau_h > 0.f ? tau_h * kTauHint : __builtin_huge_valf();
 
         if (lane == 0) { h.nj1 = 0; h.ncand = 0; }
+        // the momentum's FP64 root and quotient (a chain of some fifty operations on a pipe
+        // that takes one in 16 cycles) run while the rows arrive, not at the end
+        double t_keep = 0.0;
+        float coef = 0.f;
+        if (lane == 0) {
+            t_keep = 0.5 * (1.0 + sqrt(1.0 + 4.0 * tprev * tprev));
+            coef = (float)((tprev - 1.0) / t_keep);
+        }
+        coef = __shfl_sync(0xffffffffu, coef, 0);
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncwarp();
-        // u = v - eta G (split slices after the first are added from global memory, in
-        // order); J0 entries become 0 now, J1 entries once they are listed below.
+        if (!summed && a.gsplits > 1) stream_sum<VEC>(a, base, lane, su);
+        // u = v - eta G; J0 entries become 0 now, J1 entries once they are listed below.
         // Two running top-two pairs (even and odd positions) keep the chains short.
         float t1 = 0.f, t2 = 0.f, t1b = 0.f, t2b = 0.f;
         for (int q = lane; q < p4; q += 32) {
             float4 g = su4[q];
             const float4 v = reinterpret_cast<const float4*>(sv)[q];
             const int j0 = 4 * q;
-            for (int s = 1; s < a.gsplits; ++s) {
-                const float* gs = a.Gpart + (size_t)s * a.gstride + base;
-                g.x += gs[j0];
-                if (j0 + 1 < p) g.y += gs[j0 + 1];
-                if (j0 + 2 < p) g.z += gs[j0 + 2];
-                if (j0 + 3 < p) g.w += gs[j0 + 3];
-            }
             const uint32_t wi = smi[j0 >> 5] >> (j0 & 31), wo = smo[j0 >> 5] >> (j0 & 31);
             const float uu[4] = {v.x - eta * g.x, v.y - eta * g.y, v.z - eta * g.z, v.w - eta * g.w};
             float o[4];
@@ -483,12 +546,6 @@ __device__ __forceinline__ void stream_node(const ProxArgs& a, int b, int lane, 
             if (kglm_check((unsigned)j < (unsigned)p, a.chk, kChkProx)) su[j] = sgn_mag(u, fminf(fabsf(u) / c1, M));
         }
         __syncwarp();
-        double t_keep = 0.0, c_keep = 0.0;
-        if (lane == 0) {
-            t_keep = 0.5 * (1.0 + sqrt(1.0 + 4.0 * tprev * tprev));
-            c_keep = (tprev - 1.0) / t_keep;
-        }
-        const float coef = (float)__shfl_sync(0xffffffffu, c_keep, 0);
         float d0 = 0.f, d1 = 0.f;
         const size_t ob = (size_t)b * a.op_ld;
         constexpr int UN = VEC == 4 ? 4 : 8;          // beta_old loads in flight per lane
@@ -553,13 +610,19 @@ __global__ void __launch_bounds__(32 * kStreamMaxWarps, 1) k_prox_stream(ProxArg
     WarpHdr& h = *reinterpret_cast<WarpHdr*>(wbase);
     unsigned char* rows = wbase + align16(sizeof(WarpHdr));
     stream_pad(rows, a.p, a.W, lane);
+    // one node per CTA and split slices to add: by all warps (its row padding was zeroed above)
+    const bool coop = a.m <= (int)gridDim.x && a.gsplits > 1;
+    if (coop) {
+        if (a.active != nullptr && a.active[blockIdx.x] == 0) return;
+        stream_sum_cta(a, blockIdx.x, smem + align16(sizeof(WarpHdr)));
+    }
     // nodes go round the CTAs first (node b to CTA b mod grid), so that every SM
     // holds the same number of nodes and a last partial round is spread over all
     // SMs rather than packed onto the first few
     for (int b = warp * gridDim.x + blockIdx.x; b < a.m; b += gridDim.x * wpc) {
         if (a.active != nullptr && a.active[b] == 0) continue;
-        stream_issue<VEC>(a, b, lane, rows);
-        stream_node<VEC>(a, b, lane, h, rows);
+        stream_issue<VEC>(a, b, lane, rows, coop);
+        stream_node<VEC>(a, b, lane, h, rows, coop);
     }
 }
 
@@ -575,6 +638,17 @@ __global__ void __launch_bounds__(32 * kStreamMaxWarps, 1) k_prox_stream_group(c
     WarpHdr& h = *reinterpret_cast<WarpHdr*>(wbase);
     unsigned char* rows = wbase + align16(sizeof(WarpHdr));
     int last = -1;
+    // as in k_prox_stream: one node per CTA, its split slices added by all warps
+    bool coop = false;
+    if (g.nbase[g.np] <= (int)gridDim.x) {
+        int pi = 0;
+        while (pi + 1 < g.np && (int)blockIdx.x >= g.nbase[pi + 1]) ++pi;
+        const ProxArgs& a = g.a[pi];
+        const int b = (int)blockIdx.x - g.nbase[pi];
+        if (a.active != nullptr && a.active[b] == 0) return;
+        coop = a.gsplits > 1;
+        if (coop) stream_sum_cta(a, b, smem + align16(sizeof(WarpHdr)));
+    }
     for (int t = warp * gridDim.x + blockIdx.x; t < g.nbase[g.np]; t += gridDim.x * wpc) {
         int pi = 0;
         while (pi + 1 < g.np && t >= g.nbase[pi + 1]) ++pi;
@@ -585,8 +659,8 @@ __global__ void __launch_bounds__(32 * kStreamMaxWarps, 1) k_prox_stream_group(c
             stream_pad(rows, a.p, a.W, lane);
             last = pi;
         }
-        stream_issue<VEC>(a, b, lane, rows);
-        stream_node<VEC>(a, b, lane, h, rows);
+        stream_issue<VEC>(a, b, lane, rows, coop);
+        stream_node<VEC>(a, b, lane, h, rows, coop);
     }
 }
 
