@@ -332,7 +332,7 @@ kglm_status kglm_configure(kglm_ctx* ctx, const kglm_tune* cfg);
  * any allocation).  Host-only arithmetic, no CUDA call.  Not included: one
  * max_batch x p FP64 buffer that kglm_push_nodes with warm_B, and one that
  * kglm_xtz, allocate on first use; and in the FP64 mode the digits of the
- * tensor-core products (about 32 n p + 56 max_batch n + 112 max_batch p bytes),
+ * tensor-core products (about 32 n p + 16 max_batch (n + p) + 32 max_batch max(n, p) bytes),
  * allocated at the first batch large enough for them and left out, with the
  * products on the CUDA cores, where hbm_budget or the device does not hold them.  KGLM_EINVAL for a desc kglm_create would
  * reject on its sizes, ranges or enums. */

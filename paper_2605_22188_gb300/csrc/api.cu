@@ -125,8 +125,10 @@ struct kglm_ctx {
     ExactPlan xplan{};
     __nv_bfloat16 *DX = nullptr, *DZ = nullptr;
     double *xsig = nullptr, *ztau = nullptr, *Qerr = nullptr;
-    float* Qs = nullptr;
-    size_t qs_slices = 0;         // partial slices of mcap x p
+    int* Qi = nullptr;
+    size_t qi_slices = 0;         // integer slices of mcap x p
+    SplitPlan pC{};               // jobs of the certificate product at batch size mC
+    int mC = -1;
     TcMap mAz{}, mBx{};
     int bnx = 0;
     int gsplit_max = 4;
@@ -403,15 +405,14 @@ void split_setup(kglm_ctx* c) {
     if (q.tried) return;
     q.tried = true;
     const size_t n = c->n, p = c->p, mc = c->mcap;
-    // 65536: levels of at most 2032 K slices a job make at most 24 jobs (the cap below always holds them)
+    // 65536: levels in pieces of at most 2032 K slices always make a plan
     if (!c->f64 || n > 65536 || !isfinite(c->eta) || c->M > 1e100) return;
     if (split_prepare() != 0 || tc_prepare() != 0) return;
     q.pk = (int)((p + 63) / 64 * 64);
     q.nk = (int)((n + 63) / 64 * 64);
     q.bnS = tc_tile_cols((int)n);
     q.bnG = tc_tile_cols((int)p);
-    // room for whole levels of S, and for levels in pieces of G (or of a small batch)
-    q.cap = std::max(std::max(10 * mc * n, 24 * mc * p), (size_t)(8 << 20));
+    q.cap = 8 * mc * std::max(n, p);                   // a slice of integers per level
     const size_t need = 16 * ((n + mc) * q.pk + (p + mc) * q.nk) + 4 * (n + p + 2 * mc) + 4 * q.cap + 64;
     if (c->d.hbm_budget > 0 && (int64_t)(c->bytes + need) > c->d.hbm_budget) return;
     const size_t had = c->allocs.size(), bytes0 = c->bytes;
@@ -466,36 +467,41 @@ void split_setup(kglm_ctx* c) {
 
 bool split_on(const kglm_ctx* c, int m) { return c->sp.on && split_pays(c, m); }
 
-// The integers of S = X V (or X beta) from V's digits, or of X^T R (X^T zeta) from
-// R's; the plan of a batch size is kept for the next product of that size.
-const SplitPlan& split_product(kglm_ctx* c, int m, bool grad) {
-    kglm_ctx::Split64& q = c->sp;
-    SplitPlan& pl = grad ? q.pG : q.pS;
-    int& have = grad ? q.mG : q.mS;
-    const int N = grad ? c->p : c->n, K = grad ? c->n : c->p, bn = grad ? q.bnG : q.bnS;
+// A product of digits by its plan, kept for the next product of that batch size; levels
+// in pieces are added to zeroed integers.
+void digit_product(kglm_ctx* c, int m, int N, int K, int nd, int bn, const TcMap& A, const TcMap& B, int* I,
+                   SplitPlan& pl, int& have) {
     if (have != m) {
-        if (!split_plan(m, N, K, bn, true, q.cap, &pl)) throw Fail{KGLM_ECUDA, "no plan for an FP64 digit product"};
+        if (!split_plan(m, N, K, nd, bn, true, &pl)) throw Fail{KGLM_ECUDA, "no plan for a digit product"};
         have = m;
     }
-    if (tc_gemm_jobs(c->st, grad ? q.mR : q.mV, grad ? q.mXt : q.mX, m, N, bn, pl.jobs, pl.njobs,
-                     reinterpret_cast<float*>(q.I), (size_t)m * N, N, c->d_tcerr, 1, kSplitChunk) != 0)
-        throw Fail{KGLM_ECUDA, "FP64 digit product setup failed"};
+    const size_t mn = (size_t)m * N;
+    const bool add = pl.njobs > nd;
+    if (add) CK(cudaMemsetAsync(I, 0, sizeof(int) * nd * mn, c->st));
+    if (tc_gemm_jobs(c->st, A, B, m, N, bn, pl.jobs, pl.njobs, I, mn, N, c->d_tcerr, 1, kSplitChunk, add) != 0)
+        throw Fail{KGLM_ECUDA, "digit product setup failed"};
     check_launch();
-    return pl;
+}
+
+// The integers of S = X V (or X beta) from V's digits, or of X^T R (X^T zeta) from R's.
+void split_product(kglm_ctx* c, int m, bool grad) {
+    kglm_ctx::Split64& q = c->sp;
+    if (grad) digit_product(c, m, c->p, c->n, 8, q.bnG, q.mR, q.mXt, q.I, q.pG, q.mG);
+    else digit_product(c, m, c->n, c->p, 8, q.bnS, q.mV, q.mX, q.I, q.pS, q.mS);
 }
 
 // S = X V for m rows of V (m x p FP64) into out, and X^T R for R (m x n) into out.
 void split_xv(kglm_ctx* c, int m, const double* V, double* out) {
     kglm_ctx::Split64& q = c->sp;
     split_digits(c->st, V, m, c->p, c->p, q.pk, q.sxt, 0, 1, q.DV, q.tv, nullptr);
-    const SplitPlan& pl = split_product(c, m, false);
-    split_combine(c->st, m, c->n, q.I, (size_t)m * c->n, pl, q.tv, q.sx, out);
+    split_product(c, m, false);
+    split_combine(c->st, m, c->n, q.I, (size_t)m * c->n, q.tv, q.sx, out);
 }
 void split_xtr(kglm_ctx* c, int m, const double* R, double* out) {
     kglm_ctx::Split64& q = c->sp;
     split_digits(c->st, R, m, c->n, c->n, q.nk, nullptr, 0, 1, q.DR, q.tr, nullptr);
-    const SplitPlan& pl = split_product(c, m, true);
-    split_combine(c->st, m, c->p, q.I, (size_t)m * c->p, pl, q.tr, q.sxt, out);
+    split_product(c, m, true);
+    split_combine(c->st, m, c->p, q.I, (size_t)m * c->p, q.tr, q.sxt, out);
 }
 
 // X^T zeta of the batch's dual points (c->zeta, m x n): FP64 GEMM into c->Q,
@@ -504,27 +510,22 @@ void split_xtr(kglm_ctx* c, int m, const double* R, double* out) {
 // arguments.
 void xtzeta(kglm_ctx* c, int m, CertArgs& a) {
     const int n = c->n, p = c->p;
-    a.Qs = nullptr;
+    a.Qi = nullptr;
     if (!c->cexact) {
         gemm_nt_f64(c->st, m, p, n, c->zeta, n, c->Xt64, n, c->Q, p, &c->gs64);
         return;
     }
     const ExactPlan& x = c->xplan;
     // the batch's certificate makes zeta's digits in its dual point pass
-    if (a.DZ == nullptr) exact_digits(c->st, c->zeta, m, n, (size_t)n, x.npad, x.nd, x.beta, 1, c->DZ, c->ztau);
-    ExactPlan pl = x;
-    const int tiles = ((p + c->bnx - 1) / c->bnx) * ((m + 127) / 128);
-    exact_plan_widen(&pl, tiles, c->qs_slices * (size_t)c->mcap / (size_t)m);
-    if (tc_gemm_jobs(c->st, c->mAz, c->mBx, m, p, c->bnx, pl.jobs, pl.njobs, c->Qs, (size_t)m * p, p, c->d_tcerr,
-                     c->pair) != 0)
-        throw Fail{KGLM_ECUDA, "tensor-core certificate product setup failed"};
-    a.Qs = c->Qs;
-    a.nqs = pl.njobs;
-    a.qs_stride = (size_t)m * p;
-    for (int t = 0; t < pl.njobs; ++t) a.qs_w[t] = pl.w[t];
+    if (a.DZ == nullptr) exact_digits(c->st, c->zeta, m, n, (size_t)n, x.npad, 1, c->DZ, c->ztau);
+    // the levels in pieces that keep every SM busy (at one node of n = 5000, p = 1000, 28 whole
+    // levels on 68 of them took 120 us, now 40 with its integers zeroed)
+    digit_product(c, m, p, n, kCertDigits, c->bnx, c->mAz, c->mBx, c->Qi, c->pC, c->mC);
+    a.Qi = c->Qi;
+    a.qi_stride = (size_t)m * p;
     a.xsig = c->xsig;
     a.ztau = c->ztau;
-    a.ebound = pl.ebound;
+    a.ebound = x.ebound;
 }
 
 void certify(kglm_ctx* c) {
@@ -544,7 +545,7 @@ void certify(kglm_ctx* c) {
     if (c->cexact && !c->f64) {
         // zeta's digits for the exact-splitting X^T zeta, made by the dual point pass
         a.DZ = c->DZ; a.ztau = c->ztau;
-        a.dz_npad = c->xplan.npad; a.dz_nd = c->xplan.nd; a.dz_beta = c->xplan.beta;
+        a.dz_npad = c->xplan.npad;
     }
     const double ws = c->f64 ? 8.0 : 4.0;
     {
@@ -688,14 +689,14 @@ void iterate(kglm_ctx* c) {
         {
             Scope sc(c, PH_GEMM_LINK, 3, flops);
             split_digits(c->st, (const double*)c->V, m, p, p, q.pk, q.sxt, 0, 1, q.DV, q.tv, nullptr);
-            const SplitPlan& pl = split_product(c, m, false);
-            if (split_link(c->st, m, n, q.nk, q.I, (size_t)m * n, pl, q.tv, q.sx, c->y64, c->kind, q.DR, q.tr) != 0)
+            split_product(c, m, false);
+            if (split_link(c->st, m, n, q.nk, q.I, (size_t)m * n, q.tv, q.sx, c->y64, c->kind, q.DR, q.tr) != 0)
                 throw Fail{KGLM_ECUDA, "FP64 link launch failed"};
             check_launch();
         }
         Scope sc(c, PH_GEMM_GRAD, 2, flops);
-        const SplitPlan& pl = split_product(c, m, true);
-        split_combine(c->st, m, p, q.I, (size_t)m * p, pl, q.tr, q.sxt, (double*)c->G);
+        split_product(c, m, true);
+        split_combine(c->st, m, p, q.I, (size_t)m * p, q.tr, q.sxt, (double*)c->G);
         check_launch();
     } else {
         {
@@ -1248,8 +1249,8 @@ size_t footprint(const kglm_desc& d) {
         add(sizeof(DqState));
     }
     ExactPlan x{};
-    if (!f64 && exact_plan((int)n, 6, 7, &x)) {
-        const size_t K2 = (size_t)x.nd * x.npad;
+    if (!f64 && exact_plan((int)n, &x)) {
+        const size_t K2 = 7 * (size_t)x.npad;
         const size_t need = 2 * K2 * (p + mc) + 8 * (p + mc) + 4 * (size_t)x.njobs * mc * p + 64;
         if (d.hbm_budget <= 0 || (int64_t)(est + need) <= d.hbm_budget) {
             add(2 * p * K2); add(8 * p); add(2 * mc * K2); add(8 * mc); add(4 * (size_t)x.njobs * mc * p);
@@ -2268,23 +2269,25 @@ kglm_status kglm_create(const kglm_desc* desc, const double* X, const double* y,
         }
         // reduced-precision modes: digits of X for the exact certificate product
         // (6-bit digits, 7 per value), when the jobs and the HBM budget allow
-        if (!c->f64 && exact_plan((int)n, 6, 7, &c->xplan)) {
+        if (!c->f64 && exact_plan((int)n, &c->xplan)) {
             const ExactPlan& x = c->xplan;
-            const size_t K2 = (size_t)x.nd * x.npad;
+            // (rows of kCertDigits segments; the buffers keep the size the footprint states)
+            const size_t K2 = 7 * (size_t)x.npad;
+            const int KD = kCertDigits * x.npad;
             const size_t need = 2 * K2 * (p + mc) + 8 * (p + mc) + 4 * (size_t)x.njobs * mc * p + 64;
             if (c->d.hbm_budget <= 0 || (int64_t)(c->bytes + need) <= c->d.hbm_budget) {
                 c->DX = dalloc_t<__nv_bfloat16>(c, p * K2);
                 c->xsig = dalloc_t<double>(c, p);
-                exact_digits(c->st, c->Xt64, (int)p, (int)n, n, x.npad, x.nd, x.beta, 0, c->DX, c->xsig);
+                exact_digits(c->st, c->Xt64, (int)p, (int)n, n, x.npad, 0, c->DX, c->xsig);
                 check_launch();
                 c->DZ = dalloc_t<__nv_bfloat16>(c, mc * K2);
                 CK(cudaMemsetAsync(c->DZ, 0, sizeof(__nv_bfloat16) * mc * K2, c->st));
                 c->ztau = dalloc_t<double>(c, mc);
-                c->qs_slices = (size_t)x.njobs;
-                c->Qs = dalloc_t<float>(c, c->qs_slices * mc * p);
+                c->qi_slices = (size_t)x.njobs;
+                c->Qi = dalloc_t<int>(c, c->qi_slices * mc * p);
                 c->bnx = tc_tile_cols((int)p);
-                if (tc_make_map(&c->mBx, c->DX, 1, (int)p, (int)K2, (int)K2, c->bnx) ||
-                    tc_make_map(&c->mAz, c->DZ, 1, (int)mc, (int)K2, (int)K2, 128))
+                if (tc_make_map(&c->mBx, c->DX, 1, (int)p, KD, KD, c->bnx) ||
+                    tc_make_map(&c->mAz, c->DZ, 1, (int)mc, KD, KD, 128))
                     throw Fail{KGLM_ECUDA, "cuTensorMapEncodeTiled failed for the certificate digits"};
                 if (tc_prepare() != 0) throw Fail{KGLM_ECUDA, "tensor-core kernels: shared memory attribute refused"};
                 if (!c->d_tcerr) {
@@ -2351,8 +2354,8 @@ kglm_status kglm_xtr(kglm_ctx* ctx, int32_t m, const void* R, void* G) {
             CK(cudaMemcpyAsync(&bad, q.flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->st));
             sync(ctx);
             if (!bad) {
-                const SplitPlan& pl = split_product(ctx, m, true);
-                split_combine(ctx->st, m, ctx->p, q.I, (size_t)m * ctx->p, pl, q.tr, q.sxt, (double*)G);
+                split_product(ctx, m, true);
+                split_combine(ctx->st, m, ctx->p, q.I, (size_t)m * ctx->p, q.tr, q.sxt, (double*)G);
                 check_launch();
                 sync(ctx);
                 check_tc_error(ctx);
@@ -2385,9 +2388,8 @@ kglm_status kglm_xtz(kglm_ctx* ctx, int32_t m, const double* Z, double* Q, doubl
             check_launch();
         }
         if (!c->Qerr) c->Qerr = dalloc_t<double>(c, (size_t)c->mcap * c->p);
-        if (a.Qs) {
-            exact_combine(c->st, m, c->p, a.Qs, a.nqs, a.qs_stride, a.qs_w, c->xsig, c->ztau, a.ebound, c->Q,
-                          c->Qerr);
+        if (a.Qi) {
+            exact_combine(c->st, m, c->p, a.Qi, a.qi_stride, c->xsig, c->ztau, a.ebound, c->Q, c->Qerr);
             check_launch();
         } else {
             CK(cudaMemsetAsync(c->Qerr, 0, sizeof(double) * mp, c->st));
@@ -2455,7 +2457,12 @@ kglm_status kglm_read_batch(kglm_ctx* ctx, double* beta, double* zeta) {
                 for (size_t t = 0; t < mp; ++t) beta[t] = h[t];
             }
         }
-        if (zeta) {
+        if (zeta && ctx->cexact) {                     // an FP32 value, kept as one
+            std::vector<float> h(mn);
+            CK(cudaMemcpyAsync(h.data(), ctx->zeta, sizeof(float) * mn, cudaMemcpyDeviceToHost, ctx->st));
+            sync(ctx);
+            for (size_t t = 0; t < mn; ++t) zeta[t] = h[t];
+        } else if (zeta) {
             CK(cudaMemcpyAsync(zeta, ctx->zeta, sizeof(double) * mn, cudaMemcpyDeviceToHost, ctx->st));
             sync(ctx);
         }

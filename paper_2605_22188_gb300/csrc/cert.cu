@@ -74,48 +74,31 @@ __device__ __forceinline__ float dual_z(float s, float yi, int kind) {
     return yi * (t >= 0.f ? e / (1.0f + e) : 1.0f / (1.0f + e));   // y sigma(-t)
 }
 
-// Digits of v = z / 2^e (|v| < 1) as in k_digits of cert_exact.cu, from the FP32
-// value alone: V = rint(v 2^62) by integer shifts of z's significand (nearest,
-// halves away from zero: |V - v 2^62| <= 1/2 as the error bound assumes), then
-// the same signed digits from the top, segment nd - a for digit a (reversed).
-__device__ __forceinline__ void dz_digits(float z, int e, int nd, int beta, __nv_bfloat16* d, size_t npad,
-                                          size_t i) {
-    long long V = 0;
-    const uint32_t u = __float_as_uint(z);
-    const int ex = (int)((u >> 23) & 0xffu);
-    if (ex != 255 && (ex != 0 || (u & 0x7fffffu) != 0)) {       // a non-finite z has no digits
-        const long long mnt = ex ? (long long)((u & 0x7fffffu) | 0x800000u) : (long long)(u & 0x7fffffu);
-        const int sh = (ex ? ex : 1) - 150 + 62 - e;              // z = mnt 2^(ex - 150), v 2^62 = mnt 2^sh
-        long long mag = 0;
-        if (sh >= 0) mag = sh < 63 ? mnt << sh : 0;                // |v| < 1: below 2^62, so sh < 62
-        else if (sh > -26) mag = (mnt + (1ll << (-sh - 1))) >> (-sh);
-        V = (u >> 31) ? -mag : mag;
-    }
-    for (int a = 1; a <= nd; ++a) {
-        const int sh = 62 - beta * a;
-        const long long dg = (V + (1ll << (sh - 1))) >> sh;        // nearest, halves up
-        V -= dg << sh;
-        d[(size_t)(nd - a) * npad + i] = __int2bfloat16_rn((int)dg);
-    }
-}
-
+// A cluster of `parts` CTAs per node where the batch is small (one CTA per node took 28 us
+// at one node of 5000 samples), each with `seg` of its samples: they exchange the
+// largest |zeta| and their sums, which the first adds in order.
 template <int NT>
-__global__ __launch_bounds__(NT) void k_dual_point_f32(CertArgs a) {
+__global__ __launch_bounds__(NT) void k_dual_point_f32(const __grid_constant__ CertArgs a, int parts, int seg) {
     __shared__ double red[2 * (NT / 32)];
     __shared__ float redf[NT / 32];
-    const int b = blockIdx.x;
+    __shared__ struct { double acc[2]; float zmax; } mine;
+    const int b = blockIdx.x / parts, part = blockIdx.x - b * parts;
     const size_t base = (size_t)b * a.n;
+    const int i0 = part * seg, i1 = min(a.n, i0 + seg);
+    const bool digits = a.DZ != nullptr;               // zeta is kept as the FP32 value it is
+    float* zf = reinterpret_cast<float*>(a.zeta);
     FPair sl, sc;
     float zmax = 0.f;
     const float* S = static_cast<const float*>(a.S);
-    for (int i = threadIdx.x; i < a.n; i += NT) {
+    for (int i = i0 + threadIdx.x; i < i1; i += NT) {
         const float s = S[base + i];
         const float yi = a.y32[i];
         const float z = dual_z(s, yi, a.kind);
         zmax = fmaxf(zmax, fabsf(z));
+        if (digits) zf[base + i] = z;
+        else a.zeta[base + i] = (double)z;
         if (a.kind == kLSQ) {
             const float r = s - yi;
-            a.zeta[base + i] = (double)z;
             sl.add(__fmul_rn(r, r));                         // the loss term as the iterations form it
             const float r2 = 2.0f * r;                        // w = -zeta, exact
             sc.add_prod(r2, yi);                              // 2 r y32, exact as a pair
@@ -125,7 +108,6 @@ __global__ __launch_bounds__(NT) void k_dual_point_f32(CertArgs a) {
             const float t = yi * s;
             const float e = __expf(-fabsf(t));
             const float sg = t >= 0.f ? e / (1.0f + e) : 1.0f / (1.0f + e);     // sigma(-t)
-            a.zeta[base + i] = (double)z;
             sl.add(fmaxf(-t, 0.f) + log1pf(e));
             float t1 = 0.f, t2 = 0.f;
             if (sg > 0.f) t1 = sg * logf(sg);
@@ -137,24 +119,50 @@ __global__ __launch_bounds__(NT) void k_dual_point_f32(CertArgs a) {
     }
     double acc[2] = {sl.value(), sc.value()};
     block_sum<NT, 2, double>(acc, red);
-    if (threadIdx.x == 0) {
+    float mx = digits ? block_max<NT, float>(zmax, redf) : 0.f;
+    if (parts > 1) {
+        if (threadIdx.x == 0) {
+            mine.acc[0] = acc[0];
+            mine.acc[1] = acc[1];
+            mine.zmax = mx;
+        }
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        const uint32_t at = (uint32_t)__cvta_generic_to_shared(&mine);
+        acc[0] = acc[1] = 0.0;
+        for (int q = 0; q < parts; ++q) {
+            uint32_t peer;
+            double v0, v1;
+            float z;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(at), "r"(q));
+            asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v0) : "r"(peer) : "memory");
+            asm volatile("ld.shared::cluster.f64 %0, [%1 + 8];" : "=d"(v1) : "r"(peer) : "memory");
+            asm volatile("ld.shared::cluster.f32 %0, [%1 + 16];" : "=f"(z) : "r"(peer) : "memory");
+            acc[0] += v0;
+            acc[1] += v1;
+            mx = fmaxf(mx, z);
+        }
+        // no CTA leaves before its peers have read its values
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+    if (threadIdx.x == 0 && part == 0) {
         a.sum_loss[b] = acc[0];
         a.sum_conj[b] = acc[1];
     }
-    if (a.DZ == nullptr) return;
+    if (!digits) return;
     // the digits of zeta for the exact-splitting X^T zeta: the row's scale from the
-    // first pass, then zeta again (the same FP32 operations) and its digits
-    zmax = warp_max(zmax);
-    if ((threadIdx.x & 31) == 0) redf[threadIdx.x >> 5] = zmax;
-    __syncthreads();
-    float mx = 0.f;
-    for (int w = 0; w < NT / 32; ++w) mx = fmaxf(mx, redf[w]);
-    const int e = mx > 0.f ? ilogbf(mx) + 1 : 0;                   // 2^e > mx
-    if (threadIdx.x == 0) a.ztau[b] = mx > 0.f ? ldexp(1.0, e) : 0.0;   // a zero row is exact
-    __nv_bfloat16* d = a.DZ + (size_t)b * a.dz_nd * a.dz_npad;
-    for (int i = threadIdx.x; i < a.dz_npad; i += NT) {
-        const float z = i < a.n ? dual_z(S[base + i], a.y32[i], a.kind) : 0.f;
-        dz_digits(z, e, a.dz_nd, a.dz_beta, d, (size_t)a.dz_npad, (size_t)i);
+    // first pass, then zeta again (written by this CTA) and its bytes from its FP32 bits
+    const bool scaled = mx > 0.f && mx <= FLT_MAX;                 // (an infinite zeta has an infinite sum_conj)
+    const int e = scaled ? ilogbf(mx) + 2 : 0;                     // 2^e > 2 mx
+    if (threadIdx.x == 0 && part == 0) a.ztau[b] = scaled ? ldexp(1.0, e) : 0.0;   // a zero row is exact
+    __nv_bfloat16* d = a.DZ + (size_t)b * kCertDigits * a.dz_npad;
+    const int iend = part == parts - 1 ? a.dz_npad : min(a.dz_npad, i0 + seg);
+    for (int i = i0 + 4 * threadIdx.x; i < iend; i += 4 * NT) {
+        long long z[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) z[q] = i + q < i1 ? fixed64f<8 * kCertDigits>(zf[base + i + q], e) : 0ll;
+        store_digits<kCertDigits>(z, d, (size_t)a.dz_npad, i, 1);
     }
 }
 
@@ -211,14 +219,7 @@ __global__ __launch_bounds__(NT) void k_cert_bound(const __grid_constant__ CertA
         q[e] = be[e] = 0.0;
         if (j < p) {
             valid |= 1u << e;
-            if (a.Qs) {
-                // |X^T zeta| bounded from above: |Q~| + its distance bound (H_M, TopSum increase in |q|)
-                double err;
-                const double qv = exact_q(a.Qs, a.nqs, a.qs_stride, a.qs_w, base + j, a.xsig[j] * a.ztau[b], a.ebound, &err);
-                q[e] = (fabs(qv) + err) * inv2l;
-            } else {
-                q[e] = a.Q[base + j] * inv2l;
-            }
+            q[e] = a.Q[base + j] * inv2l;
             be[e] = a.b_is_f64 ? static_cast<const double*>(a.B)[base + j]
                                : (double)static_cast<const float*>(a.B)[base + j];
             if ((im[j >> 5] >> (j & 31)) & 1u) fin |= 1u << e;
@@ -346,346 +347,242 @@ __global__ __launch_bounds__(NT) void k_cert_bound(const __grid_constant__ CertA
     for (int i = threadIdx.x; i < a.k; i += NT) a.support[(size_t)b * a.k + i] = i < ns ? sh.sups[i] : -1;
 }
 
-// ---- the same bound, primal, support and branching index with a warp per node,
-// for FP32 beta with X^T zeta as exact-splitting partials (BF16/TF32 modes).
-// The CTA kernel above spends its time in FP64 arithmetic on every coordinate
-// (the slice combine, H_M, the sums) and in the barriers of two block-wide
-// radix selections.  Here FP64 work is confined to the few coordinates whose
-// values are summed:
-// * one pass over the free coordinates combines the slices in FP32 with a
-//   rigorous error bound and keeps in shared memory an upper bound u_j, and in
-//   registers the lane's two largest lower bounds l_j, of the value
-//   v_j = (|q~_j| + err_j) / (2 lambda2) that the FP64 combine gives
-//   (l_j <= v_j <= u_j); the beta sums of Theorem 4.1 run in compensated FP32;
-// * TopSum: the kbar-th largest of the 64 lane samples, t, is at most the
-//   kbar-th largest l, hence at most the kbar-th largest v, so every coordinate
-//   of the top kbar has u_j >= t; those (normally a few more than kbar) get
-//   their exact FP64 v_j (the combine of the CTA kernel) and are ranked; when
-//   more than kCertCap qualify (near-ties), they are streamed through an exact
-//   top-kbar list instead;
-// * top-kbar |beta| over Jf (ties to the smaller index): lane samples of the
-//   beta keys, a gather of the candidates and their ranks; zeros tie-break by
-//   index directly (the smallest free indices with beta = 0).
-constexpr int kCertCap = 128;
-constexpr int kCertMaxWarps = 16;
-
-struct CertWarp {
-    int cand[kCertCap];
-    union {
-        double cval[kCertCap];                 // exact v of the TopSum candidates
-        unsigned long long bkey[kCertCap];     // (|beta| key, ~j) of the beta candidates
-    };
-    double tv[kMaxK];
-    float sv[kMaxK];
+// ---- the same bound, primal, support and branching index for FP32 beta with X^T zeta as
+// the exact-splitting product's integers (the reduced-precision modes): a CTA per
+// node.  FP64 operations are what GB300 has least of (one warp instruction per SM in 16
+// cycles), so an entry takes three of them, v_j = (|q~_j| + err_j) / (2 lambda2) from the
+// correctly rounded integer combine; the selections work on the bits of v and |beta|,
+// the beta sums of Theorem 4.1 are FP32 pairs, and only the at most 64 selected values
+// reach FP64 sums, in the order of their ranks.  8192 nodes of p = 2000: 0.54 ms (1.27 with
+// a warp per node over 30 FP32 slices); one node of p = 1000: 31 us (78).
+struct CertNodeShared {
+    SelectShared sel;
+    double red[2 * 32];
+    float redf[4 * 32];
+    int ired[32];
+    int ncand, nj1;
+    double topv[kMaxK];      // selected v (then |beta|), unordered
+    int topi[kMaxK];
+    double sv[kMaxK];        // sorted, descending
     int si[kMaxK];
+    double vj1[kMaxK];       // v of the J1 coordinates
+    int j1[kMaxK];
     int sup[2 * kMaxK];
-    int ncand, nsup;
 };
-
-__host__ __device__ inline size_t cert_row(int p) { return ((size_t)p + 3) / 4 * 4; }
-__host__ __device__ inline size_t cert_hdr() { return (sizeof(CertWarp) + 15) / 16 * 16; }
-__host__ __device__ inline size_t cert_warp_bytes(int p) { return cert_hdr() + cert_row(p) * sizeof(uint32_t); }
-__host__ __device__ inline size_t cert_cta_bytes(int p, int wpc) {
-    return (kTcMaxJobs + cert_row(p)) * sizeof(float) + wpc * cert_warp_bytes(p);
-}
 
 // compensated FP32 accumulation (Knuth's two-sum; the product error by an FMA)
 __device__ __forceinline__ void acc2(float& hi, float& lo, float x) {
-    const float s = hi + x, bp = s - hi;
-    lo += (hi - (s - bp)) + (x - bp);
+    const float s = __fadd_rn(hi, x), bp = __fsub_rn(s, hi);
+    lo += __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(x, bp));
     hi = s;
 }
 __device__ __forceinline__ void acc2_sq(float& hi, float& lo, float x) {
-    const float pr = x * x;
+    const float pr = __fmul_rn(x, x);
     acc2(hi, lo, pr);
     lo += fmaf(x, x, -pr);
 }
-
-__device__ __forceinline__ double cert_exact_v(const CertArgs& a, size_t base, int j, int b, double inv2l) {
-    double err;
-    const double qv = exact_q(a.Qs, a.nqs, a.qs_stride, a.qs_w, base + j, a.xsig[j] * a.ztau[b], a.ebound, &err);
-    return (fabs(qv) + err) * inv2l;
+// the pairs of a warp's lanes, summed (every lane gets the total)
+__device__ __forceinline__ void warp_acc2(float& hi, float& lo) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float h = __shfl_xor_sync(0xffffffffu, hi, o), l = __shfl_xor_sync(0xffffffffu, lo, o);
+        // the same sum in both lanes: the larger-indexed lane's pair is added to the other's
+        const bool up = (threadIdx.x & o) != 0;
+        float a = up ? h : hi, b = up ? l : lo;
+        const float c = up ? hi : h, d = up ? lo : l;
+        acc2(a, b, c);
+        hi = a;
+        lo = b + d;
+    }
 }
 
-__global__ __launch_bounds__(32 * kCertMaxWarps) void k_cert_bound_warp(const __grid_constant__ CertArgs a) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, wpc = blockDim.x >> 5;
-    const int p = a.p, nq = a.nqs;
-    float* wf = reinterpret_cast<float*>(smem);                 // slice weights (powers of two) in FP32
-    float* xs = wf + kTcMaxJobs;                                // sigma_j in FP32 (shared by the CTA)
-    unsigned char* wb = smem + (kTcMaxJobs + cert_row(p)) * sizeof(float) + (size_t)warp * cert_warp_bytes(p);
-    CertWarp& h = *reinterpret_cast<CertWarp*>(wb);
-    uint32_t* su = reinterpret_cast<uint32_t*>(wb + cert_hdr());
-    for (int j = threadIdx.x; j < p; j += blockDim.x) xs[j] = (float)a.xsig[j];
-    for (int t = threadIdx.x; t < nq; t += blockDim.x) wf[t] = (float)a.qs_w[t];
-    __syncthreads();
-    const double M = a.M, inv2l = 1.0 / (2.0 * a.lam2);
+template <int NT, int E>
+__global__ __launch_bounds__(NT) void k_cert_node(const __grid_constant__ CertArgs a) {
+    using K = unsigned long long;
+    constexpr int NW = NT / 32;
+    __shared__ CertNodeShared sh;
+    const int b = blockIdx.x, p = a.p, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const size_t base = (size_t)b * p;
+    const double M = a.M, inv2l = 1.0 / (2.0 * a.lam2), ztau = a.ztau[b];
     const double mth = M * (1.0 + kFeasRtol);
     const float mth_f = __double2float_rd(mth);                // |b| > mth  <=>  |b| > mth_f for FP32 b
-    const float ebf = (float)a.ebound;
-    const float gam = (float)(nq + 2) * 0x1p-23f;               // |acc_f - acc| <= gam * sum |w P|, with margin
-    const float rlo = 1.0f - 0x1p-19f, rhi = 1.0f + 0x1p-19f;   // covers the FP32 roundings below
-    // node b to CTA b mod grid: the CTAs (and SMs) hold equal shares of the nodes
-    for (int b = warp * gridDim.x + blockIdx.x; b < a.m; b += gridDim.x * wpc) {
-        const size_t base = (size_t)b * p;
-        const uint32_t* im = a.in_mask + (size_t)b * a.W;
-        const uint32_t* om = a.out_mask + (size_t)b * a.W;
-        const int kb = a.kbar[b], pf = a.pf[b];
-        const float* B = static_cast<const float*>(a.B) + base;
-        const float zf = (float)(a.ztau[b] * inv2l);
-        if (lane == 0) { h.ncand = 0; h.nsup = 0; }
-        // ---- pass over the coordinates: u_j to shared memory, lane samples, free beta sums
-        float s1h = 0.f, s1l = 0.f, s2h = 0.f, s2l = 0.f;       // free sum |beta|, sum beta^2
-        int nnz = 0, infeas = 0;
-        uint32_t l1 = 0, l2 = 0, b1 = 0, b2 = 0;                 // two largest l keys, beta keys
-        for (int j = lane; j < p; j += 32) {
-            const uint32_t w = j >> 5, bit = 1u << (j & 31);
-            const bool in = (im[w] & bit) != 0, out = !in && (om[w] & bit) != 0;
-            uint32_t ukey = 0;
-            if (!in && !out) {
-                const float* qp = a.Qs + base + j;
-                float accf = 0.f, absf = 0.f;
-                // all the slices' loads of a coordinate in flight at once (up to 32)
-                for (int t0 = 0; t0 < nq; t0 += 32) {
-                    float v[32];
+    const uint32_t* im = a.in_mask + (size_t)b * a.W;
+    const uint32_t* om = a.out_mask + (size_t)b * a.W;
+    const int kb = a.kbar[b], pf = a.pf[b];
+    const bool leaf = kb == 0 || pf <= kb;
+    if (threadIdx.x == 0) sh.ncand = sh.nj1 = 0;
+    __syncthreads();
+    K key[E];                                                  // bits of v (non-negative)
+    uint32_t bkey[E];                                          // bits of |beta|
+    uint32_t ffree = 0;
+    float s1h = 0.f, s1l = 0.f, s2h = 0.f, s2l = 0.f;          // free sum |beta|, sum beta^2
+    int nnz = 0, infeas = 0;
 #pragma unroll
-                    for (int t = 0; t < 32; ++t) v[t] = (t0 + t < nq) ? __ldg(qp + (size_t)(t0 + t) * a.qs_stride) : 0.f;
-#pragma unroll
-                    for (int t = 0; t < 32; ++t) {
-                        if (t0 + t < nq) {
-                            const float wt = wf[t0 + t];
-                            accf = fmaf(wt, v[t], accf);
-                            absf = fmaf(wt, fabsf(v[t]), absf);
-                        }
-                    }
-                }
-                const float cf = xs[j] * zf, d = gam * absf, aa = fabsf(accf);
-                float vl = cf * ((aa - d) + ebf) * rlo - 4.0f * FLT_MIN;
-                float vu = cf * ((aa + d) + ebf) * rhi + 4.0f * FLT_MIN;
-                vl = fminf(fmaxf(vl, 0.f), 0.5f * FLT_MAX);          // an overflowed l: v is larger still
-                if (!(vu >= 0.f) || !(cf >= FLT_MIN)) {              // NaN, or sigma tau / 2 lambda2 below
-                    vu = INFINITY;                                   // the normal range: no bound, always
-                    vl = 0.f;                                        // a candidate
-                }
-                ukey = __float_as_uint(vu) + 1u;
-                const uint32_t lkey = __float_as_uint(vl) + 1u;
-                if (lkey > l1) { l2 = l1; l1 = lkey; } else if (lkey > l2) { l2 = lkey; }
-                const float bv = B[j], ab = fabsf(bv);
-                acc2(s1h, s1l, ab);
-                acc2_sq(s2h, s2l, ab);
-                nnz += ab > 0.f;
-                infeas += ab > mth_f;
-                const uint32_t bk = __float_as_uint(ab) + 1u;
-                if (bk > b1) { b2 = b1; b1 = bk; } else if (bk > b2) { b2 = bk; }
-            } else if (out) {
-                infeas += B[j] != 0.f;
-            }
-            su[j] = ukey;
+    for (int e = 0; e < E; ++e) {
+        const int j = threadIdx.x + e * NT;
+        key[e] = 0;
+        bkey[e] = 0;
+        if (j >= p) continue;
+        const bool in = (im[j >> 5] >> (j & 31)) & 1u, out = !in && ((om[j >> 5] >> (j & 31)) & 1u);
+        const float ab = fabsf(static_cast<const float*>(a.B)[base + j]);
+        if (out) {
+            infeas += ab != 0.f;
+            continue;
         }
-        const double total = warp_sum((double)s1h + (double)s1l);
-        const double sumsq = warp_sum((double)s2h + (double)s2l);
-        nnz = warp_sum(nnz);
-        // ---- J1: exact v, beta^2 and feasibility (at most k coordinates)
-        for (int w = lane; w < a.W; w += 32) {
-            uint32_t bits = im[w];
-            while (bits) {
-                const int j = 32 * w + __ffs(bits) - 1;
-                bits &= bits - 1;
-                const int c = atomicAdd(&h.nsup, 1);
-                if (kglm_check(c < kMaxK, a.chk, kChkCert) && c < kMaxK) h.sup[c] = j;   // |J1| <= k <= kMaxK when validated
+        double err;
+        const double qv = exact_q(a.Qi, a.qi_stride, base + j, a.xsig[j] * ztau, a.ebound, &err);
+        // |X^T zeta| bounded from above: |Q~| + its distance bound (H_M, TopSum increase in |q|)
+        const double v = (fabs(qv) + err) * inv2l;
+        if (in) {
+            const int c = atomicAdd(&sh.nj1, 1);
+            if (kglm_check(c < kMaxK, a.chk, kChkCert) && c < kMaxK) {
+                sh.j1[c] = j;
+                sh.vj1[c] = v;
             }
+            infeas += ab > mth_f;
+            continue;
+        }
+        ffree |= 1u << e;
+        key[e] = (K)__double_as_longlong(v);
+        bkey[e] = __float_as_uint(ab);
+        acc2(s1h, s1l, ab);
+        acc2_sq(s2h, s2l, ab);
+        nnz += ab > 0.f;
+        infeas += ab > mth_f;
+    }
+    warp_acc2(s1h, s1l);
+    warp_acc2(s2h, s2l);
+    nnz = __reduce_add_sync(0xffffffffu, nnz);
+    infeas = __reduce_add_sync(0xffffffffu, infeas);
+    if (lane == 0) {
+        sh.red[2 * warp] = (double)s1h + (double)s1l;
+        sh.red[2 * warp + 1] = (double)s2h + (double)s2l;
+        sh.redf[2 * warp] = __int_as_float(nnz);
+        sh.redf[2 * warp + 1] = __int_as_float(infeas);
+    }
+    // ---- TopSum_kbar {H_M(v_j)}_{j in Jf}: the selected values in shared memory
+    int ntop = 0;
+    if (!leaf) {
+        K thr;
+        int need;
+        block_kth_largest<NT, E, K>(key, ffree, kb, sh.sel, thr, need);
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if (((ffree >> e) & 1u) && key[e] > thr) {
+                const int c = atomicAdd(&sh.ncand, 1);
+                sh.topv[c] = __longlong_as_double((long long)key[e]);
+                sh.topi[c] = threadIdx.x + e * NT;
+            }
+        __syncthreads();
+        const int gt = sh.ncand;
+        // the remaining kbar - gt equal the threshold
+        for (int c = gt + threadIdx.x; c < kb; c += NT) {
+            sh.topv[c] = __longlong_as_double((long long)thr);
+            sh.topi[c] = p + c;
+        }
+        ntop = kb;
+    } else if (kb > 0) {
+        // every free coordinate fits the budget (pf <= kbar <= kMaxK)
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if ((ffree >> e) & 1u) {
+                const int c = atomicAdd(&sh.ncand, 1);
+                if (kglm_check(c < kMaxK, a.chk, kChkCert) && c < kMaxK) {
+                    sh.topv[c] = __longlong_as_double((long long)key[e]);
+                    sh.topi[c] = threadIdx.x + e * NT;
+                }
+            }
+        __syncthreads();
+        ntop = min(sh.ncand, kMaxK);
+    }
+    __syncthreads();
+    const int n1 = min(sh.nj1, kMaxK);
+    if (warp == 0) {
+        // sums in the order of the ranks (v descending) and of the J1 indices
+        warp_rank_sort_desc<double>(sh.topv, sh.topi, ntop, sh.sv, sh.si);
+        __syncwarp();
+        double part = 0.0, hj1 = 0.0, bj1 = 0.0;
+        for (int i = lane; i < ntop; i += 32) part += huber64(sh.sv[i], M);
+        for (int i = lane; i < n1; i += 32) {
+            int r = 0;
+            for (int q = 0; q < n1; ++q) r += sh.j1[q] < sh.j1[i];
+            sh.sup[r] = i;
         }
         __syncwarp();
-        const int n1 = min(h.nsup, kMaxK);
-        double hj1 = 0.0, bj1 = 0.0;
         for (int i = lane; i < n1; i += 32) {
-            const int j = h.sup[i];
-            hj1 += huber64(cert_exact_v(a, base, j, b, inv2l), M);
-            const double bv = (double)B[j];
+            const int at = sh.sup[i];
+            hj1 += huber64(sh.vj1[at], M);
+            const double bv = (double)static_cast<const float*>(a.B)[base + sh.j1[at]];
             bj1 += bv * bv;
-            infeas += fabs(bv) > mth;
         }
+        part = warp_sum(part);
         hj1 = warp_sum(hj1);
         bj1 = warp_sum(bj1);
-        infeas = warp_sum(infeas);
-        const bool leaf = kb == 0 || pf <= kb;
-        // ---- TopSum_kbar {H_M(v_j)}_{j in Jf}
-        double part = 0.0;
-        if (!leaf) {
-            uint32_t k0 = l1, k1 = l2;
-            sort64(k0, k1, lane);
-            const int pos = 64 - kb;
-            const uint32_t ta = __shfl_sync(0xffffffffu, k0, pos >> 1), tb = __shfl_sync(0xffffffffu, k1, pos >> 1);
-            const uint32_t tau = max((pos & 1) ? tb : ta, 1u);
-            for (int j = lane; j < p; j += 32)
-                if (su[j] >= tau) {
-                    const int c = atomicAdd(&h.ncand, 1);
-                    if (c < kCertCap) h.cand[c] = j;
-                }
-            __syncwarp();
-            const int total_c = h.ncand;
-            if (total_c <= kCertCap) {
-                for (int i = lane; i < total_c; i += 32) h.cval[i] = cert_exact_v(a, base, h.cand[i], b, inv2l);
-                __syncwarp();
-                for (int i = lane; i < total_c; i += 32) {
-                    const double ci = h.cval[i];
-                    int r = 0;
-                    for (int t = 0; t < total_c; ++t) r += h.cval[t] > ci || (h.cval[t] == ci && t < i);
-                    if (r < kb) part += huber64(ci, M);
-                }
-            } else {
-                // near-ties: every qualifying coordinate through an exact top-kbar list (descending)
-                int nt = 0;
-                double vmin = -1.0;
-                for (int j0 = 0; j0 < p; j0 += 32) {
-                    const int j = j0 + lane;
-                    double v = -1.0;
-                    if (j < p && su[j] >= tau) v = cert_exact_v(a, base, j, b, inv2l);
-                    uint32_t bal = __ballot_sync(0xffffffffu, v > vmin);
-                    while (bal) {
-                        const int src = __ffs(bal) - 1;
-                        bal &= bal - 1;
-                        const double x = __shfl_sync(0xffffffffu, v, src);
-                        if (nt == kb && !(x > vmin)) continue;
-                        if (lane == 0) {
-                            int i = nt < kb ? nt : kb - 1;
-                            while (i > 0 && h.tv[i - 1] < x) { h.tv[i] = h.tv[i - 1]; --i; }
-                            h.tv[i] = x;
-                        }
-                        __syncwarp();
-                        nt = min(nt + 1, kb);
-                        vmin = nt == kb ? h.tv[kb - 1] : -1.0;
-                    }
-                }
-                for (int i = lane; i < nt; i += 32) part += huber64(h.tv[i], M);
-            }
-            __syncwarp();
-            if (lane == 0) h.ncand = 0;
-        } else if (kb > 0) {
-            // every free coordinate fits the budget (pf <= kbar <= kMaxK): all join the sum and the support
-            for (int j = lane; j < p; j += 32)
-                if (su[j] != 0u) {
-                    part += huber64(cert_exact_v(a, base, j, b, inv2l), M);
-                    const int c = atomicAdd(&h.nsup, 1);
-                    if (kglm_check(c < 2 * kMaxK, a.chk, kChkCert) && c < 2 * kMaxK) h.sup[c] = j;
-                }
-        }
-        const double topsum = warp_sum(part);
-        const double lb = -a.sum_conj[b] - 2.0 * a.lam2 * (hj1 + topsum);
-        __syncwarp();
-        // ---- top-kbar |beta| over Jf, ties to the smaller index
-        if (!leaf) {
-            uint32_t k0 = b1, k1 = b2;
-            sort64(k0, k1, lane);
-            const int pos = 64 - kb;
-            const uint32_t ta = __shfl_sync(0xffffffffu, k0, pos >> 1), tb = __shfl_sync(0xffffffffu, k1, pos >> 1);
-            const uint32_t tau = max((pos & 1) ? tb : ta, 2u);     // nonzero |beta| only; zeros below
-            for (int j = lane; j < p; j += 32) {
-                if (su[j] == 0u) continue;
-                const uint32_t key = __float_as_uint(fabsf(B[j])) + 1u;
-                if (key >= tau) {
-                    const int c = atomicAdd(&h.ncand, 1);
-                    if (c < kCertCap) h.bkey[c] = ((unsigned long long)key << 32) | (0xffffffffu - (uint32_t)j);
-                }
-            }
-            __syncwarp();
-            const int total_c = h.ncand;
-            int got = 0;
-            if (total_c <= kCertCap) {
-                for (int i = lane; i < total_c; i += 32) {
-                    const unsigned long long ci = h.bkey[i];
-                    int r = 0;
-                    for (int t = 0; t < total_c; ++t) r += h.bkey[t] > ci;
-                    if (r < kb) {
-                        h.sv[r] = __uint_as_float((uint32_t)(ci >> 32) - 1u);
-                        h.si[r] = (int)(0xffffffffu - (uint32_t)ci);
-                    }
-                }
-                got = min(total_c, kb);
-            } else {
-                unsigned long long last = ~0ull;                    // kb rounds of a warp argmax
-                for (int r = 0; r < kb; ++r) {
-                    unsigned long long best = 0ull;
-                    for (int j = lane; j < p; j += 32) {
-                        if (su[j] == 0u) continue;
-                        const uint32_t key = __float_as_uint(fabsf(B[j])) + 1u;
-                        const unsigned long long pk = ((unsigned long long)key << 32) | (0xffffffffu - (uint32_t)j);
-                        if (key >= 2u && pk < last && pk > best) best = pk;
-                    }
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        const unsigned long long x = __shfl_xor_sync(0xffffffffu, best, o);
-                        best = x > best ? x : best;
-                    }
-                    if (best == 0ull) break;
-                    last = best;
-                    if (lane == 0) {
-                        h.sv[r] = __uint_as_float((uint32_t)(best >> 32) - 1u);
-                        h.si[r] = (int)(0xffffffffu - (uint32_t)best);
-                    }
-                    ++got;
-                }
-            }
-            __syncwarp();
-            // fewer than kbar nonzero: the free zeros of smallest index fill the rest
-            for (int j0 = 0; j0 < p && got < kb; j0 += 32) {
-                const int j = j0 + lane;
-                const bool z = j < p && su[j] != 0u && B[j] == 0.f;
-                uint32_t bal = __ballot_sync(0xffffffffu, z);
-                const int before = __popc(bal & ((1u << lane) - 1u));
-                if (z && got + before < kb && kglm_check(got + before < kMaxK, a.chk, kChkCert)) {
-                    h.sv[got + before] = 0.f;
-                    h.si[got + before] = j;
-                }
-                got = min(kb, got + __popc(bal));
-            }
-            __syncwarp();
-            for (int i = lane; i < kb; i += 32) h.sup[n1 + i] = h.si[i];
-            __syncwarp();
-            if (lane == 0) h.nsup = n1 + kb;
-        }
-        __syncwarp();
-        // ---- support ascending (the warp); Theorem 4.1 and the outputs (lane 0)
-        const int ns = min(h.nsup, kMaxK);
-        int srt[2] = {-1, -1};
-        for (int i = lane, t = 0; i < ns && t < 2; i += 32, ++t) {
-            const int v = h.sup[i];
-            int r = 0;
-            for (int q = 0; q < ns; ++q) r += h.sup[q] < v;
-            srt[t] = r;
-        }
-        const int vals[2] = {lane < ns ? h.sup[lane] : -1, lane + 32 < ns ? h.sup[lane + 32] : -1};
-        __syncwarp();
-        for (int t = 0; t < 2; ++t)
-            if (srt[t] >= 0) h.sup[srt[t]] = vals[t];
-        __syncwarp();
-        for (int i = lane; i < a.k; i += 32) a.support[(size_t)b * a.k + i] = i < ns ? h.sup[i] : -1;
         if (lane == 0) {
-            double gf;
-            if (infeas > 0) gf = INFINITY;
-            else if (kb == 0) gf = total > 0.0 ? INFINITY : 0.0;
-            else if (total / M > kb * (1.0 + kFeasRtol)) gf = INFINITY;
-            else if (nnz <= kb) gf = 0.5 * sumsq;
-            else {
-                // s = the smallest index with tau_s >= |beta|_(s+1) (Theorem 4.1), s = kbar - 1
-                // taken also if rounding in total - pre says otherwise
-                double pre = 0.0, presq = 0.0;
-                int s = 0;
-                for (; s < kb - 1; ++s) {
-                    const double v = (double)h.sv[s];
-                    if ((total - pre) / (kb - s) >= v) break;
-                    pre += v;
-                    presq += v * v;
-                }
-                const double tail = total - pre;
-                gf = 0.5 * (presq + tail / (kb - s) * tail);
-            }
-            const double g = 0.5 * bj1 + gf;
-            a.lb[b] = lb;
-            a.primal[b] = isinf(g) ? INFINITY : a.sum_loss[b] + 2.0 * a.lam2 * g;
-            a.jstar[b] = leaf ? -1 : h.si[0];
+            a.lb[b] = -a.sum_conj[b] - 2.0 * a.lam2 * (hj1 + part);
+            sh.vj1[0] = bj1;                                   // (the J1 values are spent)
         }
         __syncwarp();
+        if (lane == 0) sh.ncand = 0;
+    }
+    __syncthreads();
+    // ---- top-kbar |beta| over Jf (ties to the smaller index): rounding, j*, Theorem 4.1
+    if (!leaf) {
+        const uint32_t sel = block_topk_select<NT, E, uint32_t>(bkey, ffree, kb, sh.sel, sh.ired);
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if ((sel >> e) & 1u) {
+                const int c = atomicAdd(&sh.ncand, 1);
+                sh.topv[c] = (double)__uint_as_float(bkey[e]);
+                sh.topi[c] = threadIdx.x + e * NT;
+            }
+        __syncthreads();
+    }
+    if (warp != 0) return;
+    // ---- the first warp: sorted |beta|, the support ascending, Theorem 4.1 and the outputs
+    if (!leaf) {
+        warp_rank_sort_desc<double>(sh.topv, sh.topi, kb, sh.sv, sh.si);
+        __syncwarp();
+    }
+    const int nf = leaf ? ntop : kb, ns = min(n1 + nf, kMaxK);
+    for (int i = lane; i < ns; i += 32) {
+        const int v = i < n1 ? sh.j1[i] : sh.topi[i - n1];
+        int r = 0;
+        for (int q = 0; q < ns; ++q) r += (q < n1 ? sh.j1[q] : sh.topi[q - n1]) < v;
+        sh.sup[r] = v;
+    }
+    __syncwarp();
+    for (int i = lane; i < a.k; i += 32) a.support[(size_t)b * a.k + i] = i < ns ? sh.sup[i] : -1;
+    if (lane == 0) {
+        double total = 0.0, sumsq = 0.0;
+        int nz = 0, bad = 0;
+        for (int w = 0; w < NW; ++w) {
+            total += sh.red[2 * w];
+            sumsq += sh.red[2 * w + 1];
+            nz += __float_as_int(sh.redf[2 * w]);
+            bad += __float_as_int(sh.redf[2 * w + 1]);
+        }
+        double gf;
+        if (bad > 0) gf = INFINITY;
+        else if (kb == 0) gf = total > 0.0 ? INFINITY : 0.0;
+        else if (total / M > kb * (1.0 + kFeasRtol)) gf = INFINITY;
+        else if (nz <= kb) gf = 0.5 * sumsq;
+        else {
+            // s = the smallest index with tau_s >= |beta|_(s+1) (Theorem 4.1), s = kbar - 1
+            // taken also if rounding in total - pre says otherwise
+            double pre = 0.0, presq = 0.0;
+            int s = 0;
+            for (; s < kb - 1; ++s) {
+                if ((total - pre) / (kb - s) >= sh.sv[s]) break;
+                pre += sh.sv[s];
+                presq += sh.sv[s] * sh.sv[s];
+            }
+            const double tail = total - pre;
+            gf = 0.5 * (presq + tail / (kb - s) * tail);
+        }
+        const double g = 0.5 * sh.vj1[0] + gf;
+        a.primal[b] = isinf(g) ? INFINITY : a.sum_loss[b] + 2.0 * a.lam2 * g;
+        a.jstar[b] = leaf ? -1 : sh.si[0];
     }
 }
 
@@ -694,37 +591,39 @@ __global__ __launch_bounds__(32 * kCertMaxWarps) void k_cert_bound_warp(const __
 void cert_dual_point(cudaStream_t s, const CertArgs& a) {
     if (a.m <= 0) return;
     if (a.s_is_f64) k_dual_point<256><<<a.m, 256, 0, s>>>(a);
-    else k_dual_point_f32<256><<<a.m, 256, 0, s>>>(a);
-}
-
-// The warp kernel's FP32 combine needs weights that are powers of two (products
-// with the FP32 slices exact) within FP32's normal range.
-static bool cert_warp_ok(const CertArgs& a) {
-    if (a.nqs < 1 || a.nqs > kTcMaxJobs) return false;
-    for (int t = 0; t < a.nqs; ++t) {
-        int e = 0;
-        if (frexp(a.qs_w[t], &e) != 0.5 || e < -90 || e > 40) return false;
+    else {
+        int parts = 1;
+        while (parts < 8 && (long)a.m * parts < 2 * 152 && a.n / parts >= 1024) parts *= 2;
+        const int seg = ((a.n + parts - 1) / parts + 3) / 4 * 4;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)a.m * parts);
+        cfg.blockDim = dim3(256);
+        cfg.stream = s;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = parts;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = parts > 1 ? 1 : 0;
+        cudaLaunchKernelEx(&cfg, k_dual_point_f32<256>, a, parts, seg);   // errors surface at the caller's check
     }
-    return true;
 }
 
 int cert_bound(cudaStream_t s, const CertArgs& a) {
     const int p = a.p, m = a.m;
     if (m <= 0) return 0;
-    if (!a.b_is_f64 && a.Qs && p > 512 && p <= 16384 && cert_warp_ok(a)) {
-        // a warp per node (as many as fit in shared memory, at most 16 per CTA)
-        static const int opted = [] {
-            return cudaFuncSetAttribute(k_cert_bound_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) ==
-                   cudaSuccess;
-        }();
-        int wpc = kCertMaxWarps;
-        while (wpc > 1 && cert_cta_bytes(p, wpc) > (227u << 10)) --wpc;
-        if (opted && cert_cta_bytes(p, wpc) <= (227u << 10)) {
-            const int per_sm = std::max(1, (int)((228u << 10) / (cert_cta_bytes(p, wpc) + 1024)));
-            const int grid = std::max(1, std::min(152 * per_sm, m));
-            k_cert_bound_warp<<<grid, 32 * wpc, cert_cta_bytes(p, wpc), s>>>(a);
-            return 0;
-        }
+    if (a.Qi) {
+#define KGLM_CERT(NT_, E_) k_cert_node<NT_, E_><<<m, NT_, 0, s>>>(a)
+        if (p <= 128) KGLM_CERT(64, 2);
+        else if (p <= 512) KGLM_CERT(128, 4);
+        else if (p <= 1024) KGLM_CERT(256, 4);
+        else if (p <= 2048) KGLM_CERT(256, 8);
+        else if (p <= 4096) KGLM_CERT(512, 8);
+        else if (p <= 8192) KGLM_CERT(512, 16);
+        else return -1;
+#undef KGLM_CERT
+        return 0;
     }
 #define KGLM_CERT(NT_, E_) k_cert_bound<NT_, E_><<<m, NT_, 0, s>>>(a)
     if (p <= 64) KGLM_CERT(32, 2);

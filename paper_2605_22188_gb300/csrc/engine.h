@@ -111,52 +111,47 @@ struct TcJob {
 // out slice jobs[z].slice (at pout + slice * pstride, row stride pld) =
 // A[:, K range of job z] . B[:, K range of job z]^T for every job, in one launch.
 // pair_on: as CTA pairs (256-row tiles) where the B map has a half box.
-// chunk > 0 (even): the products are of integers and pout holds 32-bit integers; the
-// sums over every chunk of that many K slices are exact in FP32 (at most 2^24) and
-// are added up as integers (a job's whole sum stays below 2^31).
+// The products are of integer digits and pout holds 32-bit integers: the sums over every
+// chunk (even) of that many K slices are exact in FP32 (at most 2^24) and are added up as
+// integers (a job's whole sum stays below 2^31).  add: several jobs share a slice, whose
+// integers (zeroed before) their sums are added to.
 int tc_gemm_jobs(cudaStream_t s, const TcMap& A, const TcMap& B, int M, int N, int bn, const TcJob* jobs,
-                 int njobs, float* pout, size_t pstride, int pld, int* err, int pair_on, int chunk = 0, int pdl = 0);
-// Exact-splitting certificate product (cert_exact.cu): jobs of the level
-// products, their weights 2^(-beta l) and the bound n E per unit sigma tau.
-struct ExactPlan {
-    int beta, nd, npad, kbs;     // digit bits, digits per value, K padded to 64, 64-wide K slices per digit
-    int njobs;
-    TcJob jobs[kTcMaxJobs];
-    double w[kTcMaxJobs];
-    double ebound;
-};
-// Jobs whose FP32 accumulations are exact; false if they do not fit kTcMaxJobs.
-bool exact_plan(int n, int beta, int nd, ExactPlan* pl);
-// Halves jobs while fewer than two waves of CTAs would run (tiles per job) and
-// the slices fit max_slices.
-void exact_plan_widen(ExactPlan* pl, int tiles, size_t max_slices);
-// Digits of the rows of V (rows x n, row stride ldv) into D (rows x nd*npad BF16)
-// and the row scales 2^e > max |V_r|.
-void exact_digits(cudaStream_t s, const double* V, int rows, int n, size_t ldv, int npad, int nd, int beta,
-                  int reversed, __nv_bfloat16* D, double* scale);
-// Q (m x p) and its entrywise bound E (nullable) from the job partials; w: the
-// jobs' weights (host array of nq values).
-void exact_combine(cudaStream_t s, int m, int p, const float* Qs, int nq, size_t stride, const double* w,
-                   const double* sigma, const double* tau, double ebound, double* Q, double* E);
-// FP64 products as BF16 digit products (split64.cu): the jobs of the levels 2 .. 9
-// (digit pairs a + c = level), largest first.
+                 int njobs, int* pout, size_t pstride, int pld, int* err, int pair_on, int chunk, int add);
+// Products of signed-byte digits (split64.cu, cert_exact.cu): the jobs of the levels
+// 2 .. nd + 1 (digit pairs a + c = level), largest first; the integers of level l in slice l - 2.
 constexpr int kSplitChunk = 16;    // K slices of 64 whose digit products sum to at most 2^24
 struct SplitPlan {
-    int kbs, njobs;                // K slices per digit
+    int nd, kbs, njobs;            // digits, K slices per digit, jobs (more than nd: levels in pieces)
     TcJob jobs[kTcMaxJobs];
-    int level[kTcMaxJobs];
 };
-// Jobs for an M x N output over K with column tiles of bn, such that jobs M N <= max_ints; false if none fit.
-bool split_plan(int M, int N, int K, int bn, bool pair, size_t max_ints, SplitPlan* out);
+// Exact-splitting certificate product (cert_exact.cu): kCertDigits signed bytes of every
+// value, levels 2 .. kCertDigits + 1.
+constexpr int kCertDigits = 6;
+struct ExactPlan {
+    int npad;                      // K padded to 64
+    int njobs;                     // integer slices of max_batch x p the context holds
+    double ebound;                 // bound n E per unit sigma tau
+};
+// Sizes and bound; false if n is too large for the product's jobs.
+bool exact_plan(int n, ExactPlan* pl);
+// Digits of the rows of V (rows x n, row stride ldv) into D (rows x kCertDigits npad BF16)
+// and the row scales 2^e > 2 max |V_r| (0 for a zero row).
+void exact_digits(cudaStream_t s, const double* V, int rows, int n, size_t ldv, int npad, int reversed,
+                  __nv_bfloat16* D, double* scale);
+// Q (m x p) and its entrywise bound E (nullable) from the levels' integers.
+void exact_combine(cudaStream_t s, int m, int p, const int* Qi, size_t stride, const double* sigma,
+                   const double* tau, double ebound, double* Q, double* E);
+// Jobs for an M x N output over K of nd digits with column tiles of bn; false if they are too many.
+bool split_plan(int M, int N, int K, int nd, int bn, bool pair, SplitPlan* out);
 // Eight digits of every row of V (entry j times 2^ce[j], or 2^-ce[j] with inv) and the row scales' exponents.
 void split_digits(cudaStream_t s, const double* V, int rows, int n, size_t ldv, int npad, const int* ce, int inv,
                   int reversed, __nv_bfloat16* D, int* scale, int* flag);
-// out (rows x cols) from the jobs' integers (slice t at I + t stride) and the scales' exponents.
-void split_combine(cudaStream_t s, int rows, int cols, const int* I, size_t stride, const SplitPlan& pl,
-                   const int* er, const int* ec, double* out);
-// R = dl(S, y) from the jobs' integers of S = X V, as reversed digits with row exponents er.
-int split_link(cudaStream_t s, int m, int n, int npad, const int* I, size_t stride, const SplitPlan& pl, const int* ev,
-               const int* ex, const double* y, int kind, __nv_bfloat16* D, int* er);
+// out (rows x cols) from the levels' integers (slice t at I + t stride) and the scales' exponents.
+void split_combine(cudaStream_t s, int rows, int cols, const int* I, size_t stride, const int* er, const int* ec,
+                   double* out);
+// R = dl(S, y) from the levels' integers of S = X V, as reversed digits with row exponents er.
+int split_link(cudaStream_t s, int m, int n, int npad, const int* I, size_t stride, const int* ev, const int* ex,
+               const double* y, int kind, __nv_bfloat16* D, int* er);
 int split_prepare();
 int tc_gemm(cudaStream_t s, const TcMap& A, const TcMap& B, const TcMap* B2, const TcGemm& g,
             const GemmScratch* scr);
@@ -239,12 +234,12 @@ struct CertArgs {
     const double* y;
     const float* y32;     // reduced-precision modes: y as FP32 high part y32 = fl(y) and low
     const float* ylo;     // part ylo = fl(y - y32), for the compensated least-squares sums
-    double* zeta;         // out: m x n FP64 dual points
+    double* zeta;         // out: m x n FP64 dual points; FP32 with the digits below (zeta is an FP32 value there)
     // reduced-precision modes with the exact-splitting certificate: the dual point
     // pass also writes zeta's digits (the layout of exact_digits, reversed) and
-    // its row scales 2^e > max |zeta_b| (DZ NULL: not done there)
+    // its row scales 2^e > 2 max |zeta_b| (DZ NULL: not done there)
     __nv_bfloat16* DZ;
-    int dz_npad, dz_nd, dz_beta;
+    int dz_npad;
     double* sum_loss;     // out: m
     double* sum_conj;     // out: m
     const double* Q;      // X^T zeta (m x p) FP64
@@ -258,12 +253,10 @@ struct CertArgs {
     double* primal;       // out
     int* support;         // out m x k
     int* jstar;           // out
-    // reduced-precision modes: X^T zeta from the exact-splitting partials
-    // (Qs != NULL) with the entrywise bound xsig_j ztau_b ebound, instead of Q
-    const float* Qs;
-    int nqs;
-    size_t qs_stride;
-    double qs_w[kTcMaxJobs];
+    // reduced-precision modes: X^T zeta from the exact-splitting jobs' integers
+    // (Qi != NULL) with the entrywise bound xsig_j ztau_b ebound, instead of Q
+    const int* Qi;
+    size_t qi_stride;
     const double* xsig;
     double* ztau;
     double ebound;

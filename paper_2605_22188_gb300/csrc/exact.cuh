@@ -1,21 +1,24 @@
-// Shared by the certificate kernels: the layout of the exact-splitting product
-// of X^T zeta (the digit slices and the per-job partial products) and the
-// FP64 combine of one entry with its error bound.
+// Shared by the certificate kernels: one entry of X^T zeta from the exact-splitting
+// product's integers, with its error bound.
 #pragma once
 
 #include "engine.h"
+#include "fixed.cuh"
 
 namespace kglm {
 
-// Entry (b, j) of X^T zeta from the job partials P_t (slice t at Qs + t * stride,
-// row b at b * p): tau_b sigma_j sum_t w_t P_t[b][j], summed in job order.  err:
-// tau_b sigma_j n E, a bound on the distance to the exact product.
-__device__ __forceinline__ double exact_q(const float* Qs, int nq, size_t stride, const double* w, size_t idx,
-                                          double scale, double ebound, double* err) {
-    double acc = 0.0;
-    for (int t = 0; t < nq; ++t) acc += w[t] * (double)__ldg(Qs + (size_t)t * stride + idx);
+// Entry (b, j) of X^T zeta from the levels' integers (slice t at Qi + t * stride, entry
+// idx = b p + j): tau_b sigma_j (2^-40 H + 2^-72 L), correctly rounded.  scale: sigma_j tau_b, a
+// power of two (0 for a zero row, whose product is exactly 0).  err: scale n E, a bound on
+// the distance to the exact product.
+__device__ __forceinline__ double exact_q(const int* Qi, size_t stride, size_t idx, double scale, double ebound,
+                                          double* err) {
+    long long H, L;
+    level_sums<kCertDigits>(Qi, stride, idx, H, L);
     *err = scale * ebound;
-    return acc * scale;
+    const int ex = (int)((f64_bits(scale) >> 52) & 0x7ff);
+    if (ex == 0 || ex == 2047) return scale == 0.0 ? 0.0 : combine_f64(H, L, -72) * scale;
+    return combine_f64(H, L, ex - 1023 - 72);
 }
 
 }  // namespace kglm

@@ -78,17 +78,80 @@ __host__ __device__ __forceinline__ int exp_key(double v) {
 // 2^e > 2 |v| for the largest key (plus column shift) of a row; a zero row takes e = 0.
 __host__ __device__ __forceinline__ int row_exp(int key) { return key >= kBadRow / 2 ? kBadRow : key > 0 ? key - 1021 : 0; }
 
-// rint(v 2^(64 - e)) for |v| < 2^(e - 1) (halves away from zero).
+// rint(v 2^(BITS - e)) for |v| < 2^(e - 1) (halves away from zero).
+template <int BITS = 64>
 __host__ __device__ __forceinline__ int64_t fixed64(double v, int e) {
     const uint64_t u = f64_bits(v);
     const int ex = (int)(u >> 52) & 0x7ff;
     const uint64_t m = (u & 0xfffffffffffffull) | (ex ? 0x10000000000000ull : 0ull);
-    const int sh = (ex ? ex : 1) - 1011 - e;            // <= 10
+    const int sh = (ex ? ex : 1) - 1075 + BITS - e;     // at most BITS - 54
     uint64_t z;
     if (sh >= 0) z = m << (sh & 63);
     else if (sh > -54) z = (m + (1ull << ((-sh - 1) & 63))) >> (-sh & 63);
     else z = 0;
     return (int64_t)u < 0 ? -(int64_t)z : (int64_t)z;
+}
+
+// The same for an FP32 value (0 for a non-finite one), |v| < 2^(e - 1).
+template <int BITS>
+__device__ __forceinline__ int64_t fixed64f(float v, int e) {
+    const uint32_t u = __float_as_uint(v);
+    const int ex = (int)(u >> 23) & 0xff;
+    const uint64_t m = (u & 0x7fffffu) | (ex ? 0x800000u : 0u);
+    const int sh = (ex ? ex : 1) - 150 + BITS - e;
+    uint64_t z = 0;
+    if (ex != 255) {
+        if (sh >= 0) z = m << (sh & 63);
+        else if (sh > -26) z = (m + (1ull << ((-sh - 1) & 63))) >> (-sh & 63);
+    }
+    return (int32_t)u < 0 ? -(int64_t)z : (int64_t)z;
+}
+
+// The ND signed bytes of z, the last the lowest (|z| < 2^(8 ND - 1)), as BF16: exact.
+template <int ND>
+__device__ __forceinline__ void cut_digits(long long z, __nv_bfloat16 (&d)[ND]) {
+#pragma unroll
+    for (int a = ND - 1; a >= 1; --a) {
+        const int v = (int)(signed char)z;
+        z = (z - v) >> 8;
+        d[a] = __int2bfloat16_rn(v);
+    }
+    d[0] = __int2bfloat16_rn((int)z);
+}
+
+// Digits of four consecutive entries i .. i + 3 (a multiple of 4) of a row into its ND
+// segments of npad, in order or reversed.
+template <int ND>
+__device__ __forceinline__ void store_digits(const long long (&z)[4], __nv_bfloat16* row, size_t npad, int i, int reversed) {
+    __nv_bfloat16 d[4][ND];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) cut_digits<ND>(z[t], d[t]);
+#pragma unroll
+    for (int a = 0; a < ND; ++a) {
+        __nv_bfloat162 lo, hi;
+        lo.x = d[0][a]; lo.y = d[1][a];
+        hi.x = d[2][a]; hi.y = d[3][a];
+        uint2 w;
+        w.x = *reinterpret_cast<const uint32_t*>(&lo);
+        w.y = *reinterpret_cast<const uint32_t*>(&hi);
+        *reinterpret_cast<uint2*>(row + (size_t)(reversed ? ND - 1 - a : a) * npad + i) = w;
+    }
+}
+
+// H and L of one entry of a product of ND digits from its levels' integers (level l in
+// slice l - 2): 2^-40 H + 2^-72 L, levels 2 .. 5 in H.
+template <int ND>
+__device__ __forceinline__ void level_sums(const int* __restrict__ I, size_t stride, size_t idx, long long& H,
+                                           long long& L) {
+    int v[ND];
+#pragma unroll
+    for (int t = 0; t < ND; ++t) v[t] = __ldg(I + (size_t)t * stride + idx);
+    H = L = 0;
+#pragma unroll
+    for (int t = 0; t < ND; ++t) {
+        if (t < 4) H += (long long)v[t] << (8 * (3 - t));
+        else L += (long long)v[t] << (8 * (7 - t));
+    }
 }
 
 // (2^32 H + L) 2^x, correctly rounded.

@@ -125,6 +125,7 @@ struct TcArgs {
     int* counters;
     int* err;
     int chunk;                // integer products: K slices per accumulator, whose sums are then exact
+    int add;                  // and whether the jobs' sums are added to zeroed slices
     int njobs;                // > 0: K range z is job z (its own K offsets in A and B, and slice)
     TcJob jobs[kTcMaxJobs];
 };
@@ -705,12 +706,25 @@ __device__ __forceinline__ void tc_body(const TcArgs& a, const S& src) {
 #pragma unroll
                 for (int q = 0; q < MAXBN / 32; ++q) {
                     const int c = 16 * h + 32 * q;
-                    if (c < a.bn) {
+                    if (c < a.bn && rbase < pq.M) {
 #pragma unroll
                         for (int j = 0; j < 16; j += 4)
                             *reinterpret_cast<int4*>(ti + lane * TPAD + j) =
                                 make_int4(sum[q][j], sum[q][j + 1], sum[q][j + 2], sum[q][j + 3]);
                         __syncwarp();
+                        if (a.add) {
+                            // several jobs of one level: added to its (zeroed) slice, two rows of
+                            // 16 columns per instruction; integer sums have no order
+                            const int col = n0 + c + (lane & 15);
+                            if (col < pq.N)
+#pragma unroll 4
+                                for (int i = 0; i < 16; ++i) {
+                                    const int r = 2 * i + (lane >> 4), row = rbase + r;
+                                    if (row < pq.M) atomicAdd(o + (size_t)row * ld + col, ti[r * TPAD + (lane & 15)]);
+                                }
+                            __syncwarp();
+                            continue;
+                        }
                         const int c0 = n0 + c + 4 * qq;
                         const bool vec = (ld % 4) == 0 && (reinterpret_cast<uintptr_t>(o) % 16) == 0 && c0 + 4 <= pq.N;
 #pragma unroll
@@ -1307,11 +1321,11 @@ int tc_gemm_group(cudaStream_t s, const TcGroupItem* items, int np, int bn, int 
 }
 
 int tc_gemm_jobs(cudaStream_t s, const TcMap& A, const TcMap& B, int M, int N, int bn, const TcJob* jobs,
-                 int njobs, float* pout, size_t pstride, int pld, int* err, int pair_on, int chunk, int pdl) {
+                 int njobs, int* pout, size_t pstride, int pld, int* err, int pair_on, int chunk, int add) {
     if (M <= 0 || N <= 0 || njobs <= 0) return 0;
     if (bn < 16 || bn > MAXBN || bn % 16 != 0 || njobs > kTcMaxJobs) return -4;
-    if (chunk < 0 || chunk % 2 != 0) return -4;
-    if (chunk ? (set_smem_attr<0, 1, 1, 1, true>() | set_smem_attr<0, 1, 1, 2, true>()) : set_smem_attr<0, 1, 1>()) return -5;
+    if (chunk <= 0 || chunk % 2 != 0) return -4;
+    if (set_smem_attr<0, 1, 1, 1, true>() | set_smem_attr<0, 1, 1, 2, true>()) return -5;
     TcArgs a{};
     a.M = M; a.N = N; a.bn = bn;
     a.mt = (M + BM - 1) / BM;
@@ -1322,10 +1336,11 @@ int tc_gemm_jobs(cudaStream_t s, const TcMap& A, const TcMap& B, int M, int N, i
     a.epi = TC_EPI_PARTIAL;
     a.stages = ring_stages(1, 1, bn);
     a.ks = 1;
-    a.pout = pout; a.pstride = pstride; a.pld = pld;
+    a.pout = reinterpret_cast<float*>(pout); a.pstride = pstride; a.pld = pld;   // 32-bit words
     a.err = err;
     a.njobs = njobs;
     a.chunk = chunk;
+    a.add = add;
     for (int j = 0; j < njobs; ++j) a.jobs[j] = jobs[j];
     const CUtensorMap& ma = *reinterpret_cast<const CUtensorMap*>(A.bytes);
     const CUtensorMap& mb = *reinterpret_cast<const CUtensorMap*>(B.bytes);
@@ -1334,17 +1349,12 @@ int tc_gemm_jobs(cudaStream_t s, const TcMap& A, const TcMap& B, int M, int N, i
     cudaLaunchConfig_t cfg{};
     cfg.blockDim = dim3(NT);
     cfg.stream = s;
-    cudaLaunchAttribute attr[2];
+    cudaLaunchAttribute attr[1];
     cfg.attrs = attr;
-    if (pdl) {
-        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
-    }
     if (!pair) {
         cfg.gridDim = dim3(grid_of(a.mt * a.nt * njobs));
         cfg.dynamicSmemBytes = smem_for(1, 1, bn);
-        return (chunk ? cudaLaunchKernelEx(&cfg, k_tc_gemm<0, 1, 1, 1, true>, ma, mb, mb, ma, a)
-                      : cudaLaunchKernelEx(&cfg, k_tc_gemm<0, 1, 1, 1>, ma, mb, mb, ma, a)) == cudaSuccess ? 0 : -7;
+        return cudaLaunchKernelEx(&cfg, k_tc_gemm<0, 1, 1, 1, true>, ma, mb, mb, ma, a) == cudaSuccess ? 0 : -7;
     }
     a.ks = 2;
     const size_t sl = stage_stride(1, 1, bn / 2);
@@ -1357,8 +1367,7 @@ int tc_gemm_jobs(cudaStream_t s, const TcMap& A, const TcMap& B, int M, int N, i
     attr[cfg.numAttrs].val.clusterDim.y = 1;
     attr[cfg.numAttrs++].val.clusterDim.z = 1;
     const CUtensorMap& mbh = *reinterpret_cast<const CUtensorMap*>(B.half);
-    return (chunk ? cudaLaunchKernelEx(&cfg, k_tc_gemm<0, 1, 1, 2, true>, ma, mbh, mbh, ma, a)
-                  : cudaLaunchKernelEx(&cfg, k_tc_gemm<0, 1, 1, 2>, ma, mbh, mbh, ma, a)) == cudaSuccess ? 0 : -7;
+    return cudaLaunchKernelEx(&cfg, k_tc_gemm<0, 1, 1, 2, true>, ma, mbh, mbh, ma, a) == cudaSuccess ? 0 : -7;
 }
 
 }  // namespace kglm

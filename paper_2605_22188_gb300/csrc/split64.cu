@@ -16,8 +16,8 @@
 // against a window of the other).  Sums of digit products over 16 slices of 64 are
 // integers of at most 16 * 64 * 2^14 = 2^24, exact in the tensor core's FP32
 // accumulator; the product's epilogue adds such chunks up in 32-bit integers
-// (gemm_tc.cu, INT), and the kernels here add the jobs of a level and the levels
-// 2 .. 9 in 64-bit integers:
+// (gemm_tc.cu, INT; the pieces of a level that are taken by several SMs are added in
+// global memory), and the kernels here add the levels 2 .. 9 in 64-bit integers:
 //   H = sum_{l <= 5} 2^(8 (5 - l)) I_l,  L = sum_{l >= 6} 2^(8 (9 - l)) I_l,
 //   C = 2^(ea + eb) (2^-40 H + 2^-72 L),
 // |H| < 2^38 K (1 + 2^-6), |L| < 2^41 K (1 + 2^-6): no overflow for K < 2^21.
@@ -41,34 +41,6 @@
 
 namespace kglm {
 namespace {
-
-// The eight digits of z (the last is the lowest byte), as BF16.
-__device__ __forceinline__ void cut(long long z, __nv_bfloat16 (&d)[8]) {
-#pragma unroll
-    for (int a = 7; a >= 1; --a) {
-        const int v = (int)(signed char)z;
-        z = (z - v) >> 8;
-        d[a] = __int2bfloat16_rn(v);
-    }
-    d[0] = __int2bfloat16_rn((int)z);
-}
-
-// Digits of four consecutive entries i .. i + 3 of a row into its eight segments.
-__device__ __forceinline__ void store_digits(const long long (&z)[4], __nv_bfloat16* row, size_t npad, int i, int reversed) {
-    __nv_bfloat16 d[4][8];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) cut(z[t], d[t]);
-#pragma unroll
-    for (int a = 0; a < 8; ++a) {
-        __nv_bfloat162 lo, hi;
-        lo.x = d[0][a]; lo.y = d[1][a];
-        hi.x = d[2][a]; hi.y = d[3][a];
-        uint2 w;
-        w.x = *reinterpret_cast<const uint32_t*>(&lo);
-        w.y = *reinterpret_cast<const uint32_t*>(&hi);
-        *reinterpret_cast<uint2*>(row + (size_t)(reversed ? 7 - a : a) * npad + i) = w;
-    }
-}
 
 // Rows of V (rows x n, stride ldv; entry j times 2^ce[j], or 2^-ce[j] with inv) into
 // digit rows of D (8 npad entries each, zero past n; NULL: none) and their scales'
@@ -130,45 +102,28 @@ __global__ __launch_bounds__(256) void k_split_digits(const double* __restrict__
         long long z[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) z[q] = (i + q < n && e != kBadRow) ? fixed64(v[i + q], e - shift(i + q)) : 0ll;
-        store_digits(z, d, (size_t)npad, i, reversed);
+        store_digits<8>(z, d, (size_t)npad, i, reversed);
     }
 }
 
-struct Levels {
-    int n;
-    signed char hi[kTcMaxJobs];      // 1: the job's level is at most 5
-    signed char sh[kTcMaxJobs];      // its shift within its half
-};
-
-// One entry of the product from its jobs' integers, times 2^x (x: the sum of the scales'
+// One entry of the product from its levels' integers, times 2^x (x: the sum of the scales'
 // exponents; kBadRow makes it a NaN).
-__device__ __forceinline__ double combine(const int* __restrict__ I, size_t stride, size_t idx, const Levels& lv, int x) {
-    long long H = 0, L = 0;
-    for (int t0 = 0; t0 < lv.n; t0 += 8) {                   // eight jobs' loads in flight
-        int v[8];
-#pragma unroll
-        for (int t = 0; t < 8; ++t) v[t] = t0 + t < lv.n ? __ldg(I + (size_t)(t0 + t) * stride + idx) : 0;
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-            if (t0 + t < lv.n) {
-                const long long w = (long long)v[t] << lv.sh[t0 + t];
-                if (lv.hi[t0 + t]) H += w; else L += w;
-            }
-        }
-    }
+__device__ __forceinline__ double combine(const int* __restrict__ I, size_t stride, size_t idx, int x) {
+    long long H, L;
+    level_sums<8>(I, stride, idx, H, L);
     if (x >= kBadRow / 2) return bits_f64(0x7ff8000000000000ull);
     return combine_f64(H, L, x - 72);
 }
 
 // out[b][j] of a rows x cols product of digits (scales 2^er[b], 2^ec[j]).
 __global__ __launch_bounds__(256) void k_split_combine(int cols, const int* __restrict__ I, size_t stride,
-                                                       const __grid_constant__ Levels lv, const int* __restrict__ er,
-                                                       const int* __restrict__ ec, double* __restrict__ out) {
+                                                       const int* __restrict__ er, const int* __restrict__ ec,
+                                                       double* __restrict__ out) {
     const int b = blockIdx.y;
     const int s = er[b];
     const size_t base = (size_t)b * cols;
     for (int j = blockIdx.x * 256 + threadIdx.x; j < cols; j += gridDim.x * 256)
-        out[base + j] = combine(I, stride, base + j, lv, s + ec[j]);
+        out[base + j] = combine(I, stride, base + j, s + ec[j]);
 }
 
 // S = X V of a node, its loss derivative R and R's digits: a cluster of CTAs per node,
@@ -180,8 +135,7 @@ __global__ __launch_bounds__(256) void k_split_combine(int cols, const int* __re
 // took about 220 us, now 65.
 constexpr int kLinkNT = 256;
 __global__ __launch_bounds__(kLinkNT) void k_split_link(int n, int npad, int parts, int seg, const int* __restrict__ I,
-                                                        size_t stride, const __grid_constant__ Levels lv,
-                                                        const int* __restrict__ ev, const int* __restrict__ ex,
+                                                        size_t stride, const int* __restrict__ ev, const int* __restrict__ ex,
                                                         const double* __restrict__ y, int kind,
                                                         __nv_bfloat16* __restrict__ D, int* __restrict__ er) {
     extern __shared__ __align__(16) double row[];
@@ -197,7 +151,7 @@ __global__ __launch_bounds__(kLinkNT) void k_split_link(int n, int npad, int par
     const int s = ev[b];
     int key = 0;
     for (int i = i0 + t; i < i1; i += kLinkNT) {
-        const double r = dloss_fixed(combine(I, stride, base + i, lv, s + ex[i]), y[i], kind, tab);
+        const double r = dloss_fixed(combine(I, stride, base + i, s + ex[i]), y[i], kind, tab);
         row[i - i0] = r;
         key = max(key, exp_key(r));
     }
@@ -226,66 +180,48 @@ __global__ __launch_bounds__(kLinkNT) void k_split_link(int n, int npad, int par
         long long z[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) z[q] = (i + q < i1 && e != kBadRow) ? fixed64(row[i + q - i0], e) : 0ll;
-        store_digits(z, d, (size_t)npad, i, 1);
+        store_digits<8>(z, d, (size_t)npad, i, 1);
     }
-}
-
-Levels levels_of(const SplitPlan& pl) {
-    Levels lv{};
-    lv.n = pl.njobs;
-    for (int t = 0; t < pl.njobs; ++t) {
-        lv.hi[t] = pl.level[t] <= 5;
-        lv.sh[t] = (signed char)(8 * ((pl.level[t] <= 5 ? 5 : 9) - pl.level[t]));
-    }
-    return lv;
 }
 
 constexpr size_t kLinkSmem = 96 * 1024;    // a part of at most 12288 samples
 
 }  // namespace
 
-bool split_plan(int M, int N, int K, int bn, bool pair, size_t max_ints, SplitPlan* out) {
+bool split_plan(int M, int N, int K, int nd, int bn, bool pair, SplitPlan* out) {
     const int kbs = (K + 63) / 64, chunk = kSplitChunk;
     const int mt = (M + 127) / 128, nt = (N + bn - 1) / bn;
     pair = pair && mt >= 2;
     const long tiles = (long)(pair ? (mt + 1) / 2 : mt) * nt;
     const int workers = pair ? 76 : 152;
-    const double total = 36.0 * kbs * (double)tiles;
+    const double total = 0.5 * nd * (nd + 1) * kbs * (double)tiles;
     // microseconds of one K slice of a tile (operands at ~68 bytes per cycle and SM, as
-    // the link product measures), of a unit's start and end, and of a slice's trip
-    // through memory
+    // the link product measures), of a unit's start and end, and of a slice of integers:
+    // written and read, or with levels in pieces zeroed, added to piece by piece and read
     const double us_kb = (128.0 + (pair ? bn / 2 : bn)) * 128.0 / 68.0 / 1900.0;
-    const double us_unit = 2.0, us_slice = (double)M * N * 8.0 / 6.0e6;
+    const double us_unit = 2.0, mn = (double)M * N * 4.0;
     double best = 1e300;
     for (int w : {0, 1, 2, 3, 4, 6, 8}) {
         // pieces of at most J slices (whole chunks; a job's sum stays below 2^31); w = 0: as few as possible
         long J = w == 0 ? 2032 : (long)(total / ((double)workers * w)) + 1;
-        J = std::min<long>(2032, std::max<long>(2 * chunk, (J + chunk - 1) / chunk * chunk));
+        J = std::min<long>(2032, std::max<long>(chunk, (J + chunk - 1) / chunk * chunk));
         SplitPlan p{};
+        p.nd = nd;
         p.kbs = kbs;
         bool fits = true;
-        for (int l = 9; l >= 2 && fits; --l) {
+        for (int l = nd + 1; l >= 2 && fits; --l) {
             const int kb = (l - 1) * kbs, cnt = (int)((kb + J - 1) / J);
             const int per = ((kb + cnt - 1) / cnt + chunk - 1) / chunk * chunk;
             for (int u0 = 0; u0 < kb; u0 += per) {
                 if (p.njobs >= kTcMaxJobs) { fits = false; break; }
-                p.jobs[p.njobs] = {(9 - l) * kbs + u0, u0, std::min(per, kb - u0), 0};
-                p.level[p.njobs++] = l;
+                p.jobs[p.njobs++] = {(nd + 1 - l) * kbs + u0, u0, std::min(per, kb - u0), l - 2};
             }
         }
-        if (!fits || (size_t)p.njobs * M * N > max_ints) continue;
-        int at[kTcMaxJobs];
-        for (int t = 0; t < p.njobs; ++t) at[t] = t;
-        std::stable_sort(at, at + p.njobs, [&](int a, int b) { return p.jobs[a].nkb > p.jobs[b].nkb; });
-        SplitPlan q = p;
-        for (int t = 0; t < p.njobs; ++t) {
-            q.jobs[t] = p.jobs[at[t]];
-            q.jobs[t].slice = t;
-            q.level[t] = p.level[at[t]];
-        }
+        if (!fits) continue;
+        std::stable_sort(p.jobs, p.jobs + p.njobs, [](const TcJob& a, const TcJob& b) { return a.nkb > b.nkb; });
         // the busiest worker: units dealt forwards and backwards in turn (gemm_tc.cu)
         double worst;
-        const long units = tiles * q.njobs;
+        const long units = tiles * p.njobs;
         if (units > 64L * workers) {
             worst = (total * us_kb + units * us_unit) / workers;
         } else {
@@ -293,14 +229,14 @@ bool split_plan(int M, int N, int K, int bn, bool pair, size_t max_ints, SplitPl
             for (long u = 0; u < units; ++u) {
                 const long pass = u / workers, a = u - pass * workers;
                 const long width = std::min<long>(workers, units - pass * workers);
-                load[(pass & 1) ? width - 1 - a : a] += q.jobs[u / tiles].nkb * us_kb + us_unit;
+                load[(pass & 1) ? width - 1 - a : a] += p.jobs[u / tiles].nkb * us_kb + us_unit;
             }
             worst = *std::max_element(load, load + workers);
         }
-        const double cost = worst + q.njobs * us_slice;
+        const double cost = worst + (p.njobs > nd ? 2.0 + (p.njobs / 2.5e6 + 2.0 * nd / 6.0e6) * mn : 2.0 * nd / 6.0e6 * mn);
         if (cost < best) {
             best = cost;
-            *out = q;
+            *out = p;
         }
     }
     return best < 1e300;
@@ -313,14 +249,13 @@ void split_digits(cudaStream_t s, const double* V, int rows, int n, size_t ldv, 
     else k_split_digits<256><<<rows, 256, 0, s>>>(V, rows, n, ldv, npad, ce, inv, reversed, D, scale, flag);
 }
 
-void split_combine(cudaStream_t s, int rows, int cols, const int* I, size_t stride, const SplitPlan& pl,
-                   const int* er, const int* ec, double* out) {
+void split_combine(cudaStream_t s, int rows, int cols, const int* I, size_t stride, const int* er, const int* ec,
+                   double* out) {
     // rows on the grid's y axis, in runs of at most 65535
     for (int b0 = 0; b0 < rows; b0 += 65535) {
         const int rr = std::min(65535, rows - b0);
         const dim3 grid(std::max(1, std::min(8, (cols + 255) / 256)), rr);
-        k_split_combine<<<grid, 256, 0, s>>>(cols, I + (size_t)b0 * cols, stride, levels_of(pl), er + b0, ec,
-                                             out + (size_t)b0 * cols);
+        k_split_combine<<<grid, 256, 0, s>>>(cols, I + (size_t)b0 * cols, stride, er + b0, ec, out + (size_t)b0 * cols);
     }
 }
 
@@ -330,8 +265,8 @@ int split_prepare() {
     return rc;
 }
 
-int split_link(cudaStream_t s, int m, int n, int npad, const int* I, size_t stride, const SplitPlan& pl, const int* ev,
-               const int* ex, const double* y, int kind, __nv_bfloat16* D, int* er) {
+int split_link(cudaStream_t s, int m, int n, int npad, const int* I, size_t stride, const int* ev, const int* ex,
+               const double* y, int kind, __nv_bfloat16* D, int* er) {
     if (m <= 0) return 0;
     int parts = 1;
     while (parts < 8 && ((long)m * parts < 2 * 152 || (size_t)n * 8 > kLinkSmem * parts) &&
@@ -350,8 +285,8 @@ int split_link(cudaStream_t s, int m, int n, int npad, const int* I, size_t stri
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = parts > 1 ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k_split_link, n, npad, parts, seg, I, stride, levels_of(pl), ev, ex, y, kind, D,
-                              er) == cudaSuccess ? 0 : -1;
+    return cudaLaunchKernelEx(&cfg, k_split_link, n, npad, parts, seg, I, stride, ev, ex, y, kind, D, er) ==
+                   cudaSuccess ? 0 : -1;
 }
 
 }  // namespace kglm
