@@ -322,7 +322,9 @@ kglm_status kglm_autotune(kglm_ctx* ctx, int32_t iters, uint64_t seed, kglm_tune
 
 /* Set the tuning choices by hand (the fields of kglm_tune; a 0 tile, split cap
  * batch or sub_batches keeps the current value; `timed` and the rates are
- * ignored).  The
+ * ignored).  Until a tile is set here or by kglm_autotune the engine picks the
+ * tiles, and until `pair` is set the CTA pairs, from the sizes of each product;
+ * no result depends on them.  The
  * split cap may not exceed the slices allocated at creation.  pdl 0 launches
  * the iteration kernels without programmatic dependent launch. */
 kglm_status kglm_configure(kglm_ctx* ctx, const kglm_tune* cfg);

@@ -40,6 +40,13 @@ struct SavedSolve {
     int64_t nodes = 0, batches = 0, next_id = 0;
 };
 
+// Column tile, CTA pairs and split-K slices (0: the launcher's own count) of a product.
+struct Tiling {
+    int bn;
+    bool pair;
+    int splits;
+};
+
 struct kglm_ctx {
     kglm_desc d{};
     cudaStream_t st = nullptr;
@@ -97,6 +104,10 @@ struct kglm_ctx {
     TcMap mA1{}, mB1{}, mB1lo{}, mA2{}, mB2{}, mA1lo{}, mA2lo{}, mB2lo{};
     TcMap gB1{}, gB2{};            // X and X^T maps at the bucketed tile widths of grouped launches
     int gbn1 = 0, gbn2 = 0;
+    // tiles by rule (pick_tiling) until kglm_configure or kglm_autotune sets them
+    bool tiles_auto = true, pair_auto = true;
+    std::map<std::pair<int, int>, Tiling> tilings;   // by (rows, product)
+    std::map<std::pair<int, int>, TcMap> bmaps;      // B operands' maps by (operand, tile width)
     // FP32-accurate mode: beta as a TF32 hi + lo operand for the certificate's X beta
     float *Bop = nullptr, *Bop_lo = nullptr;
     TcMap mAb{}, mAblo{};
@@ -345,7 +356,6 @@ void harvest(kglm_ctx* c) {
     cudaGetLastError();
 }
 
-void check_tc_error(kglm_ctx* c);
 
 double delta_of(const kglm_ctx* c, double ub) { return isfinite(ub) ? c->gap_tol * fmax(1.0, fabs(ub)) : 0.0; }
 
@@ -528,6 +538,90 @@ void xtzeta(kglm_ctx* c, int m, CertArgs& a) {
     a.ebound = x.ebound;
 }
 
+// ---- tiles of the tensor-core products where nobody set them
+// Microseconds of an M x N product over nkb K slices of 128 bytes at column tile bn: the
+// busiest worker's units, each bound by its products (2 cycles per column, slice and
+// part product) or by its operands' way from L2.  Measured on S = X V of 2048 nodes, n =
+// 10000, p = 2000: single CTAs take 0.50 us a slice whether the tile has 128 columns or
+// 224 (up to 87 KB/us), pairs 0.39 to 0.41 us at 192 to 256 columns (78 KB/us per CTA).
+// Plus the last unit's epilogue and a pair's cluster launch.
+double tiling_cost(int M, int N, int nkb, int na, int nb, int bn, bool pair, int splits) {
+    const int mt = (M + 127) / 128, nt = (N + bn - 1) / bn;
+    const long units = (long)(pair ? (mt + 1) / 2 : mt) * nt * splits;
+    const int workers = pair ? 76 : 152;
+    const double per = (nkb + splits - 1) / splits;
+    const double mma = 2.0 * bn * (na + nb - 1) / 1900.0;
+    const double load = pair ? std::max((128.0 + bn / 2) * 0.128 / 78.0, 0.38)
+                             : std::max((128.0 * na + (double)bn * nb) * 0.128 / 87.0, 0.48);
+    const double unit = per * std::max(mma, load) + 0.5;
+    return (double)((units + workers - 1) / workers) * unit + 2.5 * bn / 256.0 + (pair ? 1.5 : 0.0);
+}
+
+// The column tile and CTA pairs of a product of M nodes.  The
+// default widths leave SMs idle in the last wave (2048 nodes, p = 2000: 128 units on
+// 152 SMs) and take in twice the operand bytes a pair does.  The number of split-K
+// slices stays the default width's, and a product's sums run over K in the same order at
+// any width and in pairs, so that no bit of a result depends on the choice.  2048
+// nodes, n = 10000, p = 2000: S 147 -> 70 us per launch, G 81 -> 65,
+// X beta 420 -> 365; 64 nodes,
+// n = 1373, p = 611: G 16.3 -> 11.3 us.
+enum { TILE_LINK = 0, TILE_GRAD = 1, TILE_CERT = 2 };   // S = X V, G = X^T R, the certificate's X beta (TF32 hi + lo)
+Tiling pick_tiling(kglm_ctx* c, int M, int which) {
+    const bool grad = which == TILE_GRAD, cert = which == TILE_CERT;
+    const int def = grad ? c->bn2 : cert && c->tc_kind == 0 ? c->bnc : c->bn1;
+    if (!c->tiles_auto) return {def, cert ? false : c->pair, 0};
+    const auto key = std::make_pair(M, which);
+    const auto it = c->tilings.find(key);
+    if (it != c->tilings.end()) return it->second;
+    const int N = grad ? c->p : c->n, K = grad ? c->n : c->p, ke = c->tc_kind == 0 && !cert ? 64 : 32;
+    const int nkb = (K + ke - 1) / ke, mt = (M + 127) / 128;
+    const int na = c->x3 || cert ? 2 : 1, nb = grad ? (c->x3 ? 2 : 1) : (c->xlo || cert ? 2 : 1);
+    const int tiles = mt * ((N + def - 1) / def);
+    // the default's split-K (tc_gemm)
+    int splits = grad ? std::max(1, std::min(c->gsplit_max, std::min((nkb + 3) / 4, std::max(1, 152 / tiles))))
+                      : (tiles < 152 ? std::min((nkb + 3) / 4, std::max(1, 152 / tiles)) : 1);
+    Tiling best{def, false, splits};
+    if (grad || splits == 1) {
+        const bool can_pair = c->tc_kind == 0 && !cert && mt >= 2;
+        double cost = tiling_cost(M, N, nkb, na, nb, def, best.pair, splits);
+        for (int bn = 64; bn <= tc_tile_cols(N); bn += 16)
+            for (int pr = 0; pr <= (can_pair ? 1 : 0); ++pr) {
+                if (!c->pair_auto && (pr != 0) != (c->pair && can_pair)) continue;
+                const double t = tiling_cost(M, N, nkb, na, nb, bn, pr != 0, splits);
+                if (t < 0.97 * cost) {
+                    cost = t;
+                    best = {bn, pr != 0, splits};
+                }
+            }
+    } else {
+        best.splits = 0;                                // a split link product keeps its launcher's plan
+    }
+    if (c->tilings.size() >= 256) c->tilings.clear();
+    c->tilings[key] = best;
+    return best;
+}
+
+// The map of a B operand (0, 1: X and its low part; 2, 3: X^T and its low part; 4, 5: the
+// BF16 mode's X as TF32 hi and lo) at a tile width.
+const TcMap& b_map(kglm_ctx* c, int which, int bn) {
+    if (bn == (which < 2 ? c->bn1 : which < 4 ? c->bn2 : c->bnc)) {
+        const TcMap* m[6] = {&c->mB1, &c->mB1lo, &c->mB2, &c->mB2lo, &c->mXc, &c->mXclo};
+        return *m[which];
+    }
+    const auto key = std::make_pair(which, bn);
+    auto it = c->bmaps.find(key);
+    if (it == c->bmaps.end()) {
+        const int ob = c->tc_kind == 0 && which < 4;
+        TcMap m{};
+        const void* base[6] = {c->Xop, c->Xop_lo, c->Xtop, c->Xtop_lo, c->Xc, c->Xc_lo};
+        if (which == 2 || which == 3 ? tc_make_map(&m, base[which], ob, c->p, c->n, c->nK, bn)
+                                     : tc_make_map(&m, base[which], ob, c->n, c->p, c->pK, bn))
+            throw Fail{KGLM_ECUDA, "cuTensorMapEncodeTiled failed for a tile width"};
+        it = c->bmaps.emplace(key, m).first;
+    }
+    return it->second;
+}
+
 void certify(kglm_ctx* c) {
     Nvtx range("certificate");
     const int m = c->m, n = c->n, p = c->p;
@@ -561,11 +655,13 @@ void certify(kglm_ctx* c) {
             convert_pad_f32(c->st, (const float*)c->B, m, p, c->Bop, c->pK, 0, c->Bop_lo);
             check_launch();
             const bool own = c->tc_kind == 0;
+            const Tiling t = pick_tiling(c, m, TILE_CERT);
             TcGemm g{};
-            g.kind = 1; g.M = m; g.N = n; g.K = p; g.bn = own ? c->bnc : c->bn1;
+            g.kind = 1; g.M = m; g.N = n; g.K = p; g.bn = t.bn;
             g.epi = TC_EPI_STORE_F32; g.out = c->R; g.ldo = n; g.err = c->d_tcerr;
             g.A2 = &c->mAblo;
-            if (tc_gemm(c->st, c->mAb, own ? c->mXc : c->mB1, own ? &c->mXclo : &c->mB1lo, g, &c->gtc) != 0)
+            if (tc_gemm(c->st, c->mAb, b_map(c, own ? 4 : 0, t.bn), &b_map(c, own ? 5 : 1, t.bn), g,
+                        t.splits == 1 ? nullptr : &c->gtc) != 0)
                 throw Fail{KGLM_ECUDA, "tensor-core launch failed (certificate X beta)"};
         } else {
             gemm_nt_f32(c->st, m, n, p, (const float*)c->B, p, c->X32, p, (float*)c->R, n, &c->gs32);
@@ -643,15 +739,17 @@ void iterate_rows(kglm_ctx* c, cudaStream_t st, int row0, int mr, bool sub) {
     {
         Scope sc(c, PH_GEMM_LINK, 1, flops);
         TcGemm g{};
-        g.kind = c->tc_kind; g.M = mr; g.N = n; g.K = p; g.bn = c->bn1;
+        const Tiling t = pick_tiling(c, mr, TILE_LINK);
+        g.kind = c->tc_kind; g.M = mr; g.N = n; g.K = p; g.bn = t.bn;
         g.arow0 = row0;
         g.epi = c->tc_kind == 0 ? TC_EPI_LINK_BF16 : TC_EPI_LINK_F32;
         g.out = static_cast<char*>(c->Rop) + (size_t)row0 * c->nK * es;
         g.ldo = c->nK; g.y = c->y32; g.loss = c->kind; g.err = c->d_tcerr;
         if (c->x3) { g.A2 = &c->mA1lo; g.out_lo = c->Rop_lo + (size_t)row0 * c->nK; }
         g.pdl = pdl;
-        g.pair = c->pair;
-        if (tc_gemm(st, c->mA1, c->mB1, c->xlo ? &c->mB1lo : nullptr, g, sub ? nullptr : &c->gtc) != 0)
+        g.pair = t.pair;
+        if (tc_gemm(st, c->mA1, b_map(c, 0, t.bn), c->xlo ? &b_map(c, 1, t.bn) : nullptr, g,
+                    sub || t.splits == 1 ? nullptr : &c->gtc) != 0)
             throw Fail{KGLM_ECUDA, "tensor-core product setup failed"};
         check_launch();
     }
@@ -659,15 +757,17 @@ void iterate_rows(kglm_ctx* c, cudaStream_t st, int row0, int mr, bool sub) {
     {
         Scope sc(c, PH_GEMM_GRAD, 1, flops);
         TcGemm g{};
-        g.kind = c->tc_kind; g.M = mr; g.N = p; g.K = n; g.bn = c->bn2;
+        const Tiling t = pick_tiling(c, mr, TILE_GRAD);
+        g.kind = c->tc_kind; g.M = mr; g.N = p; g.K = n; g.bn = t.bn;
         g.arow0 = row0;
+        g.splits = t.splits;
         g.epi = TC_EPI_PARTIAL; g.err = c->d_tcerr;
         g.pout = c->Gpart + (size_t)row0 * p; g.pstride = (size_t)c->mcap * p; g.pld = p;
         g.max_splits = c->gsplit_max; g.splits_used = &splits;
         if (c->x3) g.A2 = &c->mA2lo;
         g.pdl = pdl;
-        g.pair = c->pair;
-        if (tc_gemm(st, c->mA2, c->mB2, c->x3 ? &c->mB2lo : nullptr, g, &c->gtc) != 0)
+        g.pair = t.pair;
+        if (tc_gemm(st, c->mA2, b_map(c, 2, t.bn), c->x3 ? &b_map(c, 3, t.bn) : nullptr, g, &c->gtc) != 0)
             throw Fail{KGLM_ECUDA, "tensor-core product setup failed"};
         check_launch();
     }
@@ -1035,16 +1135,14 @@ void finish_tc_check(kglm_ctx* c) {
     }
 }
 
-// A tensor-core product whose mbarrier wait ran out leaves a flag (the kernel
-// drained its work and freed its tensor memory before returning).
-void check_tc_error(kglm_ctx* c) {
-    int h = 0;
-    CK(cudaMemcpyAsync(&h, c->d_tcerr, sizeof(int), cudaMemcpyDeviceToHost, c->st));
+// The end of a call that ran a tensor-core product: one synchronisation, with the flag
+// that a wait that ran out leaves (the kernel drained its work and freed its tensor
+// memory before returning).
+void sync_tc(kglm_ctx* c) {
+    CK(cudaMemcpyAsync(c->pinned<int>(c->off_tcerr()), c->d_tcerr, sizeof(int), cudaMemcpyDeviceToHost, c->st));
     sync(c);
-    if (h) {
-        CK(cudaMemsetAsync(c->d_tcerr, 0, sizeof(int), c->st));
-        throw Fail{KGLM_ETIMEOUT, "a tensor-core product's pipeline wait ran out"};
-    }
+    c->tc_check_pending = true;
+    finish_tc_check(c);
 }
 
 void validate_nodes(const kglm_ctx* c, int m, const int32_t* in_ptr, const int32_t* in_idx,
@@ -1718,6 +1816,8 @@ void set_tiles(kglm_ctx* c, int bn1, int bn2) {
         throw Fail{KGLM_ECUDA, "cuTensorMapEncodeTiled failed while tuning the tiles"};
     c->bn1 = bn1;
     c->bn2 = bn2;
+    c->bmaps.clear();
+    c->tilings.clear();
     destroy_graphs(c);                     // captured launches hold the old maps
 }
 
@@ -1790,6 +1890,7 @@ void autotune_impl(kglm_ctx* c, int iters, uint64_t seed, kglm_tune* out) {
     if (c->tc) {
         // coordinate descent at the full batch: the link product's column tile,
         // then the gradient product's column tile and split cap
+        c->tiles_auto = c->pair_auto = false;
         const int cap = c->gsplit_max;
         // link tile: every width from 32 columns (multiples of 16) up to the sample count
         std::vector<int> t1;
@@ -2331,15 +2432,19 @@ kglm_status kglm_xtr(kglm_ctx* ctx, int32_t m, const void* R, void* G) {
         if (ctx->tc) {
             convert_pad_f32(ctx->st, (const float*)R, m, ctx->n, ctx->Rop, ctx->nK, ctx->tc_kind == 0, ctx->Rop_lo);
             check_launch();
+            // (more nodes than fill the SMs: no split-K, so any tile gives the same sums)
+            Tiling t{ctx->bn2, ctx->pair, 0};
+            if (((m + 127) / 128) * ((ctx->p + ctx->bn2 - 1) / ctx->bn2) >= 152) t = pick_tiling(ctx, m, TILE_GRAD);
             TcGemm g{};
-            g.kind = ctx->tc_kind; g.M = m; g.N = ctx->p; g.K = ctx->n; g.bn = ctx->bn2;
+            g.kind = ctx->tc_kind; g.M = m; g.N = ctx->p; g.K = ctx->n; g.bn = t.bn;
             g.epi = TC_EPI_STORE_F32; g.out = G; g.ldo = ctx->p; g.err = ctx->d_tcerr;
+            g.pair = t.pair;
             if (ctx->x3) g.A2 = &ctx->mA2lo;
-            if (tc_gemm(ctx->st, ctx->mA2, ctx->mB2, ctx->x3 ? &ctx->mB2lo : nullptr, g, &ctx->gtc) != 0)
+            if (tc_gemm(ctx->st, ctx->mA2, b_map(ctx, 2, t.bn), ctx->x3 ? &b_map(ctx, 3, t.bn) : nullptr, g,
+                        t.splits == 1 ? nullptr : &ctx->gtc) != 0)
                 throw Fail{KGLM_ECUDA, "tensor-core product setup failed"};
             check_launch();
-            sync(ctx);
-            check_tc_error(ctx);
+            sync_tc(ctx);
             return;
         }
         if (split_pays(ctx, m)) split_setup(ctx);
@@ -2357,8 +2462,7 @@ kglm_status kglm_xtr(kglm_ctx* ctx, int32_t m, const void* R, void* G) {
                 split_product(ctx, m, true);
                 split_combine(ctx->st, m, ctx->p, q.I, (size_t)m * ctx->p, q.tr, q.sxt, (double*)G);
                 check_launch();
-                sync(ctx);
-                check_tc_error(ctx);
+                sync_tc(ctx);
                 return;
             }
         }
@@ -2396,8 +2500,8 @@ kglm_status kglm_xtz(kglm_ctx* ctx, int32_t m, const double* Z, double* Q, doubl
         }
         CK(cudaMemcpyAsync(Q, c->Q, sizeof(double) * mp, cudaMemcpyDeviceToHost, c->st));
         if (Qerr) CK(cudaMemcpyAsync(Qerr, c->Qerr, sizeof(double) * mp, cudaMemcpyDeviceToHost, c->st));
-        sync(c);
-        if (c->cexact) check_tc_error(c);
+        if (c->cexact) sync_tc(c);
+        else sync(c);
     });
 }
 
@@ -2787,6 +2891,7 @@ kglm_status kglm_configure(kglm_ctx* ctx, const kglm_tune* cfg) {
             REQ(cfg->pair == 1 || cfg->pair == -1, "pair must be 1 (on), -1 (off) or 0 (keep)");
             if (ctx->pair != (cfg->pair == 1)) destroy_graphs(ctx);
             ctx->pair = cfg->pair == 1;
+            ctx->pair_auto = false;
         }
         if (cfg->prox_threads != 0) {
             int opts[4];
@@ -2810,6 +2915,7 @@ kglm_status kglm_configure(kglm_ctx* ctx, const kglm_tune* cfg) {
                     "split cap must be in [1, the allocated slices]");
                 ctx->gsplit_max = cfg->grad_split_cap;
             }
+            if (cfg->link_tile_cols != 0 || cfg->grad_tile_cols != 0) ctx->tiles_auto = false;
             set_tiles(ctx, b1, b2);
         }
         destroy_graphs(ctx);

@@ -77,6 +77,7 @@ struct TcGemm {
     size_t pstride;
     int pld;
     int max_splits;  // TC_EPI_PARTIAL: upper bound on the number of slices
+    int splits;      // TC_EPI_PARTIAL: that many slices instead (0: enough units to fill the SMs)
     int* splits_used;
     const TcMap* A2; // TF32 low part of A (out = (A + A2)(B + B2)^T less A2 B2^T); needs kind 1 and B2
     float* out_lo;   // TC_EPI_LINK_F32: TF32 low part of each output (NULL: none)

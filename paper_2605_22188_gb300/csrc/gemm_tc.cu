@@ -1182,7 +1182,8 @@ int tc_gemm(cudaStream_t s, const TcMap& A, const TcMap& B, const TcMap* B2, con
     // split-K: at least 4 slices of K per unit, until the units fill the SMs
     int splits = 1;
     if (g.epi == TC_EPI_PARTIAL) {
-        splits = std::max(1, std::min(g.max_splits, std::min((a.nkb + 3) / 4, std::max(1, SMS / tiles))));
+        splits = g.splits > 0 ? g.splits
+                              : std::max(1, std::min(g.max_splits, std::min((a.nkb + 3) / 4, std::max(1, SMS / tiles))));
     } else if (tiles < SMS && scr && scr->part && scr->counters && scr->n_counters >= 8 * tiles) {
         splits = std::min((a.nkb + 3) / 4, std::max(1, SMS / tiles));
         const size_t need = (size_t)splits * tiles * BM * MAXBN * sizeof(float);
