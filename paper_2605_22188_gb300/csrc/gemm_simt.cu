@@ -3,8 +3,8 @@
 // §4.2 fused into the epilogue of S (R = dl(S, y) is written, S is not).
 //
 // C[r][c] = sum_k A[r][k] B[c][k]: both operands are K-contiguous (node rows
-// of V or R against rows of X or X^T).  Each CTA computes a BM x BN tile with
-// TM x TN contiguous outputs per thread; the next K slice is prefetched into
+// of V or R against rows of X or X^T).  Each CTA computes a BM x BN tile (in FP64
+// with TM x TN contiguous outputs per thread); the next K slice is prefetched into
 // registers while the current one is multiplied from shared memory.
 //
 // Split-K: when the output has too few tiles to fill the GPU (X^T R is only
@@ -41,7 +41,6 @@ struct EpiLink {
 };
 
 template <typename T> struct Vec4;
-template <> struct Vec4<float> { using type = float4; };
 template <> struct Vec4<double> { using type = double2; };   // 16-byte vector
 
 template <typename T, int BM, int BN, int BK, int TM, int TN, bool VEC, typename Epi>
@@ -204,6 +203,163 @@ __global__ __launch_bounds__((BM / TM) * (BN / TN)) void k_gemm_nt(int R, int C,
     if (tid == 0) counters[tile] = 0;
 }
 
+// The FP32 product: 128 x 128 tiles of 16 of K, double-buffered in shared memory as
+// [K][row], the next slice prefetched into registers.  What bounds it: sm_103a takes a
+// scalar FMA at half the rate of the packed one (fma.rn.f32x2; 36 against some 72
+// TFLOP/s over the chip), and the scalar kernel ran at its 36.  So a thread's 8 x 8
+// outputs are 8 rows x 4 pairs of columns, each half of a pair the same IEEE operation
+// in the same order of K as before.  The four 16-byte quarters of a slice's rows are
+// stored at columns rotated by 8 (an exclusive or), so that neither the transposing
+// stores nor the 16-byte reads conflict.  2048 x 10000 by 1000 columns: 1139 us (36
+// TFLOP/s) with scalar FMAs, now 914 (45); 512 x 5000 by 1000: 181, now 131.  (A's entries
+// stored twice, in place of the eight packing moves per step: 1059 and 150.)
+constexpr int kF32K = 16;
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ void fma2(uint64_t& c, uint64_t a, uint64_t b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
+
+template <bool VEC, typename Epi>
+__global__ __launch_bounds__(256, 2) void k_gemm_f32(int R, int C, int K, const float* __restrict__ A, int lda,
+                                                     const float* __restrict__ B, int ldb, Epi epi, int kchunk,
+                                                     float* __restrict__ part, int* __restrict__ counters) {
+    __shared__ __align__(16) float As[2][kF32K][128];
+    __shared__ __align__(16) float Bs[2][kF32K][128];
+    __shared__ int s_last;
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const int r0 = blockIdx.y * 128, c0 = blockIdx.x * 128;
+    const int kbeg = blockIdx.z * kchunk, kend = min(K, kbeg + kchunk);
+    // a warp loads 8 rows x 64 bytes; quarter kv of row `lr` (and lr + 64)
+    const int lr = tid >> 2, kv = tid & 3;
+    float4 ra[2], rb[2];
+    auto fetch = [&](const float* P, int ld, int row, int rows, int k) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (row < rows) {
+            const float* q = P + (size_t)row * ld + k;
+            if (VEC && k + 4 <= kend) {
+                v = __ldg(reinterpret_cast<const float4*>(q));
+            } else {
+                if (k < kend) v.x = __ldg(q);
+                if (k + 1 < kend) v.y = __ldg(q + 1);
+                if (k + 2 < kend) v.z = __ldg(q + 2);
+                if (k + 3 < kend) v.w = __ldg(q + 3);
+            }
+        }
+        return v;
+    };
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {
+            ra[l] = fetch(A, lda, r0 + lr + 64 * l, R, k0 + 4 * kv);
+            rb[l] = fetch(B, ldb, c0 + lr + 64 * l, C, k0 + 4 * kv);
+        }
+    };
+    auto store = [&](int s) {
+#pragma unroll
+        for (int l = 0; l < 2; ++l) {
+            const int at = (lr + 64 * l) ^ (8 * kv);
+            As[s][4 * kv][at] = ra[l].x; As[s][4 * kv + 1][at] = ra[l].y;
+            As[s][4 * kv + 2][at] = ra[l].z; As[s][4 * kv + 3][at] = ra[l].w;
+            Bs[s][4 * kv][at] = rb[l].x; Bs[s][4 * kv + 1][at] = rb[l].y;
+            Bs[s][4 * kv + 2][at] = rb[l].z; Bs[s][4 * kv + 3][at] = rb[l].w;
+        }
+    };
+    // rows 4 ty + i and 64 + 4 ty + i, columns 4 tx + .. and 64 + 4 tx + ..
+    uint64_t acc[8][4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+    const int nt = kbeg < kend ? (kend - kbeg + kF32K - 1) / kF32K : 0;
+    if (nt > 0) {
+        load(kbeg);
+        store(0);
+    }
+    __syncthreads();
+    for (int it = 0; it < nt; ++it) {
+        if (it + 1 < nt) load(kbeg + (it + 1) * kF32K);
+        const int s = it & 1;
+#pragma unroll
+        for (int k = 0; k < kF32K; ++k) {
+            const int x = 8 * (k >> 2);
+            const float4 a0 = *reinterpret_cast<const float4*>(&As[s][k][(4 * ty) ^ x]);
+            const float4 a1 = *reinterpret_cast<const float4*>(&As[s][k][64 + ((4 * ty) ^ x)]);
+            const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(&Bs[s][k][(4 * tx) ^ x]);
+            const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(&Bs[s][k][64 + ((4 * tx) ^ x)]);
+            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const uint64_t aa = pack2(a[i], a[i]);
+                fma2(acc[i][0], aa, b0.x);
+                fma2(acc[i][1], aa, b0.y);
+                fma2(acc[i][2], aa, b1.x);
+                fma2(acc[i][3], aa, b1.y);
+            }
+        }
+        if (it + 1 < nt) store(s ^ 1);
+        __syncthreads();
+    }
+    auto out = [&] {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float2 v = unpack2(acc[i][j]);
+                const int r = r0 + 4 * ty + (i & 3) + 64 * (i >> 2), c = c0 + 4 * tx + 2 * (j & 1) + 64 * (j >> 1);
+                if (r < R && c < C) epi(r, c, v.x);
+                if (r < R && c + 1 < C) epi(r, c + 1, v.y);
+            }
+    };
+    if (gridDim.z == 1) {
+        out();
+        return;
+    }
+    // split-K: publish the partial tile, the last arriving CTA reduces it (k_gemm_nt)
+    const int tile = blockIdx.y * gridDim.x + blockIdx.x, ntile = gridDim.x * gridDim.y;
+    uint64_t* my = reinterpret_cast<uint64_t*>(part + ((size_t)blockIdx.z * ntile + tile) * (128 * 128)) + tid;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) my[(i * 4 + j) * 256] = acc[i][j];
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = (atomicAdd(&counters[tile], 1) == (int)gridDim.z - 1);
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    float2 sum[8][4];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) sum[i][j] = make_float2(0.f, 0.f);
+    for (int z = 0; z < (int)gridDim.z; ++z) {
+        const float2* ps = reinterpret_cast<const float2*>(part + ((size_t)z * ntile + tile) * (128 * 128)) + tid;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float2 v = __ldcg(ps + (i * 4 + j) * 256);
+                sum[i][j].x += v.x;
+                sum[i][j].y += v.y;
+            }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = pack2(sum[i][j].x, sum[i][j].y);
+    out();
+    if (tid == 0) counters[tile] = 0;
+}
+
 constexpr int kSMs = 152;
 
 // The FP64 product for outputs that would leave most of a 64 x 64 tile empty
@@ -321,7 +477,7 @@ __global__ __launch_bounds__(256) void k_power_step(int p, const double* __restr
 
 template <typename T>
 struct Tile;
-template <> struct Tile<float> { static constexpr int BM = 128, BN = 128, BK = 8, TM = 8, TN = 8; };
+template <> struct Tile<float> { static constexpr int BM = 128, BN = 128, BK = 8; };   // BK: what a chunk of K is a multiple of
 template <> struct Tile<double> { static constexpr int BM = 64, BN = 64, BK = 8, TM = 4, TN = 4; };
 
 // Resident CTAs per SM of the tile configuration (2 for the FP32 tile, 128
@@ -420,6 +576,28 @@ bool launch_small(cudaStream_t s, int R, int C, int K, const double* A, int lda,
     return true;
 }
 
+// The tiles of a plan: k_gemm_f32, or k_gemm_nt in FP64.
+template <typename T, typename Epi>
+void launch_tiles(cudaStream_t s, int R, int C, int K, const T* A, int lda, const T* B, int ldb, Epi epi,
+                  const GemmPlan& g, T* part, int* cnt) {
+    using TL = Tile<T>;
+    constexpr int VW = 16 / sizeof(T);
+    const bool vec = (lda % VW == 0) && (ldb % VW == 0) && ((uintptr_t)A % 16 == 0) && ((uintptr_t)B % 16 == 0);
+    const dim3 grid(g.gx, g.gy, g.splits);
+    if constexpr (sizeof(T) == 4) {
+        if (vec) k_gemm_f32<true, Epi><<<grid, 256, 0, s>>>(R, C, K, A, lda, B, ldb, epi, g.kchunk, part, cnt);
+        else k_gemm_f32<false, Epi><<<grid, 256, 0, s>>>(R, C, K, A, lda, B, ldb, epi, g.kchunk, part, cnt);
+    } else {
+        constexpr int NT = (TL::BM / TL::TM) * (TL::BN / TL::TN);
+        if (vec)
+            k_gemm_nt<T, TL::BM, TL::BN, TL::BK, TL::TM, TL::TN, true, Epi><<<grid, NT, 0, s>>>(
+                R, C, K, A, lda, B, ldb, epi, g.kchunk, part, cnt);
+        else
+            k_gemm_nt<T, TL::BM, TL::BN, TL::BK, TL::TM, TL::TN, false, Epi><<<grid, NT, 0, s>>>(
+                R, C, K, A, lda, B, ldb, epi, g.kchunk, part, cnt);
+    }
+}
+
 template <typename T, typename Epi>
 void launch(cudaStream_t s, int R, int C, int K, const T* A, int lda, const T* B, int ldb, Epi epi,
             const GemmScratch* scr) {
@@ -442,16 +620,7 @@ void launch(cudaStream_t s, int R, int C, int K, const T* A, int lda, const T* B
         }
     }
     if (K <= 0) g.kchunk = 1;
-    constexpr int VW = 16 / sizeof(T);
-    const bool vec = (lda % VW == 0) && (ldb % VW == 0) && ((uintptr_t)A % 16 == 0) && ((uintptr_t)B % 16 == 0);
-    dim3 grid(g.gx, g.gy, g.splits);
-    constexpr int NT = (TL::BM / TL::TM) * (TL::BN / TL::TN);
-    if (vec)
-        k_gemm_nt<T, TL::BM, TL::BN, TL::BK, TL::TM, TL::TN, true, Epi><<<grid, NT, 0, s>>>(
-            R, C, K, A, lda, B, ldb, epi, g.kchunk, part, cnt);
-    else
-        k_gemm_nt<T, TL::BM, TL::BN, TL::BK, TL::TM, TL::TN, false, Epi><<<grid, NT, 0, s>>>(
-            R, C, K, A, lda, B, ldb, epi, g.kchunk, part, cnt);
+    launch_tiles<T>(s, R, C, K, A, lda, B, ldb, epi, g, part, cnt);
 }
 
 // Like launch(), but when the scratch cannot hold the planned partials the
@@ -478,18 +647,9 @@ void launch_clamped(cudaStream_t s, int R, int C, int K, const T* A, int lda, co
         g.splits = 1;
         g.kchunk = K > 0 ? K : 1;
     }
-    constexpr int VW = 16 / sizeof(T);
-    const bool vec = (lda % VW == 0) && (ldb % VW == 0) && ((uintptr_t)A % 16 == 0) && ((uintptr_t)B % 16 == 0);
-    dim3 grid(g.gx, g.gy, g.splits);
-    constexpr int NT = (TL::BM / TL::TM) * (TL::BN / TL::TN);
     T* part = g.splits > 1 ? static_cast<T*>(scr.part) : nullptr;
     int* cnt = g.splits > 1 ? scr.counters : nullptr;
-    if (vec)
-        k_gemm_nt<T, TL::BM, TL::BN, TL::BK, TL::TM, TL::TN, true, Epi><<<grid, NT, 0, s>>>(
-            R, C, K, A, lda, B, ldb, epi, g.kchunk, part, cnt);
-    else
-        k_gemm_nt<T, TL::BM, TL::BN, TL::BK, TL::TM, TL::TN, false, Epi><<<grid, NT, 0, s>>>(
-            R, C, K, A, lda, B, ldb, epi, g.kchunk, part, cnt);
+    launch_tiles<T>(s, R, C, K, A, lda, B, ldb, epi, g, part, cnt);
 }
 
 template <typename T>
@@ -498,11 +658,16 @@ int ctas_per_sm() {
     // thread-safe; calls may come from several host threads at once)
     static const int cached = [] {
         using TL = Tile<T>;
-        constexpr int NT = (TL::BM / TL::TM) * (TL::BN / TL::TN);
         int n = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                &n, k_gemm_nt<T, TL::BM, TL::BN, TL::BK, TL::TM, TL::TN, true, EpiStore<T>>, NT, 0) != cudaSuccess ||
-            n <= 0) {
+        cudaError_t e;
+        if constexpr (sizeof(T) == 4) {
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_gemm_f32<true, EpiStore<T>>, 256, 0);
+        } else {
+            constexpr int NT = (TL::BM / TL::TM) * (TL::BN / TL::TN);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                &n, k_gemm_nt<T, TL::BM, TL::BN, TL::BK, TL::TM, TL::TN, true, EpiStore<T>>, NT, 0);
+        }
+        if (e != cudaSuccess || n <= 0) {
             cudaGetLastError();
             n = 2;
         }
