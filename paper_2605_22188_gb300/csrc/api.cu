@@ -422,7 +422,8 @@ void split_setup(kglm_ctx* c) {
     q.nk = (int)((n + 63) / 64 * 64);
     q.bnS = tc_tile_cols((int)n);
     q.bnG = tc_tile_cols((int)p);
-    q.cap = 8 * mc * std::max(n, p);                   // a slice of integers per level
+    // a slice of integers per level and part
+    q.cap = 8 * mc * std::max(n * split_parts((int)p, 8), p * split_parts((int)n, 8));
     const size_t need = 16 * ((n + mc) * q.pk + (p + mc) * q.nk) + 4 * (n + p + 2 * mc) + 4 * q.cap + 64;
     if (c->d.hbm_budget > 0 && (int64_t)(c->bytes + need) > c->d.hbm_budget) return;
     const size_t had = c->allocs.size(), bytes0 = c->bytes;
@@ -487,7 +488,7 @@ void digit_product(kglm_ctx* c, int m, int N, int K, int nd, int bn, const TcMap
     }
     const size_t mn = (size_t)m * N;
     const bool add = pl.njobs > nd;
-    if (add) CK(cudaMemsetAsync(I, 0, sizeof(int) * nd * mn, c->st));
+    if (add) CK(cudaMemsetAsync(I, 0, sizeof(int) * nd * pl.parts * mn, c->st));
     if (tc_gemm_jobs(c->st, A, B, m, N, bn, pl.jobs, pl.njobs, I, mn, N, c->d_tcerr, 1, kSplitChunk, add) != 0)
         throw Fail{KGLM_ECUDA, "digit product setup failed"};
     check_launch();
@@ -505,13 +506,13 @@ void split_xv(kglm_ctx* c, int m, const double* V, double* out) {
     kglm_ctx::Split64& q = c->sp;
     split_digits(c->st, V, m, c->p, c->p, q.pk, q.sxt, 0, 1, q.DV, q.tv, nullptr);
     split_product(c, m, false);
-    split_combine(c->st, m, c->n, q.I, (size_t)m * c->n, q.tv, q.sx, out);
+    split_combine(c->st, m, c->n, q.I, (size_t)m * c->n, q.pS.parts, q.tv, q.sx, out);
 }
 void split_xtr(kglm_ctx* c, int m, const double* R, double* out) {
     kglm_ctx::Split64& q = c->sp;
     split_digits(c->st, R, m, c->n, c->n, q.nk, nullptr, 0, 1, q.DR, q.tr, nullptr);
     split_product(c, m, true);
-    split_combine(c->st, m, c->p, q.I, (size_t)m * c->p, q.tr, q.sxt, out);
+    split_combine(c->st, m, c->p, q.I, (size_t)m * c->p, q.pG.parts, q.tr, q.sxt, out);
 }
 
 // X^T zeta of the batch's dual points (c->zeta, m x n): FP64 GEMM into c->Q,
@@ -533,6 +534,7 @@ void xtzeta(kglm_ctx* c, int m, CertArgs& a) {
     digit_product(c, m, p, n, kCertDigits, c->bnx, c->mAz, c->mBx, c->Qi, c->pC, c->mC);
     a.Qi = c->Qi;
     a.qi_stride = (size_t)m * p;
+    a.qi_parts = c->pC.parts;
     a.xsig = c->xsig;
     a.ztau = c->ztau;
     a.ebound = x.ebound;
@@ -790,13 +792,13 @@ void iterate(kglm_ctx* c) {
             Scope sc(c, PH_GEMM_LINK, 3, flops);
             split_digits(c->st, (const double*)c->V, m, p, p, q.pk, q.sxt, 0, 1, q.DV, q.tv, nullptr);
             split_product(c, m, false);
-            if (split_link(c->st, m, n, q.nk, q.I, (size_t)m * n, q.tv, q.sx, c->y64, c->kind, q.DR, q.tr) != 0)
+            if (split_link(c->st, m, n, q.nk, q.I, (size_t)m * n, q.pS.parts, q.tv, q.sx, c->y64, c->kind, q.DR, q.tr) != 0)
                 throw Fail{KGLM_ECUDA, "FP64 link launch failed"};
             check_launch();
         }
         Scope sc(c, PH_GEMM_GRAD, 2, flops);
         split_product(c, m, true);
-        split_combine(c->st, m, p, q.I, (size_t)m * p, q.tr, q.sxt, (double*)c->G);
+        split_combine(c->st, m, p, q.I, (size_t)m * p, q.pG.parts, q.tr, q.sxt, (double*)c->G);
         check_launch();
     } else {
         {
@@ -2460,7 +2462,7 @@ kglm_status kglm_xtr(kglm_ctx* ctx, int32_t m, const void* R, void* G) {
             sync(ctx);
             if (!bad) {
                 split_product(ctx, m, true);
-                split_combine(ctx->st, m, ctx->p, q.I, (size_t)m * ctx->p, q.tr, q.sxt, (double*)G);
+                split_combine(ctx->st, m, ctx->p, q.I, (size_t)m * ctx->p, q.pG.parts, q.tr, q.sxt, (double*)G);
                 check_launch();
                 sync_tc(ctx);
                 return;
@@ -2493,7 +2495,7 @@ kglm_status kglm_xtz(kglm_ctx* ctx, int32_t m, const double* Z, double* Q, doubl
         }
         if (!c->Qerr) c->Qerr = dalloc_t<double>(c, (size_t)c->mcap * c->p);
         if (a.Qi) {
-            exact_combine(c->st, m, c->p, a.Qi, a.qi_stride, c->xsig, c->ztau, a.ebound, c->Q, c->Qerr);
+            exact_combine(c->st, m, c->p, a.Qi, a.qi_stride, a.qi_parts, c->xsig, c->ztau, a.ebound, c->Q, c->Qerr);
             check_launch();
         } else {
             CK(cudaMemsetAsync(c->Qerr, 0, sizeof(double) * mp, c->st));

@@ -430,7 +430,7 @@ __global__ __launch_bounds__(NT) void k_cert_node(const __grid_constant__ CertAr
             continue;
         }
         double err;
-        const double qv = exact_q(a.Qi, a.qi_stride, base + j, a.xsig[j] * ztau, a.ebound, &err);
+        const double qv = exact_q(a.Qi, a.qi_stride, base + j, a.qi_parts, a.xsig[j] * ztau, a.ebound, &err);
         // |X^T zeta| bounded from above: |Q~| + its distance bound (H_M, TopSum increase in |q|)
         const double v = (fabs(qv) + err) * inv2l;
         if (in) {

@@ -62,13 +62,13 @@ __global__ __launch_bounds__(NT) void k_digits(const double* V, int n, size_t ld
 }
 
 // Q[b][j] and its bound from the jobs' integers (kglm_xtz).
-__global__ void k_exact_combine(int m, int p, const int* Qi, size_t stride,
+__global__ void k_exact_combine(int m, int p, const int* Qi, size_t stride, int parts,
                                 const double* sigma, const double* tau, double ebound, double* Q, double* E) {
     const size_t total = (size_t)m * p;
     for (size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (size_t)gridDim.x * blockDim.x) {
         const int b = (int)(idx / p), j = (int)(idx % p);
         double err;
-        Q[idx] = exact_q(Qi, stride, idx, sigma[j] * tau[b], ebound, &err);
+        Q[idx] = exact_q(Qi, stride, idx, parts, sigma[j] * tau[b], ebound, &err);
         if (E) E[idx] = err;
     }
 }
@@ -81,10 +81,10 @@ void exact_digits(cudaStream_t s, const double* V, int rows, int n, size_t ldv, 
     k_digits<<<rows, NT, 0, s>>>(V, n, ldv, npad, reversed, D, scale);
 }
 
-void exact_combine(cudaStream_t s, int m, int p, const int* Qi, size_t stride, const double* sigma,
+void exact_combine(cudaStream_t s, int m, int p, const int* Qi, size_t stride, int parts, const double* sigma,
                    const double* tau, double ebound, double* Q, double* E) {
     if (m <= 0) return;
-    k_exact_combine<<<2 * 152, 256, 0, s>>>(m, p, Qi, stride, sigma, tau, ebound, Q, E);
+    k_exact_combine<<<2 * 152, 256, 0, s>>>(m, p, Qi, stride, parts, sigma, tau, ebound, Q, E);
 }
 
 bool exact_plan(int n, ExactPlan* pl) {

@@ -119,10 +119,13 @@ struct TcJob {
 int tc_gemm_jobs(cudaStream_t s, const TcMap& A, const TcMap& B, int M, int N, int bn, const TcJob* jobs,
                  int njobs, int* pout, size_t pstride, int pld, int* err, int pair_on, int chunk, int add);
 // Products of signed-byte digits (split64.cu, cert_exact.cu): the jobs of the levels
-// 2 .. nd + 1 (digit pairs a + c = level), largest first; the integers of level l in slice l - 2.
+// 2 .. nd + 1 (digit pairs a + c = level), largest first.  A level's integers stay below
+// 2^31 over kSplitPart K slices; longer levels are taken in parts, part q of level l in
+// slice q nd + l - 2.
 constexpr int kSplitChunk = 16;    // K slices of 64 whose digit products sum to at most 2^24
+constexpr int kSplitPart = 2032;   // K slices (whole chunks) whose digit products sum to less than 2^31
 struct SplitPlan {
-    int nd, kbs, njobs;            // digits, K slices per digit, jobs (more than nd: levels in pieces)
+    int nd, kbs, njobs, parts;     // digits, K slices per digit, jobs (more than nd: levels in pieces), parts
     TcJob jobs[kTcMaxJobs];
 };
 // Exact-splitting certificate product (cert_exact.cu): kCertDigits signed bytes of every
@@ -140,19 +143,20 @@ bool exact_plan(int n, ExactPlan* pl);
 void exact_digits(cudaStream_t s, const double* V, int rows, int n, size_t ldv, int npad, int reversed,
                   __nv_bfloat16* D, double* scale);
 // Q (m x p) and its entrywise bound E (nullable) from the levels' integers.
-void exact_combine(cudaStream_t s, int m, int p, const int* Qi, size_t stride, const double* sigma,
+void exact_combine(cudaStream_t s, int m, int p, const int* Qi, size_t stride, int parts, const double* sigma,
                    const double* tau, double ebound, double* Q, double* E);
+inline int split_parts(int K, int nd) { return (nd * ((K + 63) / 64) + kSplitPart - 1) / kSplitPart; }
 // Jobs for an M x N output over K of nd digits with column tiles of bn; false if they are too many.
 bool split_plan(int M, int N, int K, int nd, int bn, bool pair, SplitPlan* out);
 // Eight digits of every row of V (entry j times 2^ce[j], or 2^-ce[j] with inv) and the row scales' exponents.
 void split_digits(cudaStream_t s, const double* V, int rows, int n, size_t ldv, int npad, const int* ce, int inv,
                   int reversed, __nv_bfloat16* D, int* scale, int* flag);
 // out (rows x cols) from the levels' integers (slice t at I + t stride) and the scales' exponents.
-void split_combine(cudaStream_t s, int rows, int cols, const int* I, size_t stride, const int* er, const int* ec,
-                   double* out);
+void split_combine(cudaStream_t s, int rows, int cols, const int* I, size_t stride, int parts, const int* er,
+                   const int* ec, double* out);
 // R = dl(S, y) from the levels' integers of S = X V, as reversed digits with row exponents er.
-int split_link(cudaStream_t s, int m, int n, int npad, const int* I, size_t stride, const int* ev, const int* ex,
-               const double* y, int kind, __nv_bfloat16* D, int* er);
+int split_link(cudaStream_t s, int m, int n, int npad, const int* I, size_t stride, int parts_k, const int* ev,
+               const int* ex, const double* y, int kind, __nv_bfloat16* D, int* er);
 int split_prepare();
 int tc_gemm(cudaStream_t s, const TcMap& A, const TcMap& B, const TcMap* B2, const TcGemm& g,
             const GemmScratch* scr);
@@ -258,6 +262,7 @@ struct CertArgs {
     // (Qi != NULL) with the entrywise bound xsig_j ztau_b ebound, instead of Q
     const int* Qi;
     size_t qi_stride;
+    int qi_parts;
     const double* xsig;
     double* ztau;
     double ebound;

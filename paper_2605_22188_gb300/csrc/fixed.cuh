@@ -138,19 +138,21 @@ __device__ __forceinline__ void store_digits(const long long (&z)[4], __nv_bfloa
     }
 }
 
-// H and L of one entry of a product of ND digits from its levels' integers (level l in
-// slice l - 2): 2^-40 H + 2^-72 L, levels 2 .. 5 in H.
+// H and L of one entry of a product of ND digits from its levels' integers (level l of
+// part q in slice q ND + l - 2): 2^-40 H + 2^-72 L, levels 2 .. 5 in H.
 template <int ND>
-__device__ __forceinline__ void level_sums(const int* __restrict__ I, size_t stride, size_t idx, long long& H,
-                                           long long& L) {
-    int v[ND];
-#pragma unroll
-    for (int t = 0; t < ND; ++t) v[t] = __ldg(I + (size_t)t * stride + idx);
+__device__ __forceinline__ void level_sums(const int* __restrict__ I, size_t stride, size_t idx, int parts,
+                                           long long& H, long long& L) {
     H = L = 0;
+    for (int q = 0; q < parts; ++q) {
+        int v[ND];
 #pragma unroll
-    for (int t = 0; t < ND; ++t) {
-        if (t < 4) H += (long long)v[t] << (8 * (3 - t));
-        else L += (long long)v[t] << (8 * (7 - t));
+        for (int t = 0; t < ND; ++t) v[t] = __ldg(I + (size_t)(q * ND + t) * stride + idx);
+#pragma unroll
+        for (int t = 0; t < ND; ++t) {
+            if (t < 4) H += (long long)v[t] << (8 * (3 - t));
+            else L += (long long)v[t] << (8 * (7 - t));
+        }
     }
 }
 

@@ -108,22 +108,22 @@ __global__ __launch_bounds__(256) void k_split_digits(const double* __restrict__
 
 // One entry of the product from its levels' integers, times 2^x (x: the sum of the scales'
 // exponents; kBadRow makes it a NaN).
-__device__ __forceinline__ double combine(const int* __restrict__ I, size_t stride, size_t idx, int x) {
+__device__ __forceinline__ double combine(const int* __restrict__ I, size_t stride, size_t idx, int parts, int x) {
     long long H, L;
-    level_sums<8>(I, stride, idx, H, L);
+    level_sums<8>(I, stride, idx, parts, H, L);
     if (x >= kBadRow / 2) return bits_f64(0x7ff8000000000000ull);
     return combine_f64(H, L, x - 72);
 }
 
 // out[b][j] of a rows x cols product of digits (scales 2^er[b], 2^ec[j]).
-__global__ __launch_bounds__(256) void k_split_combine(int cols, const int* __restrict__ I, size_t stride,
+__global__ __launch_bounds__(256) void k_split_combine(int cols, const int* __restrict__ I, size_t stride, int parts,
                                                        const int* __restrict__ er, const int* __restrict__ ec,
                                                        double* __restrict__ out) {
     const int b = blockIdx.y;
     const int s = er[b];
     const size_t base = (size_t)b * cols;
     for (int j = blockIdx.x * 256 + threadIdx.x; j < cols; j += gridDim.x * 256)
-        out[base + j] = combine(I, stride, base + j, s + ec[j]);
+        out[base + j] = combine(I, stride, base + j, parts, s + ec[j]);
 }
 
 // S = X V of a node, its loss derivative R and R's digits: a cluster of CTAs per node,
@@ -135,7 +135,7 @@ __global__ __launch_bounds__(256) void k_split_combine(int cols, const int* __re
 // took about 220 us, now 65.
 constexpr int kLinkNT = 256;
 __global__ __launch_bounds__(kLinkNT) void k_split_link(int n, int npad, int parts, int seg, const int* __restrict__ I,
-                                                        size_t stride, const int* __restrict__ ev, const int* __restrict__ ex,
+                                                        size_t stride, int parts_k, const int* __restrict__ ev, const int* __restrict__ ex,
                                                         const double* __restrict__ y, int kind,
                                                         __nv_bfloat16* __restrict__ D, int* __restrict__ er) {
     extern __shared__ __align__(16) double row[];
@@ -151,7 +151,7 @@ __global__ __launch_bounds__(kLinkNT) void k_split_link(int n, int npad, int par
     const int s = ev[b];
     int key = 0;
     for (int i = i0 + t; i < i1; i += kLinkNT) {
-        const double r = dloss_fixed(combine(I, stride, base + i, s + ex[i]), y[i], kind, tab);
+        const double r = dloss_fixed(combine(I, stride, base + i, parts_k, s + ex[i]), y[i], kind, tab);
         row[i - i0] = r;
         key = max(key, exp_key(r));
     }
@@ -202,21 +202,24 @@ bool split_plan(int M, int N, int K, int nd, int bn, bool pair, SplitPlan* out) 
     const double us_unit = 2.0, mn = (double)M * N * 4.0;
     double best = 1e300;
     for (int w : {0, 1, 2, 3, 4, 6, 8}) {
-        // pieces of at most J slices (whole chunks; a job's sum stays below 2^31); w = 0: as few as possible
-        long J = w == 0 ? 2032 : (long)(total / ((double)workers * w)) + 1;
-        J = std::min<long>(2032, std::max<long>(chunk, (J + chunk - 1) / chunk * chunk));
+        // pieces of at most J slices (whole chunks); w = 0: as few as possible
+        long J = w == 0 ? kSplitPart : (long)(total / ((double)workers * w)) + 1;
+        J = std::min<long>(kSplitPart, std::max<long>(chunk, (J + chunk - 1) / chunk * chunk));
         SplitPlan p{};
         p.nd = nd;
         p.kbs = kbs;
+        p.parts = split_parts(K, nd);
         bool fits = true;
-        for (int l = nd + 1; l >= 2 && fits; --l) {
-            const int kb = (l - 1) * kbs, cnt = (int)((kb + J - 1) / J);
-            const int per = ((kb + cnt - 1) / cnt + chunk - 1) / chunk * chunk;
-            for (int u0 = 0; u0 < kb; u0 += per) {
-                if (p.njobs >= kTcMaxJobs) { fits = false; break; }
-                p.jobs[p.njobs++] = {(nd + 1 - l) * kbs + u0, u0, std::min(per, kb - u0), l - 2};
+        for (int l = nd + 1; l >= 2 && fits; --l)
+            for (int q0 = 0; q0 < (l - 1) * kbs && fits; q0 += kSplitPart) {   // a part, in even pieces
+                const int kb = std::min(kSplitPart, (l - 1) * kbs - q0), cnt = (int)((kb + J - 1) / J);
+                const int per = ((kb + cnt - 1) / cnt + chunk - 1) / chunk * chunk;
+                for (int u0 = 0; u0 < kb; u0 += per) {
+                    if (p.njobs >= kTcMaxJobs) { fits = false; break; }
+                    p.jobs[p.njobs++] = {(nd + 1 - l) * kbs + q0 + u0, q0 + u0, std::min(per, kb - u0),
+                                         q0 / kSplitPart * nd + l - 2};
+                }
             }
-        }
         if (!fits) continue;
         std::stable_sort(p.jobs, p.jobs + p.njobs, [](const TcJob& a, const TcJob& b) { return a.nkb > b.nkb; });
         // the busiest worker: units dealt forwards and backwards in turn (gemm_tc.cu)
@@ -249,13 +252,13 @@ void split_digits(cudaStream_t s, const double* V, int rows, int n, size_t ldv, 
     else k_split_digits<256><<<rows, 256, 0, s>>>(V, rows, n, ldv, npad, ce, inv, reversed, D, scale, flag);
 }
 
-void split_combine(cudaStream_t s, int rows, int cols, const int* I, size_t stride, const int* er, const int* ec,
-                   double* out) {
+void split_combine(cudaStream_t s, int rows, int cols, const int* I, size_t stride, int parts, const int* er,
+                   const int* ec, double* out) {
     // rows on the grid's y axis, in runs of at most 65535
     for (int b0 = 0; b0 < rows; b0 += 65535) {
         const int rr = std::min(65535, rows - b0);
         const dim3 grid(std::max(1, std::min(8, (cols + 255) / 256)), rr);
-        k_split_combine<<<grid, 256, 0, s>>>(cols, I + (size_t)b0 * cols, stride, er + b0, ec, out + (size_t)b0 * cols);
+        k_split_combine<<<grid, 256, 0, s>>>(cols, I + (size_t)b0 * cols, stride, parts, er + b0, ec, out + (size_t)b0 * cols);
     }
 }
 
@@ -265,8 +268,8 @@ int split_prepare() {
     return rc;
 }
 
-int split_link(cudaStream_t s, int m, int n, int npad, const int* I, size_t stride, const int* ev, const int* ex,
-               const double* y, int kind, __nv_bfloat16* D, int* er) {
+int split_link(cudaStream_t s, int m, int n, int npad, const int* I, size_t stride, int parts_k, const int* ev,
+               const int* ex, const double* y, int kind, __nv_bfloat16* D, int* er) {
     if (m <= 0) return 0;
     int parts = 1;
     while (parts < 8 && ((long)m * parts < 2 * 152 || (size_t)n * 8 > kLinkSmem * parts) &&
@@ -285,7 +288,8 @@ int split_link(cudaStream_t s, int m, int n, int npad, const int* I, size_t stri
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = parts > 1 ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k_split_link, n, npad, parts, seg, I, stride, ev, ex, y, kind, D, er) ==
+    return cudaLaunchKernelEx(&cfg, k_split_link, n, npad, parts, seg, I, stride, parts_k, ev, ex, y, kind, D,
+                              er) ==
                    cudaSuccess ? 0 : -1;
 }
 

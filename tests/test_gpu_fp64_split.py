@@ -83,6 +83,34 @@ def test_digit_product_error(n, p, m):
         assert split <= core
 
 
+@pytest.mark.parametrize("prec,n", [("fp64", 33000), ("bf16", 22400)])
+def test_levels_past_31_bits(prec, n):
+    """Rows of one value whose leading bytes are all 127: the sums of a level's digit
+    products pass 2^31 from n = 16640 on (six-digit levels from 22188), so they are held
+    in parts.  FP64: X^T R against the exact sum (the bound above).  BF16: kglm_xtz
+    within its own entrywise bound, at a size where it runs as digits (at 33000 its
+    slices are too many and it is an FP64 sum with an entrywise bound of 0)."""
+    p, m = 130, 128
+    v = sum(127.0 * 2.0 ** (-8 * a) for a in range(1, 7))
+    rng = np.random.default_rng(0)
+    X = np.full((n, p), v) * rng.choice([1.0, 2.0, 0.5], (1, p))
+    R = np.full((m, n), v) * rng.choice([1.0, -1.0, 4.0], (m, 1))
+    y = rng.standard_normal(n)
+    with kglm.Engine(X, y, 3, 1e-2, 2.0, synth.LSQ, prec=prec, max_batch=m, lipschitz=1e5) as eng:
+        if prec == "fp64":
+            before = eng.device_bytes()
+            G = _xtr(eng, R, p)
+            assert eng.device_bytes() > before
+            err = np.zeros_like(G)
+        else:
+            G, err = eng.xtz(R)
+            assert np.all(err > 0.0)                                 # digits, not the FP64 sum
+    want = _exact(R, X, [0, 1, 77], [0, 1, 2, 129])
+    tol = 8.0 * n * 2.0 ** -64 * 16.0 * np.abs(R[[0, 1, 77]]).max(1)[:, None] * np.abs(X[:, [0, 1, 2, 129]]).max(0)
+    tol = tol + 2.0 ** -53 * np.abs(want) + err[np.ix_([0, 1, 77], [0, 1, 2, 129])]
+    assert np.all(np.abs(G[np.ix_([0, 1, 77], [0, 1, 2, 129])] - want) <= tol)
+
+
 @pytest.mark.parametrize("where", ["X", "R", "nan"])
 def test_rows_spread_over_many_binades_keep_fp64(where):
     """An outlier of 10^9 in a column of X, or in a row of R next to it, would cost the
