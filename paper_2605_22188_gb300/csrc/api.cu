@@ -102,8 +102,6 @@ struct kglm_ctx {
     void *Xop = nullptr, *Xop_lo = nullptr, *Xtop = nullptr, *Vop = nullptr, *Rop = nullptr;
     float *Xtop_lo = nullptr, *Vop_lo = nullptr, *Rop_lo = nullptr;   // low parts (FP32-accurate mode)
     TcMap mA1{}, mB1{}, mB1lo{}, mA2{}, mB2{}, mA1lo{}, mA2lo{}, mB2lo{};
-    TcMap gB1{}, gB2{};            // X and X^T maps at the bucketed tile widths of grouped launches
-    int gbn1 = 0, gbn2 = 0;
     // tiles by rule (pick_tiling) until kglm_configure or kglm_autotune sets them
     bool tiles_auto = true, pair_auto = true;
     std::map<std::pair<int, int>, Tiling> tilings;   // by (rows, product)
@@ -180,7 +178,8 @@ struct kglm_ctx {
     size_t off_kbar() const { return off_err() + 16; }
     size_t off_pf() const { return off_kbar() + 4 * pin_m; }
     size_t off_dq() const { return off_pf() + 4 * pin_m; }
-    size_t pin_bytes() const { return off_dq() + 128; }
+    size_t off_active() const { return off_dq() + 128; }
+    size_t pin_bytes() const { return off_active() + 4 * pin_m; }
     double sum_pa = 0.0;   // sum over the batch of p - |J0(b)|
     // per-phase device timers and launch counters
     struct Rec {
@@ -920,7 +919,7 @@ void run_iters(kglm_ctx* c, int count) {
 
 // The steps of one batch evaluation: the bound and iteration counters reset,
 // a certificate check after `it` iterations (bounds kept, finished nodes frozen,
-// the active flags copied to h asynchronously: the caller synchronises), and the
+// the active flags copied to pinned memory asynchronously: the caller synchronises), and the
 // final certificate, bound fold and re-optimization.
 void evaluate_begin(kglm_ctx* c, int iters) {
     const int m = c->m;
@@ -932,7 +931,7 @@ void evaluate_begin(kglm_ctx* c, int iters) {
     check_launch();
 }
 
-void evaluate_check(kglm_ctx* c, int it, std::vector<int>& h) {
+void evaluate_check(kglm_ctx* c, int it) {
     const int m = c->m;
     const double thr = c->ub_inc - delta_of(c, c->ub_inc);
     certify(c);
@@ -942,9 +941,16 @@ void evaluate_check(kglm_ctx* c, int it, std::vector<int>& h) {
                      1e-9);
         check_launch();
     }
-    h.resize(m);
     Scope sc(c, PH_COPY, 0, 4.0 * m);
-    CK(cudaMemcpyAsync(h.data(), c->active, sizeof(int) * m, cudaMemcpyDeviceToHost, c->st));
+    CK(cudaMemcpyAsync(c->pinned<int>(c->off_active()), c->active, sizeof(int) * m, cudaMemcpyDeviceToHost, c->st));
+}
+
+// After a synchronisation that follows evaluate_check: whether a node still iterates.
+bool any_active(kglm_ctx* c) {
+    const int* h = c->pinned<int>(c->off_active());
+    for (int b = 0; b < c->m; ++b)
+        if (h[b] != 0) return true;
+    return false;
 }
 
 void evaluate_end(kglm_ctx* c) {
@@ -982,17 +988,14 @@ void evaluate_end(kglm_ctx* c) {
 void evaluate_impl(kglm_ctx* c, int iters, int check_every) {
     Nvtx range("kglm evaluate: iterations, certificate, rounding, re-optimization");
     evaluate_begin(c, iters);
-    std::vector<int> h_active;
     for (int it = 0; it < iters;) {
         const int seg = check_every > 0 ? std::min(check_every, iters - it) : iters - it;
         run_iters(c, seg);
         it += seg;
         if (check_every > 0 && it % check_every == 0 && it < iters) {
-            evaluate_check(c, it, h_active);
+            evaluate_check(c, it);
             sync(c);
-            bool any = false;
-            for (int v : h_active) any |= (v != 0);
-            if (!any) break;
+            if (!any_active(c)) break;
         }
     }
     evaluate_end(c);
@@ -1000,63 +1003,73 @@ void evaluate_impl(kglm_ctx* c, int iters, int check_every) {
 
 // ---- several contexts' batches in shared launches (the serving loop)
 // BF16 contexts with single operands and p in the streaming prox's range take
-// part: per FISTA iteration one launch of S = X V + link and one of G = X^T R
-// for every (tile width, up to 8 contexts), and one streaming prox launch for
-// up to 8 contexts' nodes.  Each context keeps its own split-K (set from its
-// own shape) and node-level work, so its results do not depend on the others;
-// the tile width is bucketed from its own n and p.  Other contexts run their
-// iterations with their own launches in the same round.
+// part: per FISTA iteration one launch of S = X V + link, one of G = X^T R and one
+// streaming prox launch for up to 8 contexts' nodes.  Each context keeps its own
+// split-K (set from its own shape) and node-level work, so its results do not depend
+// on the others.  Other contexts run their iterations with their own launches in the
+// same round.
 bool groupable(const kglm_ctx* c) {
     return c->tc && c->tc_kind == 0 && !c->x3 && !c->xlo && c->p <= kStreamMaxP && c->m > 0;
 }
 
-int bucket_bn(int N) { return N >= 256 ? 256 : (N >= 128 ? 128 : 64); }
-
-void group_maps(kglm_ctx* c) {
-    const int b1 = bucket_bn(c->n), b2 = bucket_bn(c->p);
-    if (c->gbn1 == b1 && c->gbn2 == b2) return;
-    if (tc_make_map(&c->gB1, c->Xop, 1, c->n, c->p, c->pK, b1) ||
-        tc_make_map(&c->gB2, c->Xtop, 1, c->p, c->n, c->nK, b2))
-        throw Fail{KGLM_ECUDA, "cuTensorMapEncodeTiled failed for a grouped product"};
-    c->gbn1 = b1;
-    c->gbn2 = b2;
+// The column tile of a grouped product: the width whose units finish soonest on 152
+// workers (a K slice takes 0.48 us at any width, tiling_cost).  Any width gives the same
+// sums, and each context's split-K slices come from its own shape, so one launch carries
+// contexts of every size (a launch for each of three widths per product was 20 of
+// the 52 us of an iteration of six requests with one or two nodes each).
+int group_bn(const std::vector<TcGroupItem>& items) {
+    int best = 256;
+    double cost = 1e300;
+    for (int bn : {256, 192, 128, 96, 64}) {
+        long units = 0;
+        int kb = 0;
+        for (const TcGroupItem& it : items) {
+            const int mt = (it.M + 127) / 128, nkb = (it.K + 63) / 64;
+            int sp = 1;
+            if (it.max_splits > 0) {
+                const int alone = mt * ((it.N + it.splits_bn - 1) / it.splits_bn);
+                sp = std::max(1, std::min(it.max_splits, std::min((nkb + 3) / 4, std::max(1, 152 / std::max(1, alone)))));
+            }
+            units += (long)mt * ((it.N + bn - 1) / bn) * sp;
+            kb = std::max(kb, (nkb + sp - 1) / sp);
+        }
+        const double t = (double)((units + 151) / 152) * (0.5 + 0.48 * kb) + 2.5 * bn / 256.0;
+        if (t < 0.97 * cost) {
+            cost = t;
+            best = bn;
+        }
+    }
+    return best;
 }
 
 void iterate_group(const std::vector<kglm_ctx*>& A, int64_t* shared) {
     std::vector<kglm_ctx*> g;
     for (kglm_ctx* c : A) {
-        if (groupable(c)) {
-            group_maps(c);
-            g.push_back(c);
-        } else {
-            iterate(c);
-        }
+        if (groupable(c)) g.push_back(c);
+        else iterate(c);
     }
     if (g.empty()) return;
     cudaStream_t st = g[0]->st;
     std::vector<int> splits(g.size(), 1);
     for (int grad = 0; grad < 2; ++grad) {
-        std::vector<char> done(g.size(), 0);
-        for (size_t i = 0; i < g.size(); ++i) {
-            if (done[i]) continue;
-            const int bn = grad ? g[i]->gbn2 : g[i]->gbn1;
+        for (size_t i = 0; i < g.size(); i += kGroupMax) {
             std::vector<TcGroupItem> items;
             for (size_t j = i; j < g.size() && (int)items.size() < kGroupMax; ++j) {
-                if (done[j] || (grad ? g[j]->gbn2 : g[j]->gbn1) != bn) continue;
-                done[j] = 1;
                 kglm_ctx* c = g[j];
                 TcGroupItem it{};
                 it.M = c->m;
                 if (!grad) {
-                    it.A = &c->mA1; it.B = &c->gB1; it.N = c->n; it.K = c->p;
+                    it.A = &c->mA1; it.N = c->n; it.K = c->p;
                     it.out = c->Rop; it.ldo = c->nK; it.y = c->y32; it.loss = c->kind;
                 } else {
-                    it.A = &c->mA2; it.B = &c->gB2; it.N = c->p; it.K = c->n;
+                    it.A = &c->mA2; it.N = c->p; it.K = c->n;
                     it.pout = c->Gpart; it.pstride = (size_t)c->mcap * c->p; it.pld = c->p;
                     it.max_splits = c->gsplit_max; it.splits_bn = c->bn2; it.splits_used = &splits[j];
                 }
                 items.push_back(it);
             }
+            const int bn = group_bn(items);
+            for (size_t j = 0; j < items.size(); ++j) items[j].B = &b_map(g[i + j], grad ? 2 : 0, bn);
             Scope sc(g[i], grad ? PH_GEMM_GRAD : PH_GEMM_LINK, 1, 0.0);
             if (tc_gemm_group(st, items.data(), (int)items.size(), bn, grad ? TC_EPI_PARTIAL : TC_EPI_LINK_BF16,
                               g[i]->d_tcerr) != 0)
@@ -1080,8 +1093,44 @@ void iterate_group(const std::vector<kglm_ctx*>& A, int64_t* shared) {
     }
 }
 
+// f(c) for every context, side by side: each tensor-core context's work on its own
+// sub-stream, after everything on the shared stream and before what follows there.  The
+// certificates of a few nodes are chains of short launches that leave the GPU nearly
+// idle: of four requests one after another, 139 us each.
+template <typename F>
+void side_by_side(const std::vector<kglm_ctx*>& cs, F&& f) {
+    cudaStream_t st = cs[0]->st;
+    cudaEvent_t fork = nullptr;
+    if (cs.size() > 1)
+        for (kglm_ctx* c : cs)
+            if (!fork && c->tc) fork = c->ev_fork;
+    if (fork) CK(cudaEventRecord(fork, st));
+    try {
+        for (kglm_ctx* c : cs) {
+            if (!fork || !c->tc) {
+                f(c);
+                continue;
+            }
+            CK(cudaStreamWaitEvent(c->sub_st[0], fork, 0));
+            c->st = c->sub_st[0];
+            f(c);
+            c->st = st;
+            CK(cudaEventRecord(c->ev_join[0], c->sub_st[0]));
+            CK(cudaStreamWaitEvent(st, c->ev_join[0], 0));
+        }
+    } catch (...) {
+        // nothing of the contexts runs on after a failure, whatever the caller frees
+        for (kglm_ctx* c : cs) {
+            c->st = st;
+            if (fork && c->tc) cudaStreamSynchronize(c->sub_st[0]);
+        }
+        throw;
+    }
+}
+
 // evaluate_impl of every context (all on one stream), their iterations in shared
-// launches (*shared counts the launches that carried more than one context)
+// launches (*shared counts the launches that carried more than one context) and their
+// certificates side by side
 void evaluate_group(const std::vector<kglm_ctx*>& cs, int iters, int check_every, int64_t* shared) {
     Nvtx range("kglm evaluate (grouped contexts)");
     for (kglm_ctx* c : cs) {
@@ -1090,25 +1139,20 @@ void evaluate_group(const std::vector<kglm_ctx*>& cs, int iters, int check_every
     }
     for (kglm_ctx* c : cs) evaluate_begin(c, iters);
     std::vector<kglm_ctx*> A(cs);
-    std::vector<std::vector<int>> h;
     for (int it = 0; it < iters && !A.empty();) {
         const int seg = check_every > 0 ? std::min(check_every, iters - it) : iters - it;
         for (int i = 0; i < seg; ++i) iterate_group(A, shared);
         it += seg;
         if (check_every > 0 && it % check_every == 0 && it < iters) {
-            h.resize(A.size());
-            for (size_t i = 0; i < A.size(); ++i) evaluate_check(A[i], it, h[i]);
+            side_by_side(A, [&](kglm_ctx* c) { evaluate_check(c, it); });
             sync(A[0]);
             std::vector<kglm_ctx*> keep;
-            for (size_t i = 0; i < A.size(); ++i) {
-                bool any = false;
-                for (int v : h[i]) any |= (v != 0);
-                if (any) keep.push_back(A[i]);
-            }
+            for (kglm_ctx* c : A)
+                if (any_active(c)) keep.push_back(c);
             A.swap(keep);
         }
     }
-    for (kglm_ctx* c : cs) evaluate_end(c);
+    side_by_side(cs, [&](kglm_ctx* c) { evaluate_end(c); });
 }
 
 // After a synchronisation that follows evaluate_impl: the tensor-core error flag
