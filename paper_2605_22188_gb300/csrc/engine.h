@@ -48,6 +48,8 @@ void gemm_link_f64(cudaStream_t s, int m, int n, int p, const double* V, const d
 void gemm_link_f32(cudaStream_t s, int m, int n, int p, const float* V, const float* X,
                    const float* y, int kind, float* out, const GemmScratch* scr);
 
+// out[r] = sum_k A[r K + k] v[k] (FP64).
+void gemv_f64(cudaStream_t s, int rows, int K, const double* A, const double* v, double* out);
 // w = G v / ||v|| for the p x p FP64 Gram matrix; *norm = ||v||.
 void gram_power_step(cudaStream_t s, int p, const double* G, const double* v, double* w, double* norm);
 
