@@ -199,7 +199,7 @@ struct ProxArgs {
     const uint32_t* out_mask;
     const int* kbar;
     const int* pf;
-    double* tmom;         // FISTA t' per node
+    double* tmom;         // FISTA momentum state per node (momentum.cuh)
     const int* active;    // 1 = iterate this node
     double eta, c, M;     // step, c = 2 eta lambda2 = 1/rho, box
     int restart;

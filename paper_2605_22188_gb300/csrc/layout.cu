@@ -258,7 +258,7 @@ int layout_warm(cudaStream_t s, int m, int p, int W, int is_f64, const int* slot
         k_warm<float><<<blocks(n, 256), 256, 0, s>>>(m, p, W, slot, nslots, (const float*)pool, warmB, out_mask,
                                                      (float*)B, (float*)V, Vop, Vop_lo, op_ld, op_bf16);
     // t_1 = 1 (Beck and Teboulle): the first extrapolation, after x_1, takes no momentum
-    k_node_init<<<blocks(m, 256), 256, 0, s>>>(m, 1.0, tmom, active, hint);
+    k_node_init<<<blocks(m, 256), 256, 0, s>>>(m, -0.0, tmom, active, hint);   // momentum.cuh: no step yet
     return 2;
 }
 

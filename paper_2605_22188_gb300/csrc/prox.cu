@@ -32,6 +32,7 @@
 
 #include "common.cuh"
 #include "engine.h"
+#include "momentum.cuh"
 
 namespace kglm {
 namespace {
@@ -109,7 +110,9 @@ __device__ __forceinline__ void prox_node(const ProxArgs& a) {
     // them after it: holding them across the gradient loads costs registers, and
     // registers bound how many node CTAs an SM holds).
     constexpr bool EARLY = std::is_same<Grp, WarpGroup>::value;
-    const double tprev = (EARLY && G::rank() == 0) ? a.tmom[b] : 0.0;
+    T c_keep = T(0);
+    double t_keep = 0.0;
+    if (EARLY) t_keep = mom_next(a.tmom[b], c_keep);
     auto load_node = [&](int e) {
         const int j = G::rank() + e * NT;
         if constexpr (HOLD) vv[e] = bo[e] = T(0);
@@ -179,18 +182,11 @@ __device__ __forceinline__ void prox_node(const ProxArgs& a) {
         }
     }
     const Mk ffree = valid & ~fin & ~fout;
-    // FISTA t update (FP64; tmom holds t_k of the iterate x_k this step makes,
-    // t_1 = 1): without a restart t_{k+1} = (1 + sqrt(1 + 4 t_k^2)) / 2 and
+    // FISTA t update (tmom holds the state of t_k of the iterate x_k this step makes,
+    // t_1 = 1, momentum.cuh): without a restart t_{k+1} = (1 + sqrt(1 + 4 t_k^2)) / 2 and
     // v_{k+1} = x_k + ((t_k - 1) / t_{k+1}) (x_k - x_{k-1}); a restart starts over
     // from x_k (v_{k+1} = x_k, t_{k+1} = 1, so the next coefficient is 0 too).
-    // The test picks one at the end; a warp per node computes the candidates
-    // here, off the end of its critical path.
-    double t_keep = 0.0, c_keep = 0.0;
-    auto t_candidates = [&](double tp) {
-        t_keep = 0.5 * (1.0 + sqrt(1.0 + 4.0 * tp * tp));
-        c_keep = (tp - 1.0) / t_keep;
-    };
-    if (EARLY && G::rank() == 0) t_candidates(tprev);
+    // The test picks one at the end.
     const int kb = a.kbar[b], pf = a.pf[b];
 
     T theta = T(0);
@@ -352,11 +348,11 @@ __device__ __forceinline__ void prox_node(const ProxArgs& a) {
         dot[0] += (ve - bv) * (bv - be);
     }
     G::template sum<1, T>(dot, sh.red);
-    if (G::rank() == 0) {                  // FISTA t update, once per node, in FP64
-        if constexpr (!EARLY) t_candidates(a.tmom[b]);
+    if (G::rank() == 0) {                  // FISTA t update, once per node
+        if constexpr (!EARLY) t_keep = mom_next(a.tmom[b], c_keep);
         const bool rs = a.restart && dot[0] > T(0);
-        sh.coef = rs ? T(0) : T(c_keep);
-        a.tmom[b] = rs ? 1.0 : t_keep;      // restart: start over from this iterate, t = 1
+        sh.coef = rs ? T(0) : c_keep;
+        a.tmom[b] = rs ? mom_start() : t_keep;   // restart: start over from this iterate, t = 1
     }
     G::sync();
     const T coef = sh.coef;

@@ -56,6 +56,7 @@
 
 #include "common.cuh"
 #include "engine.h"
+#include "momentum.cuh"
 
 namespace kglm {
 namespace {
@@ -282,22 +283,15 @@ __device__ __forceinline__ void stream_node(const ProxArgs& a, int b, int lane, 
         float* __restrict__ V = static_cast<float*>(a.V) + base;
         float* __restrict__ Bm = static_cast<float*>(a.B) + base;
         const int kb = a.kbar[b], pf = a.pf[b];
-        const double tprev = lane == 0 ? a.tmom[b] : 0.0;
+        // the momentum's state and coefficient, from the table (momentum.cuh)
+        float coef;
+        const double t_keep = mom_next(a.tmom[b], coef);
         const bool sel = kb > 0 && pf > kb;         // a top set to select and a block to pool
         float tau_h = 0.f, th_h = 0.f;
         if (a.hint != nullptr && sel) { tau_h = a.hint[2 * b]; th_h = a.hint[2 * b + 1]; }
         const float tg = tau_h > 0.f ? tau_h * kTauHint : __builtin_huge_valf();
 
         if (lane == 0) { h.nj1 = 0; h.ncand = 0; }
-        // the momentum's FP64 root and quotient (a chain of some fifty operations on a pipe
-        // that takes one in 16 cycles) run while the rows arrive, not at the end
-        double t_keep = 0.0;
-        float coef = 0.f;
-        if (lane == 0) {
-            t_keep = 0.5 * (1.0 + sqrt(1.0 + 4.0 * tprev * tprev));
-            coef = (float)((tprev - 1.0) / t_keep);
-        }
-        coef = __shfl_sync(0xffffffffu, coef, 0);
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncwarp();
         if (!summed && a.gsplits > 1) stream_sum<VEC>(a, base, lane, su);
@@ -582,7 +576,7 @@ __device__ __forceinline__ void stream_node(const ProxArgs& a, int b, int lane, 
         const float dot = warp_sum(d0 + d1);
         const bool rs = a.restart && dot > 0.f;
         if (lane == 0) {
-            a.tmom[b] = rs ? 1.0 : t_keep;   // restart: start over from beta, t = 1
+            a.tmom[b] = rs ? mom_start() : t_keep;   // restart: start over from beta, t = 1
             if (a.hint != nullptr) {
                 a.hint[2 * b] = sel ? h.sv[kb - 1] : 0.f;
                 a.hint[2 * b + 1] = sel ? theta : 0.f;
