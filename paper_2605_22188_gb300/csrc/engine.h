@@ -307,6 +307,9 @@ int layout_masks(cudaStream_t s, int m, int p, int W, int k, const int* in_ptr, 
 int layout_validate(cudaStream_t s, int m, int k, int W, int nnz_in, int nnz_out, const int* in_ptr,
                     const int* out_ptr, const uint32_t* in_mask, const uint32_t* out_mask, const int* slot,
                     int nslots, int* err);
+// Index checks of a batch's CSR lists (device arrays, counts checked before): bits 1, 2 of *err.
+void layout_check(cudaStream_t s, int m, int p, int W, const int* in_ptr, const int* in_idx, const int* out_ptr,
+                  const int* out_idx, int* err);
 int layout_warm(cudaStream_t s, int m, int p, int W, int is_f64, const int* slot, int nslots, const void* pool,
                 const double* warmB, const uint32_t* out_mask, void* B, void* V, void* Vop, float* Vop_lo, int op_ld,
                 int op_bf16, double* tmom, int* active, float* hint);

@@ -69,6 +69,33 @@ __global__ void k_check_slots(int m, const int* slot, int nslots, int* err) {
     if (b < m && (slot[b] < -1 || slot[b] >= nslots)) atomicOr(err, 4);
 }
 
+// The index checks of a pushed batch, a warp per node with its coordinates' bits in shared
+// memory: bit 1 of *err for an index outside [0, p), bit 2 for a repeat within J1 or J0 or
+// between them.  (The counts are checked on the host.)
+constexpr int kCheckWarps = 8;
+__global__ __launch_bounds__(32 * kCheckWarps) void k_check_nodes(int m, int p, int W, const int* __restrict__ in_ptr,
+                                                                  const int* __restrict__ in_idx,
+                                                                  const int* __restrict__ out_ptr,
+                                                                  const int* __restrict__ out_idx, int* err) {
+    extern __shared__ uint32_t bits[];
+    const int lane = threadIdx.x & 31, b = blockIdx.x * kCheckWarps + (threadIdx.x >> 5);
+    uint32_t* mine = bits + (size_t)(threadIdx.x >> 5) * W;
+    if (b >= m) return;
+    for (int w = lane; w < W; w += 32) mine[w] = 0u;
+    __syncwarp();
+    int bad = 0;
+    for (int part = 0; part < 2; ++part) {
+        const int* idx = part ? out_idx : in_idx;
+        const int t1 = part ? out_ptr[b + 1] : in_ptr[b + 1];
+        for (int t = (part ? out_ptr[b] : in_ptr[b]) + lane; t < t1; t += 32) {
+            const int j = idx[t];
+            if (j < 0 || j >= p) bad |= 1;
+            else if (atomicOr(&mine[j >> 5], 1u << (j & 31)) & (1u << (j & 31))) bad |= 2;
+        }
+    }
+    if (bad) atomicOr(err, bad);
+}
+
 __global__ void k_counts(int m, int p, int k, const int* in_ptr, const int* out_ptr, int* kbar, int* pf) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= m) return;
@@ -245,6 +272,12 @@ int layout_validate(cudaStream_t s, int m, int k, int W, int nnz_in, int nnz_out
     k_validate<<<blocks(m, 128), 128, 0, s>>>(m, k, W, nnz_in, nnz_out, in_ptr, out_ptr, in_mask, out_mask, err);
     if (slot) k_check_slots<<<blocks(m, 256), 256, 0, s>>>(m, slot, nslots, err);
     return slot ? 2 : 1;
+}
+
+void layout_check(cudaStream_t s, int m, int p, int W, const int* in_ptr, const int* in_idx, const int* out_ptr,
+                  const int* out_idx, int* err) {
+    k_check_nodes<<<blocks(m, kCheckWarps), 32 * kCheckWarps, kCheckWarps * W * sizeof(uint32_t), s>>>(
+        m, p, W, in_ptr, in_idx, out_ptr, out_idx, err);
 }
 
 int layout_warm(cudaStream_t s, int m, int p, int W, int is_f64, const int* slot, int nslots, const void* pool,
