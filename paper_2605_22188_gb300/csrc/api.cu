@@ -102,9 +102,13 @@ struct kglm_ctx {
     void *Xop = nullptr, *Xop_lo = nullptr, *Xtop = nullptr, *Vop = nullptr, *Rop = nullptr;
     float *Xtop_lo = nullptr, *Vop_lo = nullptr, *Rop_lo = nullptr;   // low parts (FP32-accurate mode)
     TcMap mA1{}, mB1{}, mB1lo{}, mA2{}, mB2{}, mA1lo{}, mA2lo{}, mB2lo{};
+    // rows of the iterations and checks when the finished nodes of a batch have left them
+    // (0: every node): row r is node d_slots[r]
+    int mrun = 0;
+    int rows() const { return mrun > 0 ? mrun : m; }
     // tiles by rule (pick_tiling) until kglm_configure or kglm_autotune sets them
     bool tiles_auto = true, pair_auto = true;
-    std::map<std::pair<int, int>, Tiling> tilings;   // by (rows, product)
+    std::map<std::tuple<int, int, int>, Tiling> tilings;   // by (rows, rows of the batch, product)
     std::map<std::pair<int, int>, TcMap> bmaps;      // B operands' maps by (operand, tile width)
     // FP32-accurate mode: beta as a TF32 hi + lo operand for the certificate's X beta
     float *Bop = nullptr, *Bop_lo = nullptr;
@@ -136,8 +140,7 @@ struct kglm_ctx {
     double *xsig = nullptr, *ztau = nullptr, *Qerr = nullptr;
     int* Qi = nullptr;
     size_t qi_slices = 0;         // integer slices of mcap x p
-    SplitPlan pC{};               // jobs of the certificate product at batch size mC
-    int mC = -1;
+    std::map<int, SplitPlan> pC;  // jobs of the certificate product by its rows
     TcMap mAz{}, mBx{};
     int bnx = 0;
     int gsplit_max = 4;
@@ -595,10 +598,13 @@ void xtzeta(kglm_ctx* c, int m, CertArgs& a) {
     if (a.DZ == nullptr) exact_digits(c->st, c->zeta, m, n, (size_t)n, x.npad, 1, c->DZ, c->ztau);
     // the levels in pieces that keep every SM busy (at one node of n = 5000, p = 1000, 28 whole
     // levels on 68 of them took 120 us, now 40 with its integers zeroed)
-    digit_product(c, m, p, n, kCertDigits, c->bnx, c->mAz, c->mBx, c->Qi, c->pC, c->mC);
+    if (c->pC.size() >= 64) c->pC.clear();
+    SplitPlan& pl = c->pC[m];
+    int have = pl.njobs > 0 ? m : -1;
+    digit_product(c, m, p, n, kCertDigits, c->bnx, c->mAz, c->mBx, c->Qi, pl, have);
     a.Qi = c->Qi;
     a.qi_stride = (size_t)m * p;
-    a.qi_parts = c->pC.parts;
+    a.qi_parts = pl.parts;
     a.xsig = c->xsig;
     a.ztau = c->ztau;
     a.ebound = x.ebound;
@@ -636,13 +642,15 @@ Tiling pick_tiling(kglm_ctx* c, int M, int which) {
     const bool grad = which == TILE_GRAD, cert = which == TILE_CERT;
     const int def = grad ? c->bn2 : cert && c->tc_kind == 0 ? c->bnc : c->bn1;
     if (!c->tiles_auto) return {def, cert ? false : c->pair, 0};
-    const auto key = std::make_pair(M, which);
+    // the batch whose rows these are sets the split-K (fewer rows once finished nodes left)
+    const int Mb = c->mrun > 0 && M == c->mrun ? c->m : M;
+    const auto key = std::make_tuple(M, Mb, which);
     const auto it = c->tilings.find(key);
     if (it != c->tilings.end()) return it->second;
     const int N = grad ? c->p : c->n, K = grad ? c->n : c->p, ke = c->tc_kind == 0 && !cert ? 64 : 32;
     const int nkb = (K + ke - 1) / ke, mt = (M + 127) / 128;
     const int na = c->x3 || cert ? 2 : 1, nb = grad ? (c->x3 ? 2 : 1) : (c->xlo || cert ? 2 : 1);
-    const int tiles = mt * ((N + def - 1) / def);
+    const int tiles = ((Mb + 127) / 128) * ((N + def - 1) / def);
     // the default's split-K (tc_gemm)
     int splits = grad ? std::max(1, std::min(c->gsplit_max, std::min((nkb + 3) / 4, std::max(1, 152 / tiles))))
                       : (tiles < 152 ? std::min((nkb + 3) / 4, std::max(1, 152 / tiles)) : 1);
@@ -659,8 +667,6 @@ Tiling pick_tiling(kglm_ctx* c, int M, int which) {
                     best = {bn, pr != 0, splits};
                 }
             }
-    } else {
-        best.splits = 0;                                // a split link product keeps its launcher's plan
     }
     if (c->tilings.size() >= 256) c->tilings.clear();
     c->tilings[key] = best;
@@ -690,9 +696,11 @@ const TcMap& b_map(kglm_ctx* c, int which, int bn) {
 
 void certify(kglm_ctx* c) {
     Nvtx range("certificate");
-    const int m = c->m, n = c->n, p = c->p;
+    const int m = c->rows(), n = c->n, p = c->p;
     CertArgs a{};
+    a.rowmap = c->mrun > 0 ? c->d_slots : nullptr;
     a.m = m; a.n = n; a.p = p; a.W = c->W; a.k = c->k; a.kind = c->kind;
+    a.m_batch = c->m;
     a.lam2 = c->lam2; a.M = c->M;
     a.S = c->R;                                         // the m x n buffer is free here
     a.s_is_f64 = c->f64;
@@ -718,7 +726,8 @@ void certify(kglm_ctx* c) {
             // tensor-core modes: X beta as the TF32 hi + lo split (hi hi + hi lo + lo hi,
             // FP32 accumulate; FP32-accurate), with the TF32 modes' own X hi + lo operands
             // and, in the BF16 mode, the TF32 copies of X kept for this product
-            convert_pad_f32(c->st, (const float*)c->B, m, p, c->Bop, c->pK, 0, c->Bop_lo);
+            if (c->mrun > 0) gather_operand(c->st, m, p, c->d_slots, (const float*)c->B, c->Bop, c->Bop_lo, c->pK, 0);
+            else convert_pad_f32(c->st, (const float*)c->B, m, p, c->Bop, c->pK, 0, c->Bop_lo);
             check_launch();
             const bool own = c->tc_kind == 0;
             const Tiling t = pick_tiling(c, m, TILE_CERT);
@@ -726,6 +735,7 @@ void certify(kglm_ctx* c) {
             g.kind = 1; g.M = m; g.N = n; g.K = p; g.bn = t.bn;
             g.epi = TC_EPI_STORE_F32; g.out = c->R; g.ldo = n; g.err = c->d_tcerr;
             g.A2 = &c->mAblo;
+            g.splits = t.splits;
             if (tc_gemm(c->st, c->mAb, b_map(c, own ? 4 : 0, t.bn), &b_map(c, own ? 5 : 1, t.bn), g,
                         t.splits == 1 ? nullptr : &c->gtc) != 0)
                 throw Fail{KGLM_ECUDA, "tensor-core launch failed (certificate X beta)"};
@@ -784,6 +794,7 @@ ProxArgs prox_args_rows(kglm_ctx* c, int row0, int mr, int splits, bool pdl) {
     a.in_mask = c->in_mask + (size_t)row0 * c->W; a.out_mask = c->out_mask + (size_t)row0 * c->W;
     a.kbar = c->kbar + row0; a.pf = c->pf + row0;
     a.tmom = c->tmom + row0; a.active = c->active + row0;
+    a.rowmap = c->mrun > 0 ? c->d_slots : nullptr;
     a.hint = c->phint + 2 * (size_t)row0;
     a.eta = c->eta; a.c = c->c; a.M = c->M; a.restart = c->d.restart;
     a.pdl = pdl ? 1 : 0;
@@ -808,6 +819,7 @@ void iterate_rows(kglm_ctx* c, cudaStream_t st, int row0, int mr, bool sub) {
         const Tiling t = pick_tiling(c, mr, TILE_LINK);
         g.kind = c->tc_kind; g.M = mr; g.N = n; g.K = p; g.bn = t.bn;
         g.arow0 = row0;
+        g.splits = t.splits;
         g.epi = c->tc_kind == 0 ? TC_EPI_LINK_BF16 : TC_EPI_LINK_F32;
         g.out = static_cast<char*>(c->Rop) + (size_t)row0 * c->nK * es;
         g.ldo = c->nK; g.y = c->y32; g.loss = c->kind; g.err = c->d_tcerr;
@@ -847,7 +859,7 @@ void iterate(kglm_ctx* c) {
     const int m = c->m, n = c->n, p = c->p;
     const double flops = 2.0 * n * c->sum_pa;
     if (c->tc) {
-        iterate_rows(c, c->st, 0, m, false);
+        iterate_rows(c, c->st, 0, c->rows(), false);
         return;
     }
     if (split_on(c, m)) {
@@ -894,7 +906,7 @@ void iterate(kglm_ctx* c) {
 // Sub-batches of the current batch: rows split into nsub parts (multiples of
 // 128 rows but the last), at most one per 128 rows.
 int sub_count(const kglm_ctx* c) {
-    if (!c->tc || c->stats_on || c->nsub <= 1) return 1;
+    if (!c->tc || c->stats_on || c->nsub <= 1 || c->mrun > 0) return 1;
     return std::max(1, std::min(c->nsub, c->m / 128));
 }
 
@@ -933,8 +945,10 @@ void destroy_graphs(kglm_ctx* c) {
 // captured on first use (kernel arguments depend only on the batch size).
 void run_iters(kglm_ctx* c, int count) {
     if (count <= 0) return;
-    if (c->st == nullptr || c->st == cudaStreamLegacy || c->st == cudaStreamPerThread) {
-        for (int i = 0; i < count; ++i) iterate(c);   // the legacy streams cannot be captured
+    if (c->st == nullptr || c->st == cudaStreamLegacy || c->st == cudaStreamPerThread || c->mrun > 0) {
+        // the legacy streams cannot be captured; a batch whose finished nodes left has a row
+        // count of its own for these few iterations
+        for (int i = 0; i < count; ++i) iterate(c);
         return;
     }
     const auto key = std::make_tuple(c->m, count, c->stats_on ? 1 : 0, sub_count(c));
@@ -982,11 +996,20 @@ void run_iters(kglm_ctx* c, int count) {
     }
 }
 
+// Every node of the batch in the iterations' and checks' rows again.
+void whole_batch(kglm_ctx* c) {
+    if (c->mrun == 0) return;
+    c->mrun = 0;
+    gather_operand(c->st, c->m, c->p, nullptr, (const float*)c->V, c->Vop, c->Vop_lo, c->pK, c->tc_kind == 0);
+    check_launch();
+}
+
 // The steps of one batch evaluation: the bound and iteration counters reset,
 // a certificate check after `it` iterations (bounds kept, finished nodes frozen,
 // the active flags copied to pinned memory asynchronously: the caller synchronises), and the
 // final certificate, bound fold and re-optimization.
 void evaluate_begin(kglm_ctx* c, int iters) {
+    whole_batch(c);                                     // (an evaluation before this one may have failed)
     const int m = c->m;
     if (split_pays(c, m)) split_setup(c);              // before any capture of this batch's iterations
     const unsigned gb = (unsigned)((m + 255) / 256);
@@ -1010,15 +1033,41 @@ void evaluate_check(kglm_ctx* c, int it) {
     CK(cudaMemcpyAsync(c->pinned<int>(c->off_active()), c->active, sizeof(int) * m, cudaMemcpyDeviceToHost, c->st));
 }
 
-// After a synchronisation that follows evaluate_check: whether a node still iterates.
+// After a synchronisation that follows evaluate_check: whether a node still iterates.  Most
+// nodes of a search finish at their first check (a batch's bounds pass the incumbent, or
+// its gaps close), and the few that remain would carry the others' rows through every
+// product.  They leave the iterations and the checks where that takes at least a quarter of
+// the products' 128-row tiles (a product of 12 rows costs as much as one of 64: there the
+// captured iterations of the whole batch are the faster, 4.5 ms against 4.8 for 64 nodes,
+// n = 1373, p = 611), and from then on wherever a quarter of the rows left goes.  A search
+// of 2400 batches' nodes (n = 5000, p = 1000, 7 % of them unfinished after a check): 108.7
+// -> 100.5 ms.  Only the operand and gradient rows move (row r is node d_slots[r]); a
+// node's own arrays, its sums over K (the split-K slices stay the batch's) and so its bits
+// do not.  (Tiles or sub-batches chosen by the caller tie the split to the rows: those keep
+// every row.)  The last certificate takes the whole batch again.
 bool any_active(kglm_ctx* c) {
     const int* h = c->pinned<int>(c->off_active());
-    for (int b = 0; b < c->m; ++b)
-        if (h[b] != 0) return true;
-    return false;
+    int left = 0;
+    for (int b = 0; b < c->m; ++b) left += h[b] != 0;
+    if (left == 0) return false;
+    const int rows = left <= 16 ? 16 : left <= 128 ? (left + 31) / 32 * 32 : (left + 127) / 128 * 128;
+    const bool fewer = c->mrun > 0 ? 4 * rows <= 3 * c->mrun : 4 * ((rows + 127) / 128) <= 3 * ((c->m + 127) / 128);
+    if (c->tc && c->cexact && c->tiles_auto && c->nsub <= 1 && fewer) {
+        int* map = c->pinned<int>(c->off_kbar());           // free during an evaluation
+        int r = 0;
+        for (int b = 0; b < c->m; ++b)
+            if (h[b] != 0) map[r++] = b;
+        while (r < rows) map[r++] = -1;
+        CK(cudaMemcpyAsync(c->d_slots, map, sizeof(int) * rows, cudaMemcpyHostToDevice, c->st));
+        gather_operand(c->st, rows, c->p, c->d_slots, (const float*)c->V, c->Vop, c->Vop_lo, c->pK, c->tc_kind == 0);
+        check_launch();
+        c->mrun = rows;
+    }
+    return true;
 }
 
 void evaluate_end(kglm_ctx* c) {
+    whole_batch(c);
     const int m = c->m;
     const unsigned gb = (unsigned)((m + 255) / 256);
     certify(c);
@@ -1092,7 +1141,7 @@ int group_bn(const std::vector<TcGroupItem>& items) {
             const int mt = (it.M + 127) / 128, nkb = (it.K + 63) / 64;
             int sp = 1;
             if (it.max_splits > 0) {
-                const int alone = mt * ((it.N + it.splits_bn - 1) / it.splits_bn);
+                const int alone = ((it.M_split + 127) / 128) * ((it.N + it.splits_bn - 1) / it.splits_bn);
                 sp = std::max(1, std::min(it.max_splits, std::min((nkb + 3) / 4, std::max(1, 152 / std::max(1, alone)))));
             }
             units += (long)mt * ((it.N + bn - 1) / bn) * sp;
@@ -1122,7 +1171,8 @@ void iterate_group(const std::vector<kglm_ctx*>& A, int64_t* shared) {
             for (size_t j = i; j < g.size() && (int)items.size() < kGroupMax; ++j) {
                 kglm_ctx* c = g[j];
                 TcGroupItem it{};
-                it.M = c->m;
+                it.M = c->rows();
+                it.M_split = c->m;
                 if (!grad) {
                     it.A = &c->mA1; it.N = c->n; it.K = c->p;
                     it.out = c->Rop; it.ldo = c->nK; it.y = c->y32; it.loss = c->kind;
@@ -1146,7 +1196,7 @@ void iterate_group(const std::vector<kglm_ctx*>& A, int64_t* shared) {
     for (size_t i0 = 0; i0 < g.size(); i0 += kGroupMax) {
         ProxGroup pg{};
         pg.np = (int)std::min<size_t>(kGroupMax, g.size() - i0);
-        for (int t = 0; t < pg.np; ++t) pg.a[t] = prox_args_rows(g[i0 + t], 0, g[i0 + t]->m, splits[i0 + t], false);
+        for (int t = 0; t < pg.np; ++t) pg.a[t] = prox_args_rows(g[i0 + t], 0, g[i0 + t]->rows(), splits[i0 + t], false);
         Scope sc(g[i0], PH_PROX, 1, 0.0);
         const int rc = prox_stream_group(st, pg);
         if (rc < 0) throw Fail{KGLM_ECUDA, "prox kernel: shared memory attribute refused"};

@@ -401,9 +401,11 @@ __global__ __launch_bounds__(NT) void k_cert_node(const __grid_constant__ CertAr
     using K = unsigned long long;
     constexpr int NW = NT / 32;
     __shared__ CertNodeShared sh;
-    const int b = blockIdx.x, p = a.p, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const size_t base = (size_t)b * p;
-    const double M = a.M, inv2l = 1.0 / (2.0 * a.lam2), ztau = a.ztau[b];
+    const int row = blockIdx.x, b = a.rowmap ? a.rowmap[row] : row;
+    if (b < 0) return;
+    const int p = a.p, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const size_t base = (size_t)b * p, qbase = (size_t)row * p;
+    const double M = a.M, inv2l = 1.0 / (2.0 * a.lam2), ztau = a.ztau[row];
     const double mth = M * (1.0 + kFeasRtol);
     const float mth_f = __double2float_rd(mth);                // |b| > mth  <=>  |b| > mth_f for FP32 b
     const uint32_t* im = a.in_mask + (size_t)b * a.W;
@@ -430,7 +432,7 @@ __global__ __launch_bounds__(NT) void k_cert_node(const __grid_constant__ CertAr
             continue;
         }
         double err;
-        const double qv = exact_q(a.Qi, a.qi_stride, base + j, a.qi_parts, a.xsig[j] * ztau, a.ebound, &err);
+        const double qv = exact_q(a.Qi, a.qi_stride, qbase + j, a.qi_parts, a.xsig[j] * ztau, a.ebound, &err);
         // |X^T zeta| bounded from above: |Q~| + its distance bound (H_M, TopSum increase in |q|)
         const double v = (fabs(qv) + err) * inv2l;
         if (in) {
@@ -519,7 +521,7 @@ __global__ __launch_bounds__(NT) void k_cert_node(const __grid_constant__ CertAr
         hj1 = warp_sum(hj1);
         bj1 = warp_sum(bj1);
         if (lane == 0) {
-            a.lb[b] = -a.sum_conj[b] - 2.0 * a.lam2 * (hj1 + part);
+            a.lb[b] = -a.sum_conj[row] - 2.0 * a.lam2 * (hj1 + part);
             sh.vj1[0] = bj1;                                   // (the J1 values are spent)
         }
         __syncwarp();
@@ -581,7 +583,7 @@ __global__ __launch_bounds__(NT) void k_cert_node(const __grid_constant__ CertAr
             gf = 0.5 * (presq + tail / (kb - s) * tail);
         }
         const double g = 0.5 * sh.vj1[0] + gf;
-        a.primal[b] = isinf(g) ? INFINITY : a.sum_loss[b] + 2.0 * a.lam2 * g;
+        a.primal[b] = isinf(g) ? INFINITY : a.sum_loss[row] + 2.0 * a.lam2 * g;
         a.jstar[b] = leaf ? -1 : sh.si[0];
     }
 }
@@ -593,7 +595,7 @@ void cert_dual_point(cudaStream_t s, const CertArgs& a) {
     if (a.s_is_f64) k_dual_point<256><<<a.m, 256, 0, s>>>(a);
     else {
         int parts = 1;
-        while (parts < 8 && (long)a.m * parts < 2 * 152 && a.n / parts >= 1024) parts *= 2;
+        while (parts < 8 && (long)a.m_batch * parts < 2 * 152 && a.n / parts >= 1024) parts *= 2;
         const int seg = ((a.n + parts - 1) / parts + 3) / 4 * 4;
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3((unsigned)a.m * parts);

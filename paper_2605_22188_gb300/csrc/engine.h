@@ -79,7 +79,7 @@ struct TcGemm {
     size_t pstride;
     int pld;
     int max_splits;  // TC_EPI_PARTIAL: upper bound on the number of slices
-    int splits;      // TC_EPI_PARTIAL: that many slices instead (0: enough units to fill the SMs)
+    int splits;      // that many split-K slices instead (0: enough units to fill the SMs)
     int* splits_used;
     const TcMap* A2; // TF32 low part of A (out = (A + A2)(B + B2)^T less A2 B2^T); needs kind 1 and B2
     float* out_lo;   // TC_EPI_LINK_F32: TF32 low part of each output (NULL: none)
@@ -177,7 +177,7 @@ struct TcGroupItem {
     size_t pstride;
     int pld;
     int max_splits;
-    int splits_bn;
+    int splits_bn, M_split;   // (the rows that set the split, 0: M)
     int* splits_used;
 };
 // Up to 8 problems in one persistent launch of tile width bn, epi TC_EPI_LINK_BF16 or TC_EPI_PARTIAL.
@@ -185,6 +185,7 @@ int tc_gemm_group(cudaStream_t s, const TcGroupItem* items, int np, int bn, int 
 
 struct ProxArgs {
     int m, p, W;
+    const int* rowmap;    // NULL, or the node of each row of Gpart and Vop (-1: none); the other arrays are by node
     const void* G;        // gradient X^T R, node-major m x p (working type)
     const float* Gpart;   // or: gsplits FP32 slices of it, slice s at Gpart + s*gstride (summed in order)
     int gsplits;
@@ -252,6 +253,8 @@ struct CertArgs {
     const double* Q;      // X^T zeta (m x p) FP64
     const void* B;        // beta (m x p) working type
     int b_is_f64;
+    const int* rowmap;    // NULL, or the node of each row (-1: none): S, zeta, the sums, ztau and Qi are by row
+    int m_batch;          // the batch's nodes: they set how a node's sums are split, however many rows remain
     const uint32_t* in_mask;
     const uint32_t* out_mask;
     const int* kbar;
@@ -321,6 +324,9 @@ void convert_pad(cudaStream_t s, const double* in, int rows, int cols, int ld_in
 // (with lo != NULL, TF32 only: also the low parts)
 void convert_pad_f32(cudaStream_t s, const float* in, int rows, int cols, void* out, int ld_out, int to_bf16,
                      float* lo = nullptr);
+// Rows map[r] (r < rows; -1: left alone; NULL: r) of src (stride cols, FP32) as operand rows r.
+void gather_operand(cudaStream_t s, int rows, int cols, const int* map, const float* src, void* out, float* lo, int ld_out,
+                    int to_bf16);
 void pool_store(cudaStream_t s, int count, int p, int is_f64, const int* rows, const int* slots,
                 const void* B, void* pool);
 // a8: pruned[b] = lb[b] >= thr ; alive[b] &= !pruned

@@ -1185,7 +1185,7 @@ int tc_gemm(cudaStream_t s, const TcMap& A, const TcMap& B, const TcMap* B2, con
         splits = g.splits > 0 ? g.splits
                               : std::max(1, std::min(g.max_splits, std::min((a.nkb + 3) / 4, std::max(1, SMS / tiles))));
     } else if (tiles < SMS && scr && scr->part && scr->counters && scr->n_counters >= 8 * tiles) {
-        splits = std::min((a.nkb + 3) / 4, std::max(1, SMS / tiles));
+        splits = g.splits > 0 ? g.splits : std::min((a.nkb + 3) / 4, std::max(1, SMS / tiles));
         const size_t need = (size_t)splits * tiles * BM * MAXBN * sizeof(float);
         if (need > scr->part_bytes) splits = (int)std::max<size_t>(1, scr->part_bytes / ((size_t)tiles * BM * MAXBN * sizeof(float)));
     }
@@ -1294,7 +1294,8 @@ int tc_gemm_group(cudaStream_t s, const TcGroupItem* items, int np, int bn, int 
         // own width, so that its slices do not depend on the other problems
         int splits = 1;
         if (epi == TC_EPI_PARTIAL && q.M > 0) {
-            const int tiles_alone = q.mt * ((it.N + it.splits_bn - 1) / it.splits_bn);
+            const int mt_alone = it.M_split > 0 ? (it.M_split + BM - 1) / BM : q.mt;
+            const int tiles_alone = mt_alone * ((it.N + it.splits_bn - 1) / it.splits_bn);
             splits = std::max(1, std::min(it.max_splits, std::min((q.nkb + 3) / 4, std::max(1, SMS / tiles_alone))));
         }
         q.kb_per_split = (q.nkb + splits - 1) / splits;

@@ -181,6 +181,14 @@ __global__ __launch_bounds__(256) void k_convert_pad_f32(const float* __restrict
     }
 }
 
+__global__ __launch_bounds__(256) void k_gather_operand(int cols, const int* __restrict__ map,
+                                                        const float* __restrict__ src, void* out, float* lo, int ld_out,
+                                                        int to_bf16) {
+    const int r = blockIdx.y, b = map ? map[r] : r, c = blockIdx.x * 256 + threadIdx.x;
+    if (b < 0 || c >= cols) return;
+    store_operand2(out, lo, (size_t)r * ld_out + c, src[(size_t)b * cols + c], to_bf16);
+}
+
 __global__ void k_node_init(int m, double t0, double* tmom, int* active, float* hint) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= m) return;
@@ -306,6 +314,16 @@ void convert_pad_f32(cudaStream_t s, const float* in, int rows, int cols, void* 
     if (rows <= 0 || ld_out <= 0) return;
     const dim3 grid((unsigned)((ld_out + 1023) / 1024), (unsigned)std::min(65535, (rows + 3) / 4));
     k_convert_pad_f32<<<grid, 256, 0, s>>>(in, rows, cols, out, ld_out, to_bf16, lo);
+}
+
+void gather_operand(cudaStream_t s, int rows, int cols, const int* map, const float* src, void* out, float* lo, int ld_out,
+                    int to_bf16) {
+    for (int r0 = 0; r0 < rows; r0 += 65535) {
+        const dim3 grid(blocks(cols, 256), std::min(65535, rows - r0));
+        const size_t at = (size_t)r0 * ld_out * (to_bf16 ? 2 : 4);
+        k_gather_operand<<<grid, 256, 0, s>>>(cols, map ? map + r0 : nullptr, map ? src : src + (size_t)r0 * cols, static_cast<char*>(out) + at,
+                                              lo ? lo + (size_t)r0 * ld_out : nullptr, ld_out, to_bf16);
+    }
 }
 
 void pool_store(cudaStream_t s, int count, int p, int is_f64, const int* rows, const int* slots, const void* B,

@@ -83,15 +83,17 @@ __device__ __forceinline__ void prox_node(const ProxArgs& a) {
     __shared__ ProxShared<T, NWG> shared_all[GPC];
     const int grp = GPC == 1 ? 0 : (int)(threadIdx.x / 32);
     ProxShared<T, NWG>& sh = shared_all[grp];
-    const int b = blockIdx.x * GPC + grp;
+    const int row = blockIdx.x * GPC + grp;              // of Gpart and Vop; the node is b
     // programmatic dependent launch (no-ops without the launch attribute): let the
     // next kernel start its prologue, then wait for the gradient's producer
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (b >= a.m) return;
+    if (row >= a.m) return;
+    const int b = a.rowmap ? a.rowmap[row] : row;
+    if (b < 0) return;
     if (a.active != nullptr && a.active[b] == 0) return;
     const int p = a.p;
-    const size_t base = (size_t)b * p;
+    const size_t base = (size_t)b * p, gbase = (size_t)row * p;
     const T* __restrict__ Gm = static_cast<const T*>(a.G);
     T* __restrict__ V = static_cast<T*>(a.V);
     T* __restrict__ Bm = static_cast<T*>(a.B);
@@ -143,7 +145,7 @@ __device__ __forceinline__ void prox_node(const ProxArgs& a) {
             float t[QB][E];
 #pragma unroll
             for (int qq = 0; qq < QB; ++qq) {
-                const float* gp = a.Gpart + (size_t)(q + qq) * a.gstride + base;
+                const float* gp = a.Gpart + (size_t)(q + qq) * a.gstride + gbase;
 #pragma unroll
                 for (int e = 0; e < E; ++e) {
                     const int j = G::rank() + e * NT;
@@ -156,7 +158,7 @@ __device__ __forceinline__ void prox_node(const ProxArgs& a) {
                 for (int e = 0; e < E; ++e) gsum[e] += T(t[qq][e]);
         }
         for (; q < a.gsplits; ++q) {
-            const float* gp = a.Gpart + (size_t)q * a.gstride + base;
+            const float* gp = a.Gpart + (size_t)q * a.gstride + gbase;
 #pragma unroll
             for (int e = 0; e < E; ++e) {
                 const int j = G::rank() + e * NT;
@@ -369,7 +371,7 @@ __device__ __forceinline__ void prox_node(const ProxArgs& a) {
             const T vn = bv + coef * (bv - be);
             Bm[base + j] = bv;
             V[base + j] = vn;
-            if (a.Vop != nullptr) store_operand2(a.Vop, a.Vop_lo, (size_t)b * a.op_ld + j, (float)vn, a.op_bf16);
+            if (a.Vop != nullptr) store_operand2(a.Vop, a.Vop_lo, (size_t)row * a.op_ld + j, (float)vn, a.op_bf16);
         }
     }
 }

@@ -218,9 +218,9 @@ __device__ __forceinline__ void stream_sum(const ProxArgs& a, size_t base, int l
 // most one node: a batch that small has up to 16 slices, whose loads one warp takes
 // longer over than over much of the rest (a launch between its events: 28.6 us at one
 // node of p = 1000, now 18.9; 17.9 at 64 nodes of p = 611, now 15.9).
-__device__ __forceinline__ void stream_sum_cta(const ProxArgs& a, int b, unsigned char* rows0) {
+__device__ __forceinline__ void stream_sum_cta(const ProxArgs& a, int row, unsigned char* rows0) {
     float* su = reinterpret_cast<float*>(rows0 + 2 * mask_bytes(a.W));
-    const float* G = a.Gpart + (size_t)b * a.p;
+    const float* G = a.Gpart + (size_t)row * a.p;
     for (int j = threadIdx.x; j < a.p; j += blockDim.x) {
         float g = G[j];
         for (int s0 = 1; s0 < a.gsplits; s0 += 8) {
@@ -239,7 +239,7 @@ __device__ __forceinline__ void stream_sum_cta(const ProxArgs& a, int b, unsigne
 // A. node b's masks, G and V rows into the row set `rows` (asynchronous copies,
 // one commit group); summed: G is there already.
 template <int VEC>
-__device__ __forceinline__ void stream_issue(const ProxArgs& a, int b, int lane, unsigned char* rows, bool summed) {
+__device__ __forceinline__ void stream_issue(const ProxArgs& a, int row, int b, int lane, unsigned char* rows, bool summed) {
     const int p = a.p, W = a.W, nq = p / VEC;
     uint32_t* smi = reinterpret_cast<uint32_t*>(rows);
     uint32_t* smo = reinterpret_cast<uint32_t*>(rows + mask_bytes(W));
@@ -247,7 +247,7 @@ __device__ __forceinline__ void stream_issue(const ProxArgs& a, int b, int lane,
     float* sv = su + row_bytes(p) / sizeof(float);
     const size_t base = (size_t)b * p;
     const float* V = static_cast<const float*>(a.V) + base;
-    const float* G0 = a.gsplits == 0 ? static_cast<const float*>(a.G) + base : a.Gpart + base;
+    const float* G0 = a.gsplits == 0 ? static_cast<const float*>(a.G) + base : a.Gpart + (size_t)row * p;
     for (int q = lane; q < W; q += 32) {
         cp_async4(smi + q, a.in_mask + (size_t)b * W + q);
         cp_async4(smo + q, a.out_mask + (size_t)b * W + q);
@@ -268,7 +268,7 @@ __device__ __forceinline__ void stream_issue(const ProxArgs& a, int b, int lane,
 // stream_issue (the node's scalars are read while they arrive), laid out for
 // a.p and a.W with the padding zeroed.
 template <int VEC>
-__device__ __forceinline__ void stream_node(const ProxArgs& a, int b, int lane, WarpHdr& h, unsigned char* rows,
+__device__ __forceinline__ void stream_node(const ProxArgs& a, int row, int b, int lane, WarpHdr& h, unsigned char* rows,
                                             bool summed) {
     const int p = a.p, p4 = (p + 3) >> 2, W = a.W;
     uint32_t* smi = reinterpret_cast<uint32_t*>(rows);
@@ -294,7 +294,7 @@ __device__ __forceinline__ void stream_node(const ProxArgs& a, int b, int lane, 
         if (lane == 0) { h.nj1 = 0; h.ncand = 0; }
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncwarp();
-        if (!summed && a.gsplits > 1) stream_sum<VEC>(a, base, lane, su);
+        if (!summed && a.gsplits > 1) stream_sum<VEC>(a, (size_t)row * p, lane, su);
         // u = v - eta G; J0 entries become 0 now, J1 entries once they are listed below.
         // Two running top-two pairs (even and odd positions) keep the chains short.
         float t1 = 0.f, t2 = 0.f, t1b = 0.f, t2b = 0.f;
@@ -541,7 +541,7 @@ __device__ __forceinline__ void stream_node(const ProxArgs& a, int b, int lane, 
         }
         __syncwarp();
         float d0 = 0.f, d1 = 0.f;
-        const size_t ob = (size_t)b * a.op_ld;
+        const size_t ob = (size_t)row * a.op_ld;
         constexpr int UN = VEC == 4 ? 4 : 8;          // beta_old loads in flight per lane
         using VT = typename std::conditional<VEC == 4, float4, float>::type;
         for (int q0 = lane; q0 < nq; q0 += 32 * UN) {
@@ -607,16 +607,18 @@ __global__ void __launch_bounds__(32 * kStreamMaxWarps, 1) k_prox_stream(ProxArg
     // one node per CTA and split slices to add: by all warps (its row padding was zeroed above)
     const bool coop = a.m <= (int)gridDim.x && a.gsplits > 1;
     if (coop) {
-        if (a.active != nullptr && a.active[blockIdx.x] == 0) return;
+        const int b = a.rowmap ? a.rowmap[blockIdx.x] : (int)blockIdx.x;
+        if (b < 0 || (a.active != nullptr && a.active[b] == 0)) return;
         stream_sum_cta(a, blockIdx.x, smem + align16(sizeof(WarpHdr)));
     }
     // nodes go round the CTAs first (node b to CTA b mod grid), so that every SM
     // holds the same number of nodes and a last partial round is spread over all
     // SMs rather than packed onto the first few
-    for (int b = warp * gridDim.x + blockIdx.x; b < a.m; b += gridDim.x * wpc) {
-        if (a.active != nullptr && a.active[b] == 0) continue;
-        stream_issue<VEC>(a, b, lane, rows, coop);
-        stream_node<VEC>(a, b, lane, h, rows, coop);
+    for (int r = warp * gridDim.x + blockIdx.x; r < a.m; r += gridDim.x * wpc) {
+        const int b = a.rowmap ? a.rowmap[r] : r;
+        if (b < 0 || (a.active != nullptr && a.active[b] == 0)) continue;
+        stream_issue<VEC>(a, r, b, lane, rows, coop);
+        stream_node<VEC>(a, r, b, lane, h, rows, coop);
     }
 }
 
@@ -638,23 +640,23 @@ __global__ void __launch_bounds__(32 * kStreamMaxWarps, 1) k_prox_stream_group(c
         int pi = 0;
         while (pi + 1 < g.np && (int)blockIdx.x >= g.nbase[pi + 1]) ++pi;
         const ProxArgs& a = g.a[pi];
-        const int b = (int)blockIdx.x - g.nbase[pi];
-        if (a.active != nullptr && a.active[b] == 0) return;
+        const int r = (int)blockIdx.x - g.nbase[pi], b = a.rowmap ? a.rowmap[r] : r;
+        if (b < 0 || (a.active != nullptr && a.active[b] == 0)) return;
         coop = a.gsplits > 1;
-        if (coop) stream_sum_cta(a, b, smem + align16(sizeof(WarpHdr)));
+        if (coop) stream_sum_cta(a, r, smem + align16(sizeof(WarpHdr)));
     }
     for (int t = warp * gridDim.x + blockIdx.x; t < g.nbase[g.np]; t += gridDim.x * wpc) {
         int pi = 0;
         while (pi + 1 < g.np && t >= g.nbase[pi + 1]) ++pi;
         const ProxArgs& a = g.a[pi];
-        const int b = t - g.nbase[pi];
-        if (a.active != nullptr && a.active[b] == 0) continue;
+        const int r = t - g.nbase[pi], b = a.rowmap ? a.rowmap[r] : r;
+        if (b < 0 || (a.active != nullptr && a.active[b] == 0)) continue;
         if (pi != last) {
             stream_pad(rows, a.p, a.W, lane);
             last = pi;
         }
-        stream_issue<VEC>(a, b, lane, rows, coop);
-        stream_node<VEC>(a, b, lane, h, rows, coop);
+        stream_issue<VEC>(a, r, b, lane, rows, coop);
+        stream_node<VEC>(a, r, b, lane, h, rows, coop);
     }
 }
 
