@@ -68,7 +68,7 @@ __device__ __forceinline__ T entry_point(T a, T c, T M) {
 // value: Algorithm 1's prox_{rho_bar H_M}(xi_bar) written in the scale of u).
 template <typename T>
 __device__ __forceinline__ T model_root(T nt, T St, T nl, T Sl, T c, T M) {
-    const T xa = c * (St + Sl) / (nt * (T(1) + c) + c * nl);
+    const T xa = c * (St + Sl) / fma(c, nl, nt * (T(1) + c));   // (which product is rounded: written out)
     if (xa <= c * M) return xa;
     return (St + Sl - nt * M) / (nt + nl);
 }
