@@ -212,8 +212,8 @@ static __device__ const unsigned long long kExp2Dev[64] = {KGLM_EXP2_TABLE};
 // of third order, y (1 + e + e^2).  Table lookup and series as in Tang, "Table-driven
 // implementation of the exponential function in IEEE floating-point arithmetic", ACM
 // TOMS 1989.  Errors before the final rounding are below 2^-58 relative: 0.52 ulp
-// (expf of FP64, an addition and a division: 1.5 ulp).
-__host__ __device__ __forceinline__ double sigmoid_neg(double t, const unsigned long long* tab) {
+// (expf of FP64, an addition and a division: 1.5 ulp).  With et, *et = e^t too (0.52 ulp).
+__host__ __device__ __forceinline__ double sigmoid_neg(double t, const unsigned long long* tab, double* et = nullptr) {
     const uint64_t u = f64_bits(t);
     const bool neg = (int64_t)u < 0;
     const int ex = (int)(u >> 52) & 0x7ff;
@@ -249,6 +249,10 @@ __host__ __device__ __forceinline__ double sigmoid_neg(double t, const unsigned 
     const int j = N & 63, k0 = N >> 6;
     const int64_t T = (int64_t)tab[j];
     const uint64_t E = (uint64_t)(T + mulhi_s(T, w));    // 2^(j/64) e^r in units of 2^-62
+    if (et) {
+        const int le = clz64(E);
+        *et = round_f64(false, E << le, false, k0 - 62 - le);
+    }
     // 1 + e^t = 2^k d in units of 2^-62
     uint64_t d;
     int k = 0;

@@ -35,6 +35,7 @@
 
 #include "common.cuh"
 #include "engine.h"
+#include "fixed.cuh"
 
 namespace kglm {
 
@@ -144,6 +145,34 @@ __device__ __forceinline__ double exp_t(double t) { return exp(t); }
 __device__ __forceinline__ float sqrt_t(float t) { return sqrtf(t); }
 __device__ __forceinline__ double sqrt_t(double t) { return sqrt(t); }
 
+// The logistic loss of samples t = y s in FP64, on a pipe of two operations per cycle per SM
+// (which the two exponentials, the logarithm and the division of a sample filled to a third
+// of the kernel's operations).  e^-|t| and 1 / (1 + e^-|t|) come from integer arithmetic,
+// and log(1 + e_1) + ... + log(1 + e_j) = log1p(Q), 1 + Q = (1 + e_1) ... (1 + e_j), is one
+// logarithm per 512 samples of a thread (Q < 2^512): Q + e + Q e in two operations keeps
+// Q's relative accuracy where every e is small, as a sum of logarithms would.
+// 1024 nodes, n = 2000, p = 200, k = 10, a whole evaluation: 18.9 -> 15.0 ms.
+struct LossSum {
+    double lin, Q;
+    int cnt;
+};
+__device__ __forceinline__ void loss_add(LossSum& L, double t, double& e, double& sig) {
+    if (fabs(t) <= 708.0) {
+        sig = sigmoid_neg(-fabs(t), kExp2Dev, &e);
+    } else {
+        e = exp(-fabs(t));
+        sig = 1.0 / (1.0 + e);
+    }
+    if (t < 0.0) L.lin -= t;
+    L.Q = fma(L.Q, e, L.Q + e);
+    if (++L.cnt == 512) {
+        L.lin += log1p(L.Q);
+        L.Q = 0.0;
+        L.cnt = 0;
+    }
+}
+__device__ __forceinline__ double loss_total(const LossSum& L) { return L.lin + log1p(L.Q); }
+
 // 4 consecutive elements from / to 16-byte aligned shared memory.
 __device__ __forceinline__ void ld4(const float* p, float (&v)[4]) {
     const float4 q = *reinterpret_cast<const float4*>(p);
@@ -217,6 +246,7 @@ __device__ void evaluate(const ReoptArgs& a, RS& sh, const Dyn<TI>& dy, const do
 #pragma unroll
     for (int o = 0; o < 4; ++o) gacc[o] = TI(0);
     TI floss = TI(0);
+    LossSum ls{0.0, 0.0, 0};
     const int CH = dy.ch, XS = dy.xs;
     for (int i0 = 0; i0 < a.n; i0 += CH) {
         const int cn = min(CH, a.n - i0);
@@ -235,9 +265,16 @@ __device__ void evaluate(const ReoptArgs& a, RS& sh, const Dyn<TI>& dy, const do
                 st4(dy.Xs + (size_t)t * XS + 4 * r4, x);
             }
             const TI yi = yv[i];
-            floss += softplus_t(-yi * s);
-            const TI sg = TI(1) / (TI(1) + exp_t(yi * s));   // sigma(-y s)
-            st2(dy.wd + 2 * t, sg * (TI(1) - sg), -yi * sg);
+            if constexpr (sizeof(TI) == 8) {
+                double e, sig;
+                loss_add(ls, yi * s, e, sig);
+                const double es = e * sig;               // sigma(-|t|); sig is sigma(|t|)
+                st2(dy.wd + 2 * t, es * sig, -yi * (yi * s < 0.0 ? sig : es));
+            } else {
+                floss += softplus_t(-yi * s);
+                const TI sg = TI(1) / (TI(1) + exp_t(yi * s));   // sigma(-y s)
+                st2(dy.wd + 2 * t, sg * (TI(1) - sg), -yi * sg);
+            }
         }
         __syncthreads();
         if (bp < pm.nbp) {
@@ -253,7 +290,7 @@ __device__ void evaluate(const ReoptArgs& a, RS& sh, const Dyn<TI>& dy, const do
                         const TI xw = xr[e] * w;
                         gacc[e] += xr[e] * dd;
 #pragma unroll
-                        for (int f = 0; f < 4; ++f) acc[e * 4 + f] += xw * xr[f];
+                        for (int f = e; f < 4; ++f) acc[e * 4 + f] += xw * xr[f];
                     }
                 }
             } else {
@@ -296,7 +333,7 @@ __device__ void evaluate(const ReoptArgs& a, RS& sh, const Dyn<TI>& dy, const do
             }
         }
     }
-    const double fl = block_total((double)floss, sh.red);
+    const double fl = block_total(sizeof(TI) == 8 ? loss_total(ls) : (double)floss, sh.red);
     if (tid == 0) {                // the ridge term once (FP64 is the slow pipe), same sum as before
         double ridge = 0.0;
         for (int r = 0; r < ks; ++r) ridge += vec[r] * vec[r];
@@ -386,7 +423,7 @@ __device__ void newton_direction(RS& sh, const Dyn<TI>& dy, int k, double M, dou
 }
 
 template <typename TI>
-__global__ __launch_bounds__(NT, sizeof(TI) == 4 ? 4 : 1) void k_reopt(ReoptArgs a) {
+__global__ __launch_bounds__(NT, sizeof(TI) == 4 ? 4 : 2) void k_reopt(ReoptArgs a) {
     // stopping level of the working precision: the predicted decrease below
     // which f can neither check Armijo nor improve
     const double tol = a.tol;
@@ -496,6 +533,7 @@ __global__ __launch_bounds__(NT, sizeof(TI) == 4 ? 4 : 1) void k_reopt(ReoptArgs
     // predictor and the running sum take FP64 operations, the slow pipe here.
     double part = 0.0;
     const bool fast = sizeof(TI) == 4 && a.kind == kLOGISTIC;
+    LossSum ls{0.0, 0.0, 0};
     for (int i = tid; i < a.n; i += NT) {
         double s = 0.0;
         for (int r = 0; r < ks; ++r) s += a.Xt[(size_t)sh.S[r] * a.n + i] * sh.b[r];
@@ -507,10 +545,14 @@ __global__ __launch_bounds__(NT, sizeof(TI) == 4 ? 4 : 1) void k_reopt(ReoptArgs
             const float m1 = __fmul_ru(__fmul_ru(fabsf(tf), 0x1p-23f * (1.f + 0x1p-22f)), slope);
             const float mg = __fadd_ru(__fadd_ru(m1, l * 0x1p-21f), 0x1p-125f);
             part += (double)__fadd_ru(l, mg);
+        } else if (a.kind == kLOGISTIC) {
+            double e, sig;
+            loss_add(ls, a.y[i] * s, e, sig);
         } else {
             part += loss64(s, a.y[i], a.kind);
         }
     }
+    if (!fast && a.kind == kLOGISTIC) part = loss_total(ls);
     const double tot = block_total(part, sh.red);
     if (tid == 0) {
         double rid = 0.0;
