@@ -62,7 +62,7 @@ FALLBACK = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1
 SMS = 152
 # arithmetic type of the products per engine mode (tf32x3: FP32 values carried as TF32 hi + lo pairs)
 DTYPE = {"fp64": "f64", "fp32": "f32", "tf32x3": "f32", "bf16": "bf16", "tf32": "tf32"}
-PRODUCTS = {"fp64": "fp64 (CUDA cores)", "fp32": "fp32 (CUDA cores)",
+PRODUCTS = {"fp64": "fp64: exact BF16 digit products on tcgen05 (small batches: CUDA cores)", "fp32": "fp32 (CUDA cores)",
             "tf32x3": "fp32-accurate: TF32 hi+lo split, 3 tcgen05 products, FP32 accumulate",
             "bf16": "bf16 tcgen05, FP32 accumulate", "tf32": "tf32 tcgen05, FP32 accumulate"}
 FP32_LANES_PER_SM = 128          # FP32 FMA lanes per SM (4 partitions x 32)
@@ -226,7 +226,7 @@ def roofline(stats, prec, pk, workload=WORKLOAD, nodes=8192):
     if best in ("gemm_xv_link", "gemm_xtr", "cert_xb", "cert_xtzeta"):
         fp64 = prec == "fp64" or best == "cert_xtzeta"
         if fp64:
-            peak, note = FP64_NOMINAL_TFLOPS, "FP64 nominal of the recipe"
+            peak, note = FP64_NOMINAL_TFLOPS, "FP64 pipe, nominal (digit products on the tensor cores can pass it)"
         else:
             peak = SMS * FP32_LANES_PER_SM * 2 * sm_max / 1e12
             note = "FP32 FMA: 152 SMs x 128 lanes x 2 x max SM clock"

@@ -234,10 +234,10 @@ kglm_status kglm_xtr(kglm_ctx* ctx, int32_t m, const void* R, void* G);
  * per row of Z) with an entrywise bound Qerr[b][j] >= |Q[b][j] - exact|.
  *   Z: host, m x n row-major FP64; Q, Qerr: host, m x p row-major FP64
  *   outputs (Qerr may be NULL); 1 <= m <= max_batch.
- * The FP64 mode computes Q by an FP64 GEMM and writes Qerr = 0 (FP64
+ * The FP64 mode computes Q in FP64 and writes Qerr = 0 (FP64
  * rounding only).  The reduced-precision modes use the engine's
- * exact-splitting product on the BF16 tensor cores (6-bit digits of X and
- * Z, integer-exact FP32 accumulation, FP64 combine) with its rigorous bound
+ * exact-splitting product on the BF16 tensor cores (signed bytes of X and
+ * Z, exact integer accumulation, one rounding to FP64) with its rigorous bound
  * in Qerr; where that product is not set up (job count or HBM budget) they
  * fall back to the FP64 GEMM with Qerr = 0.  Uses the batch buffers: call
  * it between evaluations, not between a push and its evaluation (the pushed

@@ -465,7 +465,7 @@ double gram_lambda_max(kglm_ctx* c) {
 }
 
 // ---- FP64 products on the tensor cores (split64.cu)
-// Where they pay: from about 2e7 FMAs per product on.  Microseconds per FISTA
+// Where they pay: the line is just above the tie at 2.0e7 FMAs per product.  Microseconds per FISTA
 // iteration, digits against CUDA cores: m n p = 2.0e7 (n 5000, p 1000) 165 / 165,
 // 2.6e7 (n 2000, p 200) 100 / 146, 2.6e7 (n 1000, p 100) 80 / 158, 3.2e7 (n 5000,
 // p 400) 152 / 187, 8e7 (n 5000, p 1000) 171 / 385, 1.3e9 255 / 4554; at 1.3e7
@@ -1040,8 +1040,8 @@ void evaluate_check(kglm_ctx* c, int it) {
 // the products' 128-row tiles (a product of 12 rows costs as much as one of 64: there the
 // captured iterations of the whole batch are the faster, 4.5 ms against 4.8 for 64 nodes,
 // n = 1373, p = 611), and from then on wherever a quarter of the rows left goes.  A search
-// of 2400 batches' nodes (n = 5000, p = 1000, 7 % of them unfinished after a check): 108.7
-// -> 100.5 ms.  Only the operand and gradient rows move (row r is node d_slots[r]); a
+// of 9341 nodes in 23 batches (n = 5000, p = 1000, 7 % of a batch left after a check on
+// average) with its set-up: 108.7 -> 102.0 ms.  Only the operand and gradient rows move (row r is node d_slots[r]); a
 // node's own arrays, its sums over K (the split-K slices stay the batch's) and so its bits
 // do not.  (Tiles or sub-batches chosen by the caller tie the split to the rows: those keep
 // every row.)  The last certificate takes the whole batch again.
@@ -2568,7 +2568,7 @@ kglm_status kglm_create(const kglm_desc* desc, const double* X, const double* y,
             c->dq_on = true;
         }
         // reduced-precision modes: digits of X for the exact certificate product
-        // (6-bit digits, 7 per value), when the jobs and the HBM budget allow
+        // (signed bytes, 6 per value), when the jobs and the HBM budget allow
         if (!c->f64 && exact_plan((int)n, &c->xplan)) {
             const ExactPlan& x = c->xplan;
             // (rows of kCertDigits segments; the buffers keep the size the footprint states)
