@@ -1041,10 +1041,10 @@ void evaluate_check(kglm_ctx* c, int it) {
 // captured iterations of the whole batch are the faster, 4.5 ms against 4.8 for 64 nodes,
 // n = 1373, p = 611), and from then on wherever a quarter of the rows left goes.  A search
 // of 9341 nodes in 23 batches (n = 5000, p = 1000, 7 % of a batch left after a check on
-// average) with its set-up: 108.7 -> 102.0 ms.  Only the operand and gradient rows move (row r is node d_slots[r]); a
-// node's own arrays, its sums over K (the split-K slices stay the batch's) and so its bits
-// do not.  (Tiles or sub-batches chosen by the caller tie the split to the rows: those keep
-// every row.)  The last certificate takes the whole batch again.
+// average) with its set-up: 108.7 -> 102.0 ms.  Only the operand and gradient rows move
+// (row r is node d_slots[r]); a node's own arrays, its sums over K (the split-K slices stay
+// the batch's) and so its bits do not.  (Tiles or sub-batches chosen by the caller tie the
+// split to the rows: those keep every row.)  The last certificate takes the whole batch again.
 bool any_active(kglm_ctx* c) {
     const int* h = c->pinned<int>(c->off_active());
     int left = 0;

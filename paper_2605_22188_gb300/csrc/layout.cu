@@ -321,8 +321,8 @@ void gather_operand(cudaStream_t s, int rows, int cols, const int* map, const fl
     for (int r0 = 0; r0 < rows; r0 += 65535) {
         const dim3 grid(blocks(cols, 256), std::min(65535, rows - r0));
         const size_t at = (size_t)r0 * ld_out * (to_bf16 ? 2 : 4);
-        k_gather_operand<<<grid, 256, 0, s>>>(cols, map ? map + r0 : nullptr, map ? src : src + (size_t)r0 * cols, static_cast<char*>(out) + at,
-                                              lo ? lo + (size_t)r0 * ld_out : nullptr, ld_out, to_bf16);
+        k_gather_operand<<<grid, 256, 0, s>>>(cols, map ? map + r0 : nullptr, map ? src : src + (size_t)r0 * cols,
+                                              static_cast<char*>(out) + at, lo ? lo + (size_t)r0 * ld_out : nullptr, ld_out, to_bf16);
     }
 }
 
