@@ -73,6 +73,7 @@ struct kglm_ctx {
     int *kbar = nullptr, *pf = nullptr;
     void *B = nullptr, *V = nullptr, *G = nullptr, *R = nullptr;
     double *tmom = nullptr, *zeta = nullptr, *Q = nullptr;
+    bool zeta_f32 = false;   // zeta's rows are packed FP32 values (a certificate that keeps them so)
     float* phint = nullptr;       // per node: the streaming prox's selection and threshold hints
     int *active = nullptr, *iters_done = nullptr, *support = nullptr, *jstar = nullptr;
     double *sum_loss = nullptr, *sum_conj = nullptr, *lb_now = nullptr, *primal_now = nullptr;
@@ -694,6 +695,21 @@ const TcMap& b_map(kglm_ctx* c, int which, int bn) {
     return it->second;
 }
 
+// zeta's packed FP32 rows from row `from` on in FP64, in place: the entries [hi / 2, hi) are
+// written past the last FP32 value still to be read, then [hi / 4, hi / 2) and so on.
+void widen_zeta(kglm_ctx* c, int from) {
+    if (!c->zeta_f32) return;
+    const float* z32 = reinterpret_cast<const float*>(c->zeta);
+    const size_t end = (size_t)from * c->n;
+    for (size_t hi = (size_t)c->m * c->n; hi > end;) {
+        const size_t lo = hi > 1 ? (hi + 1) / 2 : 0;
+        convert_to_f64(c->st, z32 + lo, 0, c->zeta + lo, hi - lo);
+        hi = lo;
+    }
+    c->zeta_f32 = false;
+    check_launch();
+}
+
 void certify(kglm_ctx* c) {
     Nvtx range("certificate");
     const int m = c->rows(), n = c->n, p = c->p;
@@ -715,6 +731,7 @@ void certify(kglm_ctx* c) {
         a.DZ = c->DZ; a.ztau = c->ztau;
         a.dz_npad = c->xplan.npad;
     }
+    c->zeta_f32 = a.DZ != nullptr;
     const double ws = c->f64 ? 8.0 : 4.0;
     {
         Scope sc(c, PH_CERT_XB, split_on(c, m) ? 3 : 1, 2.0 * n * c->sum_pa);
@@ -2683,6 +2700,7 @@ kglm_status kglm_xtz(kglm_ctx* ctx, int32_t m, const double* Z, double* Q, doubl
         REQ(Z && Q, "Z and Q are required");
         kglm_ctx* c = ctx;
         const size_t mp = (size_t)m * c->p;
+        widen_zeta(c, m);                              // the batch's dual points past Z's rows stay readable
         CK(cudaMemcpyAsync(c->zeta, Z, sizeof(double) * m * (size_t)c->n, cudaMemcpyHostToDevice, c->st));
         CertArgs a{};
         {
@@ -2760,7 +2778,7 @@ kglm_status kglm_read_batch(kglm_ctx* ctx, double* beta, double* zeta) {
                 for (size_t t = 0; t < mp; ++t) beta[t] = h[t];
             }
         }
-        if (zeta && ctx->cexact) {                     // an FP32 value, kept as one
+        if (zeta && ctx->zeta_f32) {                   // FP32 values, kept as such
             std::vector<float> h(mn);
             CK(cudaMemcpyAsync(h.data(), ctx->zeta, sizeof(float) * mn, cudaMemcpyDeviceToHost, ctx->st));
             sync(ctx);
