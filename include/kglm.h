@@ -335,8 +335,10 @@ kglm_status kglm_configure(kglm_ctx* ctx, const kglm_tune* cfg);
  * max_batch x p FP64 buffer that kglm_push_nodes with warm_B, and one that
  * kglm_xtz, allocate on first use; and in the FP64 mode the digits of the
  * tensor-core products (about 32 n p + 16 max_batch (n + p) + 32 max_batch max(n, p) bytes),
- * allocated at the first batch large enough for them and left out, with the
- * products on the CUDA cores, where hbm_budget or the device does not hold them.  KGLM_EINVAL for a desc kglm_create would
+ * allocated at the first batch large enough for them.  They are left out, with the
+ * products on the CUDA cores, where hbm_budget does not hold them or, without a
+ * budget, half of the device's free memory does not, and given back where one of the
+ * first-use buffers needs their room.  KGLM_EINVAL for a desc kglm_create would
  * reject on its sizes, ranges or enums. */
 kglm_status kglm_estimate_bytes(const kglm_desc* desc, int64_t* bytes);
 
@@ -414,7 +416,9 @@ kglm_status kglm_rashomon(kglm_ctx* ctx, double eps, int64_t max_models, int32_t
  * included) fits in the budget the running requests leave; a request's
  * memory returns to the budget when it finishes.  A request's nodes see the
  * same arithmetic whatever shares the launches, so its result (objective,
- * support, node count) does not depend on the other requests. */
+ * support, node count) does not depend on the other requests.  A request holds
+ * what it was admitted for and no more: FP64 requests run their products on the
+ * CUDA cores (the digits of kglm_estimate_bytes are not part of that). */
 typedef struct kglm_server kglm_server;
 
 typedef struct {

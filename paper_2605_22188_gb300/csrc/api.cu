@@ -160,6 +160,8 @@ struct kglm_ctx {
         int bnS = 0, bnG = 0;
         SplitPlan pS{}, pG{};                        // plans of batch sizes mS and mG
         int mS = -1, mG = -1;
+        size_t a0 = 0, a1 = 0, held = 0;             // their entries of allocs, and bytes
+        bool own_err = false;                        // d_tcerr is among them
     } sp;
     // host mirror of the evaluated batch
     std::vector<int> h_kbar, h_pf, h_jstar;
@@ -243,17 +245,25 @@ kglm_status guarded(kglm_ctx* ctx, F&& f) {
     }
 }
 
+bool split_release(kglm_ctx* c);
+void destroy_graphs(kglm_ctx* c);
+
+// Device memory of the context, within its budget.  What a call must have comes before the
+// optional digits of the FP64 products: they are given back where it does not fit beside them.
 void* dalloc(kglm_ctx* c, size_t bytes) {
     if (bytes == 0) bytes = 16;
-    if (c->d.hbm_budget > 0 && (int64_t)(c->bytes + bytes) > c->d.hbm_budget)
-        throw Fail{KGLM_ENOMEM, "over the HBM budget of the context"};
     void* p = nullptr;
-    // stream-ordered: no device-wide synchronization when contexts come and go
-    // while others run (the serving loop)
-    cudaError_t e = cudaMallocAsync(&p, bytes, c->st);
-    if (e != cudaSuccess) {
+    for (;;) {
+        if (c->d.hbm_budget > 0 && (int64_t)(c->bytes + bytes) > c->d.hbm_budget) {
+            if (split_release(c)) continue;
+            throw Fail{KGLM_ENOMEM, "over the HBM budget of the context"};
+        }
+        // stream-ordered: no device-wide synchronization when contexts come and go
+        // while others run (the serving loop)
+        const cudaError_t e = cudaMallocAsync(&p, bytes, c->st);
+        if (e == cudaSuccess) break;
         cudaGetLastError();
-        throw Fail{KGLM_ENOMEM, std::string("cudaMallocAsync: ") + cudaGetErrorString(e)};
+        if (!split_release(c)) throw Fail{KGLM_ENOMEM, std::string("cudaMallocAsync: ") + cudaGetErrorString(e)};
     }
     c->allocs.push_back(p);
     c->bytes += bytes;
@@ -494,14 +504,22 @@ void split_setup(kglm_ctx* c) {
     q.cap = 8 * mc * std::max(n * split_parts((int)p, 8), p * split_parts((int)n, 8));
     const size_t need = 16 * ((n + mc) * q.pk + (p + mc) * q.nk) + 4 * (n + p + 2 * mc) + 4 * q.cap + 64;
     if (c->d.hbm_budget > 0 && (int64_t)(c->bytes + need) > c->d.hbm_budget) return;
-    const size_t had = c->allocs.size(), bytes0 = c->bytes;
-    int* tcerr0 = c->d_tcerr;
+    if (c->d.hbm_budget <= 0) {
+        // without a budget: at most half of what the device has free, the rest is left to
+        // whatever else the caller sized by kglm_estimate_bytes
+        size_t avail = 0, total = 0;
+        if (cudaMemGetInfo(&avail, &total) != cudaSuccess || need > avail / 2) {
+            cudaGetLastError();
+            return;
+        }
+    }
+    q.a0 = c->allocs.size();
+    const size_t bytes0 = c->bytes;
     auto drop = [&] {
-        for (size_t i = had; i < c->allocs.size(); ++i) cudaFreeAsync(c->allocs[i], c->st);
-        c->allocs.resize(had);
-        c->bytes = bytes0;
-        c->d_tcerr = tcerr0;
-        q.on = false;
+        q.a1 = c->allocs.size();
+        q.held = c->bytes - bytes0;
+        q.on = true;
+        split_release(c);
     };
     try {
         q.DX = dalloc_t<__nv_bfloat16>(c, 8 * n * q.pk);
@@ -516,6 +534,7 @@ void split_setup(kglm_ctx* c) {
         q.flag = dalloc_t<int>(c, 1);
         if (!c->d_tcerr) {
             c->d_tcerr = dalloc_t<int>(c, 1);
+            q.own_err = true;
             CK(cudaMemsetAsync(c->d_tcerr, 0, sizeof(int), c->st));
         }
     } catch (const Fail&) {
@@ -541,7 +560,30 @@ void split_setup(kglm_ctx* c) {
         drop();
         return;
     }
+    q.a1 = c->allocs.size();
+    q.held = c->bytes - bytes0;
     q.on = true;
+}
+
+// The digits' memory back, with the captured iterations that use it; the products run on
+// the CUDA cores from here on.  False where the context holds none.
+bool split_release(kglm_ctx* c) {
+    kglm_ctx::Split64& q = c->sp;
+    if (!q.on) return false;
+    cudaStreamSynchronize(c->st);
+    destroy_graphs(c);
+    for (size_t i = q.a0; i < q.a1; ++i) cudaFreeAsync(c->allocs[i], c->st);
+    c->allocs.erase(c->allocs.begin() + q.a0, c->allocs.begin() + q.a1);
+    c->bytes -= q.held;
+    if (q.own_err) {
+        c->d_tcerr = nullptr;
+        c->tc_check_pending = false;
+    }
+    q = kglm_ctx::Split64{};
+    q.tried = true;
+    cudaStreamSynchronize(c->st);              // (freed for other streams and processes too)
+    cudaGetLastError();
+    return true;
 }
 
 bool split_on(const kglm_ctx* c, int m) { return c->sp.on && split_pays(c, m); }
