@@ -20,6 +20,7 @@
 #include "engine.h"
 #include "kglm.h"
 #include "pool.h"
+#include "tiling.h"
 
 using namespace kglm;
 
@@ -38,13 +39,6 @@ struct SavedSolve {
     std::vector<int> sup;
     std::vector<double> coef;
     int64_t nodes = 0, batches = 0, next_id = 0;
-};
-
-// Column tile, CTA pairs and split-K slices (0: the launcher's own count) of a product.
-struct Tiling {
-    int bn;
-    bool pair;
-    int splits;
 };
 
 struct kglm_ctx {
@@ -653,33 +647,7 @@ void xtzeta(kglm_ctx* c, int m, CertArgs& a) {
     a.ebound = x.ebound;
 }
 
-// ---- tiles of the tensor-core products where nobody set them
-// Microseconds of an M x N product over nkb K slices of 128 bytes at column tile bn: the
-// busiest worker's units, each bound by its products (2 cycles per column, slice and
-// part product) or by its operands' way from L2.  Measured on S = X V of 2048 nodes, n =
-// 10000, p = 2000: single CTAs take 0.50 us a slice whether the tile has 128 columns or
-// 224 (up to 87 KB/us), pairs 0.39 to 0.41 us at 192 to 256 columns (78 KB/us per CTA).
-// Plus the last unit's epilogue and a pair's cluster launch.
-double tiling_cost(int M, int N, int nkb, int na, int nb, int bn, bool pair, int splits) {
-    const int mt = (M + 127) / 128, nt = (N + bn - 1) / bn;
-    const long units = (long)(pair ? (mt + 1) / 2 : mt) * nt * splits;
-    const int workers = pair ? 76 : 152;
-    const double per = (nkb + splits - 1) / splits;
-    const double mma = 2.0 * bn * (na + nb - 1) / 1900.0;
-    const double load = pair ? std::max((128.0 + bn / 2) * 0.128 / 78.0, 0.38)
-                             : std::max((128.0 * na + (double)bn * nb) * 0.128 / 87.0, 0.48);
-    const double unit = per * std::max(mma, load) + 0.5;
-    return (double)((units + workers - 1) / workers) * unit + 2.5 * bn / 256.0 + (pair ? 1.5 : 0.0);
-}
-
-// The column tile and CTA pairs of a product of M nodes.  The
-// default widths leave SMs idle in the last wave (2048 nodes, p = 2000: 128 units on
-// 152 SMs) and take in twice the operand bytes a pair does.  The number of split-K
-// slices stays the default width's, and a product's sums run over K in the same order at
-// any width and in pairs, so that no bit of a result depends on the choice.  2048
-// nodes, n = 10000, p = 2000: S 147 -> 70 us per launch, G 81 -> 65,
-// X beta 420 -> 365; 64 nodes,
-// n = 1373, p = 611: G 16.3 -> 11.3 us.
+// ---- tiles of the tensor-core products where nobody set them (tiling.h)
 enum { TILE_LINK = 0, TILE_GRAD = 1, TILE_CERT = 2 };   // S = X V, G = X^T R, the certificate's X beta (TF32 hi + lo)
 Tiling pick_tiling(kglm_ctx* c, int M, int which) {
     const bool grad = which == TILE_GRAD, cert = which == TILE_CERT;
@@ -693,24 +661,13 @@ Tiling pick_tiling(kglm_ctx* c, int M, int which) {
     const int N = grad ? c->p : c->n, K = grad ? c->n : c->p, ke = c->tc_kind == 0 && !cert ? 64 : 32;
     const int nkb = (K + ke - 1) / ke, mt = (M + 127) / 128;
     const int na = c->x3 || cert ? 2 : 1, nb = grad ? (c->x3 ? 2 : 1) : (c->xlo || cert ? 2 : 1);
-    const int tiles = ((Mb + 127) / 128) * ((N + def - 1) / def);
-    // the default's split-K (tc_gemm)
-    int splits = grad ? std::max(1, std::min(c->gsplit_max, std::min((nkb + 3) / 4, std::max(1, 152 / tiles))))
-                      : (tiles < 152 ? std::min((nkb + 3) / 4, std::max(1, 152 / tiles)) : 1);
-    Tiling best{def, false, splits};
-    if (grad || splits == 1) {
-        const bool can_pair = c->tc_kind == 0 && !cert && mt >= 2;
-        double cost = tiling_cost(M, N, nkb, na, nb, def, best.pair, splits);
-        for (int bn = 64; bn <= tc_tile_cols(N); bn += 16)
-            for (int pr = 0; pr <= (can_pair ? 1 : 0); ++pr) {
-                if (!c->pair_auto && (pr != 0) != (c->pair && can_pair)) continue;
-                const double t = tiling_cost(M, N, nkb, na, nb, bn, pr != 0, splits);
-                if (t < 0.97 * cost) {
-                    cost = t;
-                    best = {bn, pr != 0, splits};
-                }
-            }
-    }
+    TileShape q{};
+    q.M = M; q.Mb = Mb; q.N = N; q.nkb = nkb; q.na = na; q.nb = nb; q.def = def;
+    q.max_bn = tc_tile_cols(N);
+    q.grad_splits = grad ? c->gsplit_max : 0;
+    q.can_pair = c->tc_kind == 0 && !cert && mt >= 2;
+    q.pair = c->pair_auto ? -1 : c->pair ? 1 : 0;
+    const Tiling best = choose_tiling(q);
     if (c->tilings.size() >= 256) c->tilings.clear();
     c->tilings[key] = best;
     return best;
