@@ -352,8 +352,10 @@ __global__ __launch_bounds__(NT) void k_cert_bound(const __grid_constant__ CertA
 // node.  FP64 operations are what GB300 has least of (one warp instruction per SM in 16
 // cycles), so an entry takes three of them, v_j = (|q~_j| + err_j) / (2 lambda2) from the
 // correctly rounded integer combine; the selections work on the bits of v and |beta|,
-// the beta sums of Theorem 4.1 are FP32 pairs, and only the at most 64 selected values
-// reach FP64 sums, in the order of their ranks.  8192 nodes of p = 2000: 0.54 ms (1.27 with
+// the beta sums of Theorem 4.1 are FP64 up to 512 coordinates and FP32 pairs per thread
+// beyond (a pair's squares keep some 48 bits and FP32's range: few entries per thread, added
+// up in FP64), and only the at most 64 selected values reach FP64 sums, in the order of
+// their ranks.  8192 nodes of p = 2000: 0.54 ms (1.27 with
 // a warp per node over 30 FP32 slices); one node of p = 1000: 31 us (78).
 struct CertNodeShared {
     SelectShared sel;
@@ -381,21 +383,6 @@ __device__ __forceinline__ void acc2_sq(float& hi, float& lo, float x) {
     acc2(hi, lo, pr);
     lo += fmaf(x, x, -pr);
 }
-// the pairs of a warp's lanes, summed (every lane gets the total)
-__device__ __forceinline__ void warp_acc2(float& hi, float& lo) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float h = __shfl_xor_sync(0xffffffffu, hi, o), l = __shfl_xor_sync(0xffffffffu, lo, o);
-        // the same sum in both lanes: the larger-indexed lane's pair is added to the other's
-        const bool up = (threadIdx.x & o) != 0;
-        float a = up ? h : hi, b = up ? l : lo;
-        const float c = up ? hi : h, d = up ? lo : l;
-        acc2(a, b, c);
-        hi = a;
-        lo = b + d;
-    }
-}
-
 template <int NT, int E>
 __global__ __launch_bounds__(NT) void k_cert_node(const __grid_constant__ CertArgs a) {
     using K = unsigned long long;
@@ -417,7 +404,9 @@ __global__ __launch_bounds__(NT) void k_cert_node(const __grid_constant__ CertAr
     K key[E];                                                  // bits of v (non-negative)
     uint32_t bkey[E];                                          // bits of |beta|
     uint32_t ffree = 0;
+    constexpr bool F64 = NT * E <= 512;
     float s1h = 0.f, s1l = 0.f, s2h = 0.f, s2l = 0.f;          // free sum |beta|, sum beta^2
+    double s1 = 0.0, s2 = 0.0;
     int nnz = 0, infeas = 0;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
@@ -447,18 +436,30 @@ __global__ __launch_bounds__(NT) void k_cert_node(const __grid_constant__ CertAr
         ffree |= 1u << e;
         key[e] = (K)__double_as_longlong(v);
         bkey[e] = __float_as_uint(ab);
-        acc2(s1h, s1l, ab);
-        acc2_sq(s2h, s2l, ab);
+        if constexpr (F64) {
+            const double d = (double)ab;
+            s1 += d;
+            s2 = fma(d, d, s2);
+        } else {
+            acc2(s1h, s1l, ab);
+            acc2_sq(s2h, s2l, ab);
+        }
         nnz += ab > 0.f;
         infeas += ab > mth_f;
     }
-    warp_acc2(s1h, s1l);
-    warp_acc2(s2h, s2l);
+    if constexpr (!F64) {
+        s1 = (double)s1h + (double)s1l;
+        s2 = (double)s2h + (double)s2l;
+    }
+    // both sums in one butterfly, half of the lanes each: five FP64 additions for ten
+    const bool up = lane >= 16;
+    double both = (up ? s2 : s1) + __shfl_xor_sync(0xffffffffu, up ? s1 : s2, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) both += __shfl_xor_sync(0xffffffffu, both, o);
     nnz = __reduce_add_sync(0xffffffffu, nnz);
     infeas = __reduce_add_sync(0xffffffffu, infeas);
+    if ((lane & 15) == 0) sh.red[2 * warp + (lane >> 4)] = both;
     if (lane == 0) {
-        sh.red[2 * warp] = (double)s1h + (double)s1l;
-        sh.red[2 * warp + 1] = (double)s2h + (double)s2l;
         sh.redf[2 * warp] = __int_as_float(nnz);
         sh.redf[2 * warp + 1] = __int_as_float(infeas);
     }
