@@ -13,72 +13,7 @@
 namespace kglm {
 
 constexpr int kMomN = 256;
-static __device__ const double kMomT[kMomN + 1] = {
-    0x1.0000000000000p+0, 0x1.9e3779b97f4a8p+0, 0x1.18c57edb318bcp+1, 0x1.5ff929a25216ep+1,
-    0x1.a5be9e0684cf7p+1, 0x1.ea92aec414c1bp+1, 0x1.175d732001563p+2, 0x1.3931195769aa6p+2,
-    0x1.5ad2842fd3d35p+2, 0x1.7c4ba35748cf2p+2, 0x1.9da3b03e995a3p+2, 0x1.bee0173d977c0p+2,
-    0x1.e0050602df470p+2, 0x1.008ae35d60f2fp+3, 0x1.110a7e54f2d06p+3, 0x1.218266e42a175p+3,
-    0x1.31f3800deeff4p+3, 0x1.425e8775e01abp+3, 0x1.52c41d311f95cp+3, 0x1.6324c9a448d80p+3,
-    0x1.738101fd19f2ap+3, 0x1.83d92ba8e755fp+3, 0x1.942d9f0b5a87bp+3, 0x1.a47ea9a54a95ap+3,
-    0x1.b4cc8fce1b9c1p+3, 0x1.c5178e18d08b0p+3, 0x1.d55fda7776c11p+3, 0x1.e5a5a52aebe4fp+3,
-    0x1.f5e919899f939p+3, 0x1.03152f52bcbb8p+4, 0x1.0b34cbeb9b360p+4, 0x1.1353729a17577p+4,
-    0x1.1b7131f935cf7p+4, 0x1.238e175f13813p+4, 0x1.2baa2f0197d7bp+4, 0x1.33c584161a3b0p+4,
-    0x1.3be020eccad2dp+4, 0x1.43fa0f08889e1p+4, 0x1.4c135733b08f8p+4, 0x1.542c01925910cp+4,
-    0x1.5c4415b259b76p+4, 0x1.645b9a996f1a2p+4, 0x1.6c7296d1bdc4cp+4, 0x1.74891074ecb24p+4,
-    0x1.7c9f0d3606fcfp+4, 0x1.84b4926a4d3e0p+4, 0x1.8cc9a51119199p+4, 0x1.94de49daf0745p+4,
-    0x1.9cf2852fe1a16p+4, 0x1.a5065b353e518p+4, 0x1.ad19cfd2c814cp+4, 0x1.b52ce6b75ebb9p+4,
-    0x1.bd3fa35d3ec0cp+4, 0x1.c552090ddc139p+4, 0x1.cd641ae56408bp+4, 0x1.d575dbd5efe43p+4,
-    0x1.dd874eaa70460p+4, 0x1.e598760958c4ep+4, 0x1.eda9547712280p+4, 0x1.f5b9ec5838f04p+4,
-    0x1.fdca3ff3ad3b5p+4, 0x1.02ed28ba3c3e0p+5, 0x1.06f51175c6813p+5, 0x1.0afcdb28b1710p+5,
-    0x1.0f0486c3bab03p+5, 0x1.130c152cd1e1fp+5, 0x1.1713873fbc063p+5, 0x1.1b1addceaaefbp+5,
-    0x1.1f2219a2c9da2p+5, 0x1.23293b7cc00d3p+5, 0x1.273044152a622p+5, 0x1.2b37341d0c6c9p+5,
-    0x1.2f3e0c3e39f53p+5, 0x1.3344cd1bb964cp+5, 0x1.374b77521fae1p+5, 0x1.3b520b77e63a7p+5,
-    0x1.3f588a1dbb4e0p+5, 0x1.435ef3cecd512p+5, 0x1.4765491111607p+5, 0x1.4b6b8a65857dep+5,
-    0x1.4f71b8486eb54p+5, 0x1.5377d331937f0p+5, 0x1.577ddb9472a68p+5, 0x1.5b83d1e076f32p+5,
-    0x1.5f89b68127ce1p+5, 0x1.638f89de571a7p+5, 0x1.67954c5c4c70bp+5, 0x1.6b9afe5bedea5p+5,
-    0x1.6fa0a03ae6a85p+5, 0x1.73a63253cb3a0p+5, 0x1.77abb4fe3c083p+5, 0x1.7bb1288f05e5fp+5,
-    0x1.7fb68d5840e42p+5, 0x1.83bbe3a96d857p+5, 0x1.87c12bcf906bep+5, 0x1.8bc666154c984p+5,
-    0x1.8fcb92c2fc525p+5, 0x1.93d0b21ec8ce2p+5, 0x1.97d5c46cc0a24p+5, 0x1.9bdac9eeed20cp+5,
-    0x1.9fdfc2e566a41p+5, 0x1.a3e4af8e67decp+5, 0x1.a7e99026603dap+5, 0x1.abee64e805694p+5,
-    0x1.aff32e0c63f3cp+5, 0x1.b3f7ebcaef3ebp+5, 0x1.b7fc9e5990a4ap+5, 0x1.bc0145ecb5f01p+5,
-    0x1.c005e2b75f2a0p+5, 0x1.c40a74eb2bc91p+5, 0x1.c80efcb86749cp+5, 0x1.cc137a4e15382p+5,
-    0x1.d017edd9fcb1bp+5, 0x1.d41c5788b3679p+5, 0x1.d820b785a826cp+5, 0x1.dc250dfb2ced4p+5,
-    0x1.e0295b1280919p+5, 0x1.e42d9ef3d8028p+5, 0x1.e831d9c66723fp+5, 0x1.ec360bb0694e0p+5,
-    0x1.f03a34d729730p+5, 0x1.f43e555f09f06p+5, 0x1.f8426d6b8c0f2p+5, 0x1.fc467d1f57373p+5,
-    0x1.0025424e1fecep+6, 0x1.02274201a70adp+6, 0x1.04293dba620cdp+6, 0x1.062b358812238p+6,
-    0x1.082d297a1b8bep+6, 0x1.0a2f199f8865cp+6, 0x1.0c3106070b6e6p+6, 0x1.0e32eebf02a10p+6,
-    0x1.1034d3d579be4p+6, 0x1.1236b5582cbbap+6, 0x1.143893548a1bep+6, 0x1.163a6dd7b531cp+6,
-    0x1.183c44ee884d6p+6, 0x1.1a3e18a596d61p+6, 0x1.1c3fe9092f506p+6, 0x1.1e41b6255d526p+6,
-    0x1.20438005eb65dp+6, 0x1.224546b664d99p+6, 0x1.24470a4217833p+6, 0x1.2648cab415709p+6,
-    0x1.284a8817368afp+6, 0x1.2a4c42761a2bap+6, 0x1.2c4df9db28a31p+6, 0x1.2e4fae5094b2ep+6,
-    0x1.30515fe05cfb1p+6, 0x1.32530e944d5b4p+6, 0x1.3454ba7600486p+6, 0x1.3656638ee0172p+6,
-    0x1.385809e8283bbp+6, 0x1.3a59ad8ae67f3p+6, 0x1.3c5b4e7ffc2b2p+6, 0x1.3e5cecd01f2b7p+6,
-    0x1.405e8883db273p+6, 0x1.426021a39290bp+6, 0x1.4461b8377facep+6, 0x1.46634c47b592ap+6,
-    0x1.4864dddc21221p+6, 0x1.4a666cfc89f4bp+6, 0x1.4c67f9b093459p+6, 0x1.4e6983ffbcd30p+6,
-    0x1.506b0bf163b93p+6, 0x1.526c918cc3465p+6, 0x1.546e14d8f5c87p+6, 0x1.566f95dcf5555p+6,
-    0x1.5871149f9c8c0p+6, 0x1.5a729127a7517p+6, 0x1.5c740b7bb386ep+6, 0x1.5e7583a241bb8p+6,
-    0x1.6076f9a1b5d8cp+6, 0x1.62786d8057c9cp+6, 0x1.6479df44541e1p+6, 0x1.667b4ef3bca7cp+6,
-    0x1.687cbc948914fp+6, 0x1.6a7e282c97856p+6, 0x1.6c7f91c1ad1b7p+6, 0x1.6e80f95976898p+6,
-    0x1.70825ef9889b4p+6, 0x1.7283c2a760bb3p+6, 0x1.748524686574bp+6, 0x1.76868441e6f26p+6,
-    0x1.7887e2391f792p+6, 0x1.7a893e5333e00p+6, 0x1.7c8a98953404bp+6, 0x1.7e8bf1041b3d1p+6,
-    0x1.808d47a4d0c59p+6, 0x1.828e9c7c282d2p+6, 0x1.848fef8ee1bdbp+6, 0x1.869140e1aae25p+6,
-    0x1.889290791e8b0p+6, 0x1.8a93de59c58d3p+6, 0x1.8c952a8817027p+6, 0x1.8e96750878a49p+6,
-    0x1.9097bddf3f273p+6, 0x1.92990510ae8f6p+6, 0x1.949a4aa0fa88dp+6, 0x1.969b8e9446b92p+6,
-    0x1.989cd0eea710dp+6, 0x1.9a9e11b4201aap+6, 0x1.9c9f50e8a7489p+6, 0x1.9ea08e90233f3p+6,
-    0x1.a0a1caae6c1f3p+6, 0x1.a2a305474bcd2p+6, 0x1.a4a43e5e7e375p+6, 0x1.a6a575f7b19a3p+6,
-    0x1.a8a6ac1686c2ep+6, 0x1.aaa7e0be9150ap+6, 0x1.aca913f357f3fp+6, 0x1.aeaa45b854ad0p+6,
-    0x1.b0ab7610f5083p+6, 0x1.b2aca5009a595p+6, 0x1.b4add28a99f57p+6, 0x1.b6aefeb23d6b8p+6,
-    0x1.b8b0297ac2bb6p+6, 0x1.bab152e75c8c1p+6, 0x1.bcb27afb32603p+6, 0x1.beb3a1b960c9dp+6,
-    0x1.c0b4c724f99cap+6, 0x1.c2b5eb41041f5p+6, 0x1.c4b70e107d3bap+6, 0x1.c6b82f9657ad9p+6,
-    0x1.c8b94fd57c317p+6, 0x1.caba6ed0c9b0dp+6, 0x1.ccbb8c8b156ebp+6, 0x1.cebca9072b328p+6,
-    0x1.d0bdc447cd726p+6, 0x1.d2bede4fb57c3p+6, 0x1.d4bff721939e3p+6, 0x1.d6c10ec00f4e3p+6,
-    0x1.d8c2252dc7507p+6, 0x1.dac33a6d51dd7p+6, 0x1.dcc44e813cc6ep+6, 0x1.dec5616c0d9bep+6,
-    0x1.e0c6733041cc9p+6, 0x1.e2c783d04ecccp+6, 0x1.e4c8934ea2361p+6, 0x1.e6c9a1ada1e90p+6,
-    0x1.e8caaeefac2dfp+6, 0x1.eacbbb1717d4bp+6, 0x1.ecccc62634543p+6, 0x1.eecdd01f49e8dp+6,
-    0x1.f0ced90499b2bp+6, 0x1.f2cfe0d85dd30p+6, 0x1.f4d0e79cc988dp+6, 0x1.f6d1ed54094d6p+6,
-    0x1.f8d2f20042effp+6, 0x1.fad3f5a395b0cp+6, 0x1.fcd4f8401a5bap+6, 0x1.fed5f9d7e3622p+6,
-    0x1.006b7d367e7aap+7, 0x1.016bfd00b68f2p+7, 0x1.026c7c4b99ebbp+7, 0x1.036cfb182591fp+7,
-    0x1.046d79675393fp+7};
+constexpr double kMomEnd = 0x1.046d79675393fp+7;   // t after kMomN steps
 static __device__ const double kMomC[kMomN] = {
     0x0.0p+0, 0x1.2083feffc8abbp-2, 0x1.bc75b6146cc75p-2, 0x1.0fe798589a647p-1,
     0x1.32931b9e07f5cp-1, 0x1.4c3fad9e9d504p-1, 0x1.60131e0c6922ep-1, 0x1.6fdf367993570p-1,
@@ -217,7 +152,7 @@ __device__ __forceinline__ double mom_next(double state, double& c) {
     if (__double2hiint(state) < 0) {
         const int i = __double2loint(state);
         c = kMomC[i];
-        return i + 1 < kMomN ? __hiloint2double((int)0x80000000, i + 1) : kMomT[kMomN];
+        return i + 1 < kMomN ? __hiloint2double((int)0x80000000, i + 1) : kMomEnd;
     }
     const double t = 0.5 * (1.0 + sqrt(1.0 + 4.0 * state * state));
     c = (state - 1.0) / t;
@@ -227,7 +162,7 @@ __device__ __forceinline__ double mom_next(double state, float& c) {
     if (__double2hiint(state) < 0) {
         const int i = __double2loint(state);
         c = kMomCf[i];
-        return i + 1 < kMomN ? __hiloint2double((int)0x80000000, i + 1) : kMomT[kMomN];
+        return i + 1 < kMomN ? __hiloint2double((int)0x80000000, i + 1) : kMomEnd;
     }
     double cd;
     const double t = mom_next(state, cd);
