@@ -1016,6 +1016,7 @@ void run_iters(kglm_ctx* c, int count) {
 void whole_batch(kglm_ctx* c) {
     if (c->mrun == 0) return;
     c->mrun = 0;
+    Scope sc(c, PH_LAYOUT, 1, 0.0);
     gather_operand(c->st, c->m, c->p, nullptr, (const float*)c->V, c->Vop, c->Vop_lo, c->pK, c->tc_kind == 0);
     check_launch();
 }
@@ -1074,6 +1075,7 @@ bool any_active(kglm_ctx* c) {
         for (int b = 0; b < c->m; ++b)
             if (h[b] != 0) map[r++] = b;
         while (r < rows) map[r++] = -1;
+        Scope sc(c, PH_LAYOUT, 1, 0.0);
         CK(cudaMemcpyAsync(c->d_slots, map, sizeof(int) * rows, cudaMemcpyHostToDevice, c->st));
         gather_operand(c->st, rows, c->p, c->d_slots, (const float*)c->V, c->Vop, c->Vop_lo, c->pK, c->tc_kind == 0);
         check_launch();
