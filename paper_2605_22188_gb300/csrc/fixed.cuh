@@ -2,7 +2,8 @@
 // per SM in 16 cycles, its integer pipes two per cycle, so that a 64 x 64-bit
 // high product (some eight instructions) costs a quarter of an FP64 FMA and a
 // conversion or a rounding done with shifts a tenth of one done in FP64.  The
-// functions compile for the host too, where their errors are checked.
+// functions compile for the host too, where tests/test_fixed_host.py checks them against
+// decimal arithmetic; tests/test_gpu_fp64_digits.py takes the device's sigmoid_neg.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -60,9 +61,16 @@ __host__ __device__ __forceinline__ double round_f64(bool neg, uint64_t top, boo
     const uint32_t rem = (uint32_t)top & 0x7ffu;
     m += (rem > 0x400u || (rem == 0x400u && (rest || (m & 1u)))) ? 1u : 0u;
     const int be = x + 11 + 52 + 1023;                  // biased exponent: m in [2^52, 2^53]
-    if (be >= 1 && be <= 2045) return bits_f64(((uint64_t)neg << 63) + ((uint64_t)(be - 1) << 52) + m);
-    const double v = ldexp((double)m, x + 11);          // subnormal or overflowing results
-    return neg ? -v : v;
+    const uint64_t sign = (uint64_t)neg << 63;
+    if (be >= 1 && be <= 2046) return bits_f64(sign + ((uint64_t)(be - 1) << 52) + m);
+    if (be > 2046) return bits_f64(sign | 0x7ff0000000000000ull);
+    // a subnormal result: rounded once, at its own last place
+    const int sh = 12 - be;
+    if (sh > 64) return bits_f64(sign);
+    const uint64_t half = 1ull << (sh - 1), low = sh < 64 ? top & ((1ull << (sh & 63)) - 1) : top;
+    uint64_t d = sh < 64 ? top >> (sh & 63) : 0ull;
+    d += (low > half || (low == half && (rest || (d & 1u)))) ? 1u : 0u;
+    return bits_f64(sign | d);
 }
 
 // The row exponent's marker of a row with a non-finite entry: its products are NaN.
@@ -211,8 +219,9 @@ static __device__ const unsigned long long kExp2Dev[64] = {KGLM_EXP2_TABLE};
 // 2^-64), times the table's 2^(j / 64); the reciprocal from an FP32 seed by one step
 // of third order, y (1 + e + e^2).  Table lookup and series as in Tang, "Table-driven
 // implementation of the exponential function in IEEE floating-point arithmetic", ACM
-// TOMS 1989.  Errors before the final rounding are below 2^-58 relative: 0.52 ulp
-// (expf of FP64, an addition and a division: 1.5 ulp).  With et, *et = e^t too (0.52 ulp).
+// TOMS 1989.  Errors before the final rounding are below 2^-58 relative: below 0.54 ulp in
+// all, 0.502 at worst over the arguments of its test (exp, an addition and a division in
+// FP64: 1.9 over the same).  With et, *et = e^t too (the same bound).
 __host__ __device__ __forceinline__ double sigmoid_neg(double t, const unsigned long long* tab, double* et = nullptr) {
     const uint64_t u = f64_bits(t);
     const bool neg = (int64_t)u < 0;
