@@ -61,7 +61,9 @@ typedef enum { KGLM_LSQ = 0, KGLM_LOGISTIC = 1 } kglm_loss;
  * relative). */
 typedef enum {
     KGLM_FP64 = 0,  /* FP64 products and prox (large products as exact BF16 digit products on the
-                       tensor cores, with an error below that of an FP64 sum) */
+                       tensor cores; their error is below that of an FP64 sum in the norm:
+                       64 bits under the largest entry of a row, so that an entry far below
+                       it keeps fewer of its own) */
     KGLM_FP32 = 1,  /* FP32 products (CUDA cores) and prox */
     KGLM_BF16 = 2,  /* BF16 tensor-core products, FP32 accumulate and prox */
     KGLM_TF32 = 3,  /* TF32 tensor-core products, FP32 accumulate and prox */

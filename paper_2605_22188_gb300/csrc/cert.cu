@@ -355,8 +355,9 @@ __global__ __launch_bounds__(NT) void k_cert_bound(const __grid_constant__ CertA
 // the beta sums of Theorem 4.1 are FP64 up to 512 coordinates and FP32 pairs per thread
 // beyond (a pair's squares keep some 48 bits and FP32's range: few entries per thread, added
 // up in FP64), and only the at most 64 selected values reach FP64 sums, in the order of
-// their ranks.  8192 nodes of p = 2000: 0.54 ms (1.27 with
-// a warp per node over 30 FP32 slices); one node of p = 1000: 31 us (78).
+// their ranks.  8192 nodes of p = 2000: 0.61 ms (1.25 with a warp per node over 30 FP32
+// slices); one node of p = 1000: 32 us between its events (76).  What bounds it: the chain of
+// selections at 33 % of the warps an SM holds, issue slots 29 % busy, 235 MB in 312 us.
 struct CertNodeShared {
     SelectShared sel;
     double red[2 * 32];

@@ -29,10 +29,12 @@
 // against exact sums (tests/test_gpu_fp64_split.py) its root-mean-square error is
 // 4.3e-16 to 8e-16 of the results' size over n = 640 .. 20011, p = 111 .. 2000,
 // this one's 5e-20 to 4e-17.
-// The two bounds part where the entries of a row span many binades; the engine
-// takes this path only for instances whose rows are not spread so (the flag of
-// k_split_digits), with the columns of X scaled to comparable size (powers of two
-// moved from X to the other operand, exactly).
+// The two bounds part where the entries of a row span many binades: the error here is
+// normwise, an entry more than 2^11 below its row's largest keeps fewer bits than its
+// double.  The engine takes this path only for instances whose rows are not spread so
+// (the flag of k_split_digits over X, y and the R of kglm_xtr; the iterates and residuals
+// of an evaluation are not looked at), with the columns of X scaled to comparable size
+// (powers of two moved from X to the other operand, exactly).
 #include <algorithm>
 
 #include "common.cuh"
@@ -132,7 +134,8 @@ __global__ __launch_bounds__(256) void k_split_combine(int cols, const int* __re
 // row keep 304 CTAs in flight where the batch is small (a CTA per node left most SMs
 // idle at 8 nodes).  Integer arithmetic but for the least-squares residual (two FP64
 // operations): with FP64 sums, exp and division 1024 nodes of 2000 samples (logistic)
-// took about 220 us, now 65.
+// took about 220 us, now 57 (38 million warp instructions, issue slots 60 % busy; its 69 MB would
+// take 10).
 constexpr int kLinkNT = 256;
 __global__ __launch_bounds__(kLinkNT) void k_split_link(int n, int npad, int parts, int seg, const int* __restrict__ I,
                                                         size_t stride, int parts_k, const int* __restrict__ ev, const int* __restrict__ ex,
