@@ -318,7 +318,8 @@ typedef struct {
                                  computing a 256-row tile with one cta_group::2 product and each CTA
                                  holding half of the B tile: 1 on, -1 off (kglm_configure: 0 keeps);
                                  the digit products of the certificate and of the FP64 mode take
-                                 pairs wherever they have two row tiles */
+                                 pairs wherever they have two row tiles.  Tiles of 16
+                                 columns have no pairs */
     double nodes_per_s;       /* node evaluations per second at the chosen batch */
     double best_nodes_per_s;  /* the best rate over all batch sizes */
 } kglm_tune;

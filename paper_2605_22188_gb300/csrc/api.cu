@@ -665,7 +665,7 @@ Tiling pick_tiling(kglm_ctx* c, int M, int which) {
     q.M = M; q.Mb = Mb; q.N = N; q.nkb = nkb; q.na = na; q.nb = nb; q.def = def;
     q.max_bn = tc_tile_cols(N);
     q.grad_splits = grad ? c->gsplit_max : 0;
-    q.can_pair = c->tc_kind == 0 && !cert && mt >= 2;
+    q.can_pair = c->tc_kind == 0 && !cert && mt >= 2 && def >= kPairMinCols;
     q.pair = c->pair_auto ? -1 : c->pair ? 1 : 0;
     const Tiling best = choose_tiling(q);
     if (c->tilings.size() >= 256) c->tilings.clear();

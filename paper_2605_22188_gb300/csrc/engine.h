@@ -62,6 +62,9 @@ struct TcMap {
     alignas(64) unsigned char half[128];
     int has_half;
 };
+// Narrower tiles stay with single CTAs: half of a 16-column tile is 8 rows of B, with nothing
+// to gain from sharing them, and a 256-row product of 16 columns is no shape to rely on.
+constexpr int kPairMinCols = 32;
 // TC_EPI_PARTIAL: split z writes its partial product to pout + z*pstride (row
 // stride pld); the consumer sums the slices (no reduction in the kernel).
 enum { TC_EPI_STORE_F32 = 0, TC_EPI_LINK_F32 = 1, TC_EPI_LINK_BF16 = 2, TC_EPI_PARTIAL = 3 };

@@ -1213,7 +1213,7 @@ int tc_gemm(cudaStream_t s, const TcMap& A, const TcMap& B, const TcMap* B2, con
     // CTA pairs: BF16 single operands, at least two row tiles, no split-K link epilogue
     // (its partial tiles and arrival counters are indexed per tile), a B map with a
     // half box
-    const bool pair = g.pair && g.kind == 0 && nb == 1 && na == 1 && a.mt >= 2 &&
+    const bool pair = g.pair && g.bn >= kPairMinCols && g.kind == 0 && nb == 1 && na == 1 && a.mt >= 2 &&
                       (splits == 1 || g.epi == TC_EPI_PARTIAL) && a.njobs == 0 && B.has_half &&
                       pair_clusters() > 0;
     // a pair's ring holds this CTA's half of each B slice, two K slices per stage:
@@ -1347,7 +1347,7 @@ int tc_gemm_jobs(cudaStream_t s, const TcMap& A, const TcMap& B, int M, int N, i
     const CUtensorMap& ma = *reinterpret_cast<const CUtensorMap*>(A.bytes);
     const CUtensorMap& mb = *reinterpret_cast<const CUtensorMap*>(B.bytes);
     // CTA pairs as in tc_gemm: 256-row tiles, half of B per CTA, two K slices per stage
-    const bool pair = pair_on && a.mt >= 2 && B.has_half && pair_clusters() > 0;
+    const bool pair = pair_on && bn >= kPairMinCols && a.mt >= 2 && B.has_half && pair_clusters() > 0;
     cudaLaunchConfig_t cfg{};
     cfg.blockDim = dim3(NT);
     cfg.stream = s;

@@ -194,7 +194,7 @@ constexpr size_t kLinkSmem = 96 * 1024;    // a part of at most 12288 samples
 bool split_plan(int M, int N, int K, int nd, int bn, bool pair, SplitPlan* out) {
     const int kbs = (K + 63) / 64, chunk = kSplitChunk;
     const int mt = (M + 127) / 128, nt = (N + bn - 1) / bn;
-    pair = pair && mt >= 2;
+    pair = pair && mt >= 2 && bn >= kPairMinCols;
     const long tiles = (long)(pair ? (mt + 1) / 2 : mt) * nt;
     const int workers = pair ? 76 : 152;
     const double total = 0.5 * nd * (nd + 1) * kbs * (double)tiles;
