@@ -329,7 +329,9 @@ kglm_status kglm_autotune(kglm_ctx* ctx, int32_t iters, uint64_t seed, kglm_tune
  * batch or sub_batches keeps the current value; `timed` and the rates are
  * ignored).  Until a tile is set here or by kglm_autotune the engine picks the
  * tiles, and until `pair` is set the CTA pairs, from the sizes of each product;
- * no result depends on them.  The
+ * no result depends on them.  Tiles or sub-batches that were set (or tuned) tie the
+ * split of the sums to the rows: nodes that a check finishes then keep their rows in
+ * the products until the evaluation ends, and the certificate keeps its default tile.  The
  * split cap may not exceed the slices allocated at creation.  pdl 0 launches
  * the iteration kernels without programmatic dependent launch. */
 kglm_status kglm_configure(kglm_ctx* ctx, const kglm_tune* cfg);
